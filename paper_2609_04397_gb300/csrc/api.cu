@@ -80,6 +80,24 @@ struct DevBuf {
     size_t bytes = 0;
 };
 
+// One direction (forward, adjoint) of the sliced FP64 products
+struct SlicePlan {
+    bool applies = false;           // the planner's rule: nearly all of the work is in rows narrow enough
+    int64_t digit_bytes = 0;        // of the value tiles
+    int64_t n_chunks = 0;
+    SliceItem *items = nullptr;     // parallel to the cost-ordered work items
+    SliceChunk *chunks = nullptr;   // X rows, cut at the structures
+    int32_t *struct_rows = nullptr; // X rows of every structure
+    int64_t *struct_nnz = nullptr;  // stored entries of every structure
+    int64_t max_nnz = 0;            // of the largest structure
+    uint8_t *vdig = nullptr;        // value tiles, built on first use
+    int32_t *rexp = nullptr;        // scale exponent of every output row
+    bool no_room = false;           // an allocation failed: keep to the multiply-add kernels
+    bool stale = false;             // the values changed since the tiles were built
+    bool captured = false;          // a captured product reads the tiles: every change of the values rebuilds them
+    bool untracked = false;         // a capture changes the values with no tiles to rebuild: multiply-adds only
+};
+
 }  // namespace
 
 struct vbcsr_matrix {
@@ -130,6 +148,14 @@ struct vbcsr_matrix {
     bool panelbp_valid = false;
     uint16_t *xbp = nullptr;      // the current X as two bf16 planes [rows, pipe_ldp(k)] (hi, then lo)
     size_t xbp_elems = 0;
+    // sliced FP64 products: forward, adjoint; digits of the current X; work counter,
+    // column maxima and counts of tiny elements (one allocation, cleared by one memset)
+    SlicePlan slice[2];
+    std::vector<int64_t> struct_row, struct_col;   // first scalar row / column of every structure
+    uint64_t *xdig = nullptr;
+    size_t xdig_elems = 0;
+    uint32_t *stab = nullptr;
+    size_t stab_elems = 0;
     WorkItem *fwd_items = nullptr, *adj_items = nullptr;   // bucketed by row count
     WorkItem *fwd_lpt = nullptr, *adj_lpt = nullptr;       // all items, descending cost
     int64_t n_fwd_items = 0, n_adj_items = 0;
@@ -284,9 +310,54 @@ static void sort_by_cost(std::vector<WorkItem> &items) {
                      [](const WorkItem &x, const WorkItem &y) { return cost_class(x) > cost_class(y); });
 }
 
+// Plan of the sliced products in one direction: the value tile of every item
+// (in the order of `items`), and the rows of X in chunks of one structure each.
+// out_start / in_start: first scalar output / input row of every structure.
+static int plan_slices(vbcsr_matrix *A, SlicePlan *p, const std::vector<WorkItem> &items,
+                       const std::vector<int64_t> &out_start, const std::vector<int64_t> &in_start, cudaStream_t s) {
+    if (A->dtype != VBCSR_F64 || A->backend == VBCSR_BACKEND_CSR || items.empty() || A->nblk == 0) return VBCSR_OK;
+    std::vector<SliceItem> si(items.size());
+    std::vector<int64_t> nnz(out_start.size() - 1, 0);
+    int64_t pos = 0;
+    double wide = 0.0, all = 0.0;
+    for (size_t t = 0; t < items.size(); ++t) {
+        const WorkItem &w = items[t];
+        si[t].doff = -1;
+        si[t].pad = 0;
+        si[t].strct = (int32_t)(std::upper_bound(out_start.begin(), out_start.end() - 1, w.yrow) - out_start.begin() - 1);
+        all += (double)w.B * w.K;
+        nnz[si[t].strct] += (int64_t)w.B * w.K;
+        if (w.K > kSliceKMax) {
+            wide += (double)w.B * w.K;
+            continue;
+        }
+        si[t].doff = pos;
+        pos += (int64_t)((w.K + 15) / 16) * w.B * (kSliceDigits * 16);
+    }
+    // the wide items run multiply-adds in a kernel with fewer resident warps than the
+    // multiply-add kernels have: not for an operator with much of its work there
+    if (wide > 0.1 * all) return VBCSR_OK;
+    p->digit_bytes = pos;
+    std::vector<SliceChunk> ch;
+    std::vector<int32_t> rows(in_start.size() - 1);
+    for (size_t t = 0; t + 1 < in_start.size(); ++t) {
+        rows[t] = (int32_t)(in_start[t + 1] - in_start[t]);
+        for (int64_t r = in_start[t]; r < in_start[t + 1]; r += kSliceChunkRows)
+            ch.push_back({(int32_t)r, (int32_t)std::min<int64_t>(kSliceChunkRows, in_start[t + 1] - r), (int32_t)t});
+    }
+    p->n_chunks = (int64_t)ch.size();
+    CUDA_TRY(upload(A, &p->items, si, s), "upload sliced items");
+    CUDA_TRY(upload(A, &p->chunks, ch, s), "upload");
+    CUDA_TRY(upload(A, &p->struct_rows, rows, s), "upload");
+    CUDA_TRY(upload(A, &p->struct_nnz, nnz, s), "upload");
+    p->max_nnz = *std::max_element(nnz.begin(), nnz.end());
+    p->applies = true;
+    return VBCSR_OK;
+}
+
 static int build(vbcsr_matrix *A, int64_t n_brows, int64_t n_bcols, const int32_t *row_bsize,
                  const int32_t *col_bsize, const int64_t *block_row_ptr, const int32_t *block_col_idx,
-                 const void *values, int values_on_device, cudaStream_t s) {
+                 const void *values, int values_on_device, const int64_t *sbo, const int64_t *sco, cudaStream_t s) {
     A->n_brows = n_brows;
     A->n_bcols = n_bcols;
     A->row_b.assign(row_bsize, row_bsize + n_brows);
@@ -299,6 +370,10 @@ static int build(vbcsr_matrix *A, int64_t n_brows, int64_t n_bcols, const int32_
     A->n_cols = A->col_off[n_bcols];
     const int64_t nblk = block_row_ptr[n_brows];
     A->nblk = nblk;
+    for (int32_t t = 0; t <= A->n_structs; ++t) {
+        A->struct_row.push_back(sbo ? A->row_off[sbo[t]] : (t ? A->n_rows : 0));
+        A->struct_col.push_back(sco ? A->col_off[sco[t]] : (t ? A->n_cols : 0));
+    }
 
     // packed-order offsets
     A->uoff.assign(nblk + 1, 0);
@@ -464,6 +539,8 @@ static int build(vbcsr_matrix *A, int64_t n_brows, int64_t n_bcols, const int32_
         A->n_fwd_items = (int64_t)items.size();
         sort_by_cost(items);
         CUDA_TRY(upload(A, &A->fwd_lpt, items, s), "upload forward items");
+        const int rc = plan_slices(A, &A->slice[0], items, A->struct_row, A->struct_col, s);
+        if (rc) return rc;
     }
 
     // transposed list and adjoint work items
@@ -529,6 +606,8 @@ static int build(vbcsr_matrix *A, int64_t n_brows, int64_t n_bcols, const int32_
         A->n_adj_items = (int64_t)items.size();
         sort_by_cost(items);
         CUDA_TRY(upload(A, &A->adj_lpt, items, s), "upload adjoint items");
+        const int rc = plan_slices(A, &A->slice[1], items, A->struct_col, A->struct_row, s);
+        if (rc) return rc;
         CUDA_TRY(upload(A, &A->tl_pbase, tl_pbase, s), "upload");
         CUDA_TRY(upload(A, &A->tl_kp, tl_kp, s), "upload");
         CUDA_TRY(upload(A, &A->tl_bi, tl_bi, s), "upload");
@@ -590,7 +669,7 @@ static int build(vbcsr_matrix *A, int64_t n_brows, int64_t n_bcols, const int32_
 static int create_common(vbcsr_t **out, int64_t n_brows, int64_t n_bcols, const int32_t *row_bsize,
                          const int32_t *col_bsize, const int64_t *block_row_ptr, const int32_t *block_col_idx,
                          const void *values, int dtype, int values_on_device, void *stream, int32_t n_structs,
-                         bool zero_values = false) {
+                         const int64_t *sbo = nullptr, const int64_t *sco = nullptr, bool zero_values = false) {
     if (!out) return fail(VBCSR_ERR_INVALID_ARG, "out is NULL");
     *out = nullptr;
     if (dtype != VBCSR_F64 && dtype != VBCSR_F32 && dtype != VBCSR_C128)
@@ -611,7 +690,7 @@ static int create_common(vbcsr_t **out, int64_t n_brows, int64_t n_bcols, const 
     A->debug_checks = (dbg && dbg[0] && dbg[0] != '0') ? 1 : 0;
     try {
         rc = build(A, n_brows, n_bcols, row_bsize, col_bsize, block_row_ptr, block_col_idx, values,
-                   values_on_device, (cudaStream_t)stream);
+                   values_on_device, sbo, sco, (cudaStream_t)stream);
     } catch (const std::bad_alloc &) {
         rc = fail(VBCSR_ERR_NO_MEMORY, "host allocation in planner");
     }
@@ -664,7 +743,7 @@ extern "C" int vbcsr_create_batched(vbcsr_t **out, int64_t n_structs, const int6
             }
     }
     return create_common(out, n_brows, n_bcols, row_bsize, col_bsize, block_row_ptr, gcol.data(), values, dtype,
-                         values_on_device, stream, (int32_t)n_structs);
+                         values_on_device, stream, (int32_t)n_structs, sbo, sco);
 }
 
 // ---------------------------------------------------------------------------
@@ -718,7 +797,7 @@ extern "C" int vbcsr_create_kspace(vbcsr_t **out, int64_t n_atoms, const int32_t
         for (int64_t a = 0; a < n_atoms; ++a) rowptr[a + 1] += rowptr[a];
         const int64_t nblk = (int64_t)cols.size();
         int rc = create_common(out, n_atoms, n_atoms, bsize, bsize, rowptr.data(), cols.data(), nullptr, VBCSR_C128,
-                               0, stream, 1, true);
+                               0, stream, 1, nullptr, nullptr, true);
         if (rc) return rc;
         vbcsr_matrix *A = *out;
         auto bail = [&](int code) {
@@ -824,6 +903,67 @@ static int grow(vbcsr_t *A, T **buf, size_t *have, size_t need, cudaStream_t s, 
     return VBCSR_OK;
 }
 
+// The digit tiles of one direction, from the values now in the pages
+static int refresh_slices(vbcsr_t *A, bool trans, cudaStream_t s) {
+    SlicePlan &p = A->slice[trans];
+    const AdjList tl = {A->tl_pbase, A->tl_kp, A->tl_bi, A->tl_xrow, A->tl_vcol};
+    CUDA_TRY(launch_slice_values(trans, trans ? A->adj_lpt : A->fwd_lpt, p.items,
+                                 trans ? A->n_adj_items : A->n_fwd_items, tl, (const double *)A->panel, p.vdig, p.rexp,
+                                 s),
+             "slice values");
+    return VBCSR_OK;
+}
+
+static bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+}
+
+// The pages have (or, under capture, will have) new values. The tiles are
+// rebuilt by the next product that reads them: a training step that sets the
+// values twice and uses one direction each time builds each once. Tiles that a
+// captured product reads, and changes that are themselves captured, are rebuilt
+// here, since the host does not see the replays.
+static int slices_changed(vbcsr_t *A, cudaStream_t s) {
+    for (int t = 0; t < 2; ++t) {
+        SlicePlan &p = A->slice[t];
+        if (!p.applies) continue;
+        const bool cap = capturing(s);
+        if (!p.vdig) {
+            p.untracked |= cap;
+        } else if (cap || p.captured) {
+            int rc = refresh_slices(A, t == 1, s);
+            if (rc) return rc;
+            if (!cap) p.stale = false;
+        } else {
+            p.stale = true;
+        }
+    }
+    return VBCSR_OK;
+}
+
+// True when a native FP64 product of k columns runs sliced. From two columns:
+// at one column the multiply-add kernel needs 2 FP64 operations per 8 stored
+// bytes and the value tiles are 12 bytes per entry, so there is nothing to gain.
+static bool slice_applies(const vbcsr_t *A, bool trans, int64_t k) {
+    const SlicePlan &p = A->slice[trans];
+    return p.applies && !p.untracked && k >= 2 && k <= (1 << 20) && p.max_nnz * k >= kSliceMinWork && !A->debug_checks;
+}
+
+static size_t slice_tab_elems(const vbcsr_t *A, int64_t ldp) { return 4 + 2 * (size_t)A->n_structs * (size_t)ldp; }
+
+static bool slice_buffers_ready(const vbcsr_t *A, bool trans, int64_t k) {
+    const int64_t ldp = (k + 7) / 8 * 8, xrows = trans ? A->n_rows : A->n_cols;
+    return A->slice[trans].vdig && A->xdig_elems >= (size_t)(xrows * ldp) &&
+           A->stab_elems >= slice_tab_elems(A, ldp);
+}
+
+// Builds what a sliced product needs and is missing (*ready = true when it can
+// run). Nothing is allocated while the stream is being captured or when the
+// caller must not allocate; when the device has no room, the product runs
+// multiply-adds from then on.
+static int slice_prepare(vbcsr_t *A, bool trans, int64_t k, bool may_alloc, cudaStream_t s, bool *ready);
+
 extern "C" int vbcsr_set_values(vbcsr_t *A, const void *values, int on_device, void *stream) {
     if (!A) return fail(VBCSR_ERR_INVALID_ARG, "handle is NULL");
     if (on_device != 0 && on_device != 1) return fail(VBCSR_ERR_INVALID_ARG, "on_device must be 0 or 1");
@@ -846,6 +986,10 @@ extern "C" int vbcsr_set_values(vbcsr_t *A, const void *values, int on_device, v
         if (e2 != cudaSuccess) return cuda_fail(e2, "set_values");
     }
     if (e != cudaSuccess) return cuda_fail(e, "set_values");
+    {
+        int rc = slices_changed(A, s);
+        if (rc) return rc;
+    }
     if (A->panel32) {
         int rc = refresh_panel32(A, s);
         if (rc) return rc;
@@ -1033,9 +1177,48 @@ static bool fused_x_applies(const vbcsr_t *A, const ModePlan &p) {
 
 // dot_scale multiplies the fused dot product before it is stored (1 for the
 // public epilogue, 1 / (N k) for the Chebyshev moments).
+static int slice_prepare(vbcsr_t *A, bool trans, int64_t k, bool may_alloc, cudaStream_t s, bool *ready) {
+    *ready = slice_buffers_ready(A, trans, k);
+    SlicePlan &p = A->slice[trans];
+    const bool cap = capturing(s);
+    if (*ready) {
+        p.captured |= cap;
+        if (p.stale) {
+            // under capture the rebuild belongs to the graph: the tiles stay stale for eager calls
+            int rc = refresh_slices(A, trans, s);
+            if (rc) return rc;
+            if (!cap) p.stale = false;
+        }
+        return VBCSR_OK;
+    }
+    if (!may_alloc || p.no_room || cap) return VBCSR_OK;
+    const int64_t ldp = (k + 7) / 8 * 8, xrows = trans ? A->n_rows : A->n_cols;
+    int rc = VBCSR_OK;
+    if (!p.vdig) {
+        cudaError_t e = p.rexp ? cudaSuccess : A->alloc(&p.rexp, (size_t)(trans ? A->n_cols : A->n_rows));
+        if (e == cudaSuccess) e = A->alloc(&p.vdig, (size_t)p.digit_bytes);
+        if (e != cudaSuccess) rc = cuda_fail(e, "alloc value digits");
+        p.stale = p.vdig != nullptr;
+    }
+    if (!rc && p.stale) {
+        rc = refresh_slices(A, trans, s);
+        p.stale = rc != VBCSR_OK;
+    }
+    if (!rc)
+        rc = grow(A, &A->xdig, &A->xdig_elems, (size_t)(xrows * ldp), s, "alloc fixed-point X");
+    if (!rc) rc = grow(A, &A->stab, &A->stab_elems, slice_tab_elems(A, ldp), s, "alloc column maxima");
+    if (rc == VBCSR_ERR_NO_MEMORY) {
+        p.no_room = true;
+        return VBCSR_OK;
+    }
+    if (rc) return rc;
+    *ready = true;
+    return VBCSR_OK;
+}
+
 static int run_product(vbcsr_t *A, bool trans, int64_t k, double alpha, const void *X, int64_t ldx, double beta,
                        void *Y, int64_t ldy, const vbcsr_epilogue_t *epi, int precision, cudaStream_t s,
-                       double dot_scale = 1.0, const FusedX *fx = nullptr) {
+                       double dot_scale = 1.0, const FusedX *fx = nullptr, bool may_alloc = true) {
     if (!A) return fail(VBCSR_ERR_INVALID_ARG, "handle is NULL");
     if (k < 0) return fail(VBCSR_ERR_INVALID_ARG, "k = %lld", (long long)k);
     if (precision < VBCSR_PREC_NATIVE || precision > VBCSR_PREC_DF32)
@@ -1080,6 +1263,11 @@ static int run_product(vbcsr_t *A, bool trans, int64_t k, double alpha, const vo
     }
     if (mp.need_panelbp && !A->panelbp_valid) {
         int rc = refresh_panelbp(A, s);
+        if (rc) return rc;
+    }
+    bool sliced = f64 && mode == VBCSR_PREC_NATIVE && alpha != 0.0 && slice_applies(A, trans, k);
+    if (sliced) {
+        int rc = slice_prepare(A, trans, k, may_alloc, s, &sliced);
         if (rc) return rc;
     }
     const bool piped = mp.pipe || mp.pipe_tf;
@@ -1188,6 +1376,8 @@ static int run_product(vbcsr_t *A, bool trans, int64_t k, double alpha, const vo
     // operator has more than two row counts (the wide form's larger code then
     // runs slower, see process_item)
     const bool df_narrow = A->fwd_buckets.size() > 2;
+    SliceArgs sa;
+    memset(&sa, 0, sizeof(sa));
     int64_t used = 0;
     bool per_item_dot = false;   // the persistent CUDA-core launch writes one dot share per item
     // one launch of `kern` over items[0..n) with `warps` warps per CTA
@@ -1211,7 +1401,9 @@ static int run_product(vbcsr_t *A, bool trans, int64_t k, double alpha, const vo
             used += a.grid;
         }
         cudaError_t e;
-        if (fpipe)
+        if (sliced)
+            e = launch_slice_product(trans, a, sa, s);
+        else if (fpipe)
             e = launch_fma32_pipe(f64, a, s);
         else if (mode == VBCSR_PREC_NATIVE)
             e = cplx ? launch_fma_c128(B, trans, a, s)
@@ -1239,7 +1431,28 @@ static int run_product(vbcsr_t *A, bool trans, int64_t k, double alpha, const vo
     };
     const int64_t n_all = trans ? A->n_adj_items : A->n_fwd_items;
     int rc = VBCSR_OK;
-    if (!fma && !split) {
+    if (sliced) {
+        // FP64 on the tensor cores (sliced.cuh): the digits of X, then one launch over every
+        // item; the CUDA-core schedule and tiles do not apply
+        const SlicePlan &p = A->slice[trans];
+        const int ldp8 = (int)((k + 7) / 8 * 8);
+        uint32_t *cmax = A->stab + 4, *ccnt = cmax + (size_t)A->n_structs * ldp8;
+        CUDA_TRY(cudaMemsetAsync(A->stab, 0, slice_tab_elems(A, ldp8) * sizeof(uint32_t), s), "reset column maxima");
+        CUDA_TRY(launch_slice_panel(p.chunks, p.n_chunks, (const double *)X, ldx, (int)k, ldp8, cmax, ccnt, A->xdig, s),
+                 "slice X");
+        sa.sitems = p.items;
+        sa.vdig = p.vdig;
+        sa.rexp = p.rexp;
+        sa.xdig = A->xdig;
+        sa.cmax = cmax;
+        sa.ccnt = ccnt;
+        sa.struct_rows = p.struct_rows;
+        sa.struct_nnz = p.struct_nnz;
+        sa.ldp = ldp8;
+        a.queue = reinterpret_cast<long long *>(A->stab);
+        per_item_dot = true;
+        rc = launch(0, trans ? A->adj_lpt : A->fwd_lpt, n_all, 4, slice_kernel_ptr(trans, k), slice_smem_bytes());
+    } else if (!fma && !split) {
         // tensor-core kernel: the row count is a runtime mask, one launch serves every item
         const bool staged = !trans && (A->schedule & VBCSR_SCHED_MMA_STAGED);
         a.mma_staged = staged ? 1 : 0;
@@ -1406,9 +1619,8 @@ static int cheb_fused_buffers(vbcsr_t *A, int64_t k, int precision, void *xs[2],
 }
 
 
-extern "C" int vbcsr_chebyshev(vbcsr_t *A, int64_t k, const double *R, int64_t ldr, int64_t n_moments,
-                               double *moments, double *work, double *ckpt, int64_t ckpt_every, int precision,
-                               void *stream) {
+static int run_chebyshev(vbcsr_t *A, int64_t k, const double *R, int64_t ldr, int64_t n_moments, double *moments,
+                         double *work, double *ckpt, int64_t ckpt_every, int precision, void *stream, bool may_alloc) {
     if (!A) return fail(VBCSR_ERR_INVALID_ARG, "handle is NULL");
     if (A->dtype != VBCSR_F64 && A->dtype != VBCSR_C128)
         return fail(VBCSR_ERR_UNSUPPORTED, "the recurrence needs an FP64 or complex operator");
@@ -1445,7 +1657,8 @@ extern "C" int vbcsr_chebyshev(vbcsr_t *A, int64_t k, const double *R, int64_t l
     epi.dot_out = moments + 1;
     // with the fused form, t_n is also kept converted in xs[n & 1]
     const FusedX fx0 = {nullptr, xs[1]};
-    int rc = run_product(A, false, k, 1.0, R, ldr, 0.0, buf[1], k, &epi, precision, s, scale, xs[1] ? &fx0 : nullptr);
+    int rc = run_product(A, false, k, 1.0, R, ldr, 0.0, buf[1], k, &epi, precision, s, scale, xs[1] ? &fx0 : nullptr,
+                         may_alloc);
     if (rc) return rc;
     auto store_pair = [&](int64_t m, const double *tm, int64_t ldm, const double *tm1) -> int {
         if (!ckpt || m % ckpt_every) return VBCSR_OK;
@@ -1462,11 +1675,18 @@ extern "C" int vbcsr_chebyshev(vbcsr_t *A, int64_t k, const double *R, int64_t l
         double *tn = buf[n & 1], *tprev = buf[(n + 1) & 1];
         epi.dot_out = moments + n + 1;
         const FusedX fx = {xs[n & 1], xs[(n + 1) & 1]};
-        rc = run_product(A, false, k, 2.0, tn, k, -1.0, tprev, k, &epi, precision, s, scale, xs[0] ? &fx : nullptr);
+        rc = run_product(A, false, k, 2.0, tn, k, -1.0, tprev, k, &epi, precision, s, scale, xs[0] ? &fx : nullptr,
+                         may_alloc);
         if (rc) return rc;
         if ((rc = store_pair(n, tn, k, tprev))) return rc;
     }
     return VBCSR_OK;
+}
+
+extern "C" int vbcsr_chebyshev(vbcsr_t *A, int64_t k, const double *R, int64_t ldr, int64_t n_moments,
+                               double *moments, double *work, double *ckpt, int64_t ckpt_every, int precision,
+                               void *stream) {
+    return run_chebyshev(A, k, R, ldr, n_moments, moments, work, ckpt, ckpt_every, precision, stream, true);
 }
 
 extern "C" int vbcsr_chebyshev_backward(vbcsr_t *A, int64_t k, const double *R, int64_t ldr, int64_t M,
@@ -1641,6 +1861,10 @@ extern "C" int vbcsr_shift_scale(vbcsr_t *A, double c, double d, void *stream) {
                                 A->fl_pcol, A->fl_w, c,
                                 d, s),
              "shift_scale");
+    {
+        int rc = slices_changed(A, s);
+        if (rc) return rc;
+    }
     if (A->panel32) {
         int rc = refresh_panel32(A, s);
         if (rc) return rc;
@@ -2157,5 +2381,5 @@ extern "C" int vbcsr_chebyshev_noalloc(vbcsr_t *A, int64_t k, const double *R, i
     }
     // every element of the work panels that the recurrence reads is written
     // earlier in the same call, so nothing has to be cleared first
-    return vbcsr_chebyshev(A, k, R, ldr, n_moments, moments, work, nullptr, 0, precision, stream);
+    return run_chebyshev(A, k, R, ldr, n_moments, moments, work, nullptr, 0, precision, stream, false);
 }

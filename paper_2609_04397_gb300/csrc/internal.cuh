@@ -148,6 +148,37 @@ cudaError_t launch_fma32_pipe(bool ydouble, const ProdArgs &a, cudaStream_t s);
 const void *fma32_pipe_kernel_ptr(int64_t k, bool ydouble);
 size_t fma32_pipe_smem_bytes(int64_t k, int warps);
 
+// Sliced FP64 products on the FP16 tensor cores (sliced.cuh, spmm_sliced.cu).
+constexpr int kSliceDigits = 7;      // base-256 digits of an element
+constexpr int kSliceKMax = 768;      // widest row (virtual columns) whose level sums stay exact
+constexpr int kSliceChunkRows = 256; // X rows per CTA of the digit passes
+struct SliceItem {
+    int64_t doff;     // byte of the item's first value tile, or -1: wider than kSliceKMax, not sliced
+    int32_t strct;    // structure (of a batched operator) whose X columns the item reads
+    int32_t pad;
+};
+constexpr int64_t kSliceMinWork = 1 << 22;   // stored entries x columns of a structure below which it is not sliced
+struct SliceChunk {   // X rows of one structure
+    int32_t row0, nrows, strct;
+};
+struct SliceArgs {
+    const SliceItem *sitems;      // parallel to ProdArgs::items
+    const uint8_t *vdig;          // value tiles
+    const int32_t *rexp;          // scale exponent of every output row (0: zero row, -1: not sliced)
+    const uint64_t *xdig;         // fixed-point X, ldp columns
+    const uint32_t *cmax, *ccnt;  // [structures, ldp]: high word of the column maxima, tiny elements
+    const int32_t *struct_rows;   // X rows of every structure
+    const int64_t *struct_nnz;    // stored entries of every structure
+    int ldp;                      // k rounded up to 8
+};
+cudaError_t launch_slice_product(bool trans, const ProdArgs &a, const SliceArgs &q, cudaStream_t s);
+cudaError_t launch_slice_panel(const SliceChunk *chunks, int64_t n_chunks, const double *X, int64_t ldx, int k, int ldp,
+                               uint32_t *cmax, uint32_t *ccnt, uint64_t *out, cudaStream_t s);
+cudaError_t launch_slice_values(bool trans, const WorkItem *items, const SliceItem *sitems, int64_t n_items,
+                                const AdjList &tl, const double *panel, uint8_t *dig, int32_t *rexp, cudaStream_t s);
+const void *slice_kernel_ptr(bool trans, int64_t k);
+size_t slice_smem_bytes();
+
 // Scalar (all 1 x 1 blocks) operators: L lanes per row (2, 4 or 8 for the
 // FP64 and double-FP32 kinds, 4, 8, 16 or 32 for the FP32 ones; csr_lane_class
 // 0 and 1).

@@ -1,0 +1,208 @@
+"""The sliced form of native FP64 products (csrc/sliced.cuh): FP64 operands as
+base-256 digits on the FP16 tensor cores, with FP64 multiply-adds wherever the
+fixed point does not resolve an output.
+
+Every element is held to 1e-13 of sum |h x|: the oracle's own chain of up to
+768 multiply-adds stays within 768 2^-53 = 8.5e-14 of it, and an output that
+passes the sliced kernel's check within about 1e-14."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import synthetic as syn
+from synthetic.structures import BlockPattern
+
+pytestmark = pytest.mark.gpu
+TOL = 1e-13
+
+
+def _handle(pat, vals):
+    from paper_2609_04397_gb300 import VBCSR
+    return VBCSR.from_pattern(pat, vals, torch.float64, "cuda:0")
+
+
+def _kernels(fn):
+    from torch.profiler import ProfilerActivity, profile
+    for _ in range(2):   # the first trace of a process can come back before its buffers fill
+        with profile(activities=[ProfilerActivity.CUDA]) as prof:
+            fn()
+            torch.cuda.synchronize()
+        names = [e.name for e in prof.events() if "vbcsr" in e.name]
+        if names:
+            return names
+    return []
+
+
+def _check(H, pat, vals, X, transpose=False, alpha=1.0, beta=0.0, Y0=None, tol=TOL):
+    fn, ref_fn = (H.spmm_adjoint, oracle.spmm_adjoint) if transpose else (H.spmm, oracle.spmm)
+    Xd = torch.from_numpy(X).cuda()
+    if Y0 is None:
+        got = fn(Xd, alpha).cpu().numpy()
+        Y0 = np.zeros_like(got)
+    else:
+        got = fn(Xd, alpha, beta, torch.from_numpy(Y0.copy()).cuda()).cpu().numpy()
+    ref = ref_fn(pat, vals, X, alpha, beta, Y0)
+    scale = ref_fn(pat, np.abs(vals), np.abs(X), abs(alpha), 0.0) + abs(beta) * np.abs(Y0)
+    assert np.array_equal(np.isnan(got), np.isnan(ref))
+    fin = np.isfinite(ref)
+    assert np.array_equal(got[~fin & ~np.isnan(ref)], ref[~fin & ~np.isnan(ref)])
+    bad = np.abs(got[fin] - ref[fin]) > tol * scale[fin]
+    assert not bad.any(), (bad.sum(), np.max(np.abs(got[fin] - ref[fin]) / np.maximum(scale[fin], 1e-300)))
+    return got
+
+
+def _pattern(sizes, n=64, density=0.5, seed=1):
+    return syn.random_pattern(n, n - 3, sizes, density, seed, empty_rows=2, unsorted=True)
+
+
+# row heights 1 .. 16 and taller (chunked), rows of a multiple of 16 columns, ragged ones, some
+# wider than the 768 columns a sliced row may have, widths around the 8- and 16-column tiles
+@pytest.mark.parametrize("sizes,n,density", [((4, 9, 13), 64, 0.5), ((16,), 48, 0.6), ((1, 2, 3), 300, 0.6),
+                                             ((17, 20, 33), 40, 0.4), ((13, 15), 80, 0.6)])
+@pytest.mark.parametrize("k", [2, 8, 9, 16, 17, 40])
+def test_sliced_products_against_oracle(sizes, n, density, k):
+    pat = _pattern(sizes, n, density, seed=k)
+    vals = syn.random_values(pat, k)
+    H = _handle(pat, vals)
+    rng = np.random.default_rng(k)
+    wide = max(k, -(-(1 << 22) // pat.nnz) + 1)        # columns from which this operator is sliced
+    for cols in sorted({k, wide}):
+        X = rng.standard_normal((pat.n_cols, cols))
+        Y0 = rng.standard_normal((pat.n_rows, cols))
+        _check(H, pat, vals, X, alpha=2.0, beta=-1.0, Y0=Y0)
+        Xa = rng.standard_normal((pat.n_rows, cols))
+        _check(H, pat, vals, Xa, transpose=True)
+    assert any("slice_product" in n for n in _kernels(lambda: H.spmm(torch.from_numpy(X).cuda())))
+    H.check()
+
+
+def test_exact_level_sums_at_the_widest_row():
+    """768 equal products whose digits are all 127 or all -128 but the leading one:
+    the largest level sums there are. The exact sum is 768 h x."""
+    b = 16
+    pat = BlockPattern(np.full(120, b), np.full(48, b), np.arange(121) * 48, np.tile(np.arange(48), 120))
+    assert pat.n_cols == 768
+    for digits in (0x7D7F7F7F7F7F7F, 0x7D808080808080 - 0x01010101010100, 0x3E7F7F7F7F7F7F):
+        h = float(digits) * 2.0 ** -54
+        H = _handle(pat, np.full(pat.nnz, h))
+        for x in (h, -h, 0.75 * h):
+            X = torch.full((768, 16), x, dtype=torch.float64, device="cuda:0")
+            from fractions import Fraction
+            exact = float(768 * Fraction(h) * Fraction(x))
+            got = H.spmm(X)
+            assert (got - exact).abs().max().item() <= 4e-16 * abs(exact)
+
+
+def test_unresolved_outputs_take_multiply_adds():
+    """Graded rows and columns, zero rows and columns, panels supported on a few
+    rows, tiny and huge magnitudes, Inf and NaN: every output as accurate as the
+    multiply-add chain's, and NaN and Inf only where they belong."""
+    pat = _pattern((4, 9, 13), 90, 0.3, 5)
+    rng = np.random.default_rng(0)
+    vals = syn.random_values(pat, 5)
+    k = 24
+    X = rng.standard_normal((pat.n_cols, k))
+    cases = {}
+    cases["graded columns"] = X * np.exp(-np.arange(pat.n_cols) / 5.0)[:, None]
+    cases["one-hot"] = np.eye(pat.n_cols)[:, :k]
+    local = np.zeros_like(X)
+    local[100:180] = X[100:180]
+    cases["local"] = local
+    z = X.copy()
+    z[:, 3] = 0.0
+    z[:, 5] *= 1e-200
+    z[:, 7] *= 1e200
+    z[:, 9] = 5e-324
+    cases["scales"] = z
+    bad = X.copy()
+    bad[17, 2], bad[200, 4], bad[3, 6] = np.nan, np.inf, -np.inf
+    cases["not finite"] = bad
+    spike = X.copy()
+    spike[50] *= 1e9
+    cases["spike"] = spike
+    graded = vals * 10.0 ** rng.uniform(-12, 3, len(vals))
+    rows = np.repeat(np.arange(pat.nblk), pat.block_sizes())
+    zero = np.where(np.isin(pat.block_rows()[rows], (4, 5, 6)), 0.0, vals)
+    for v in (vals, graded, zero):
+        H = _handle(pat, v)
+        for X in cases.values():
+            with np.errstate(invalid="ignore", over="ignore"):
+                _check(H, pat, v, np.ascontiguousarray(X))
+    Xt = np.random.default_rng(1).standard_normal((pat.n_rows, k)) * np.exp(-np.arange(pat.n_rows) / 7.0)[:, None]
+    _check(H, pat, zero, Xt, transpose=True)
+
+
+def test_structures_of_a_batch_keep_their_own_scales():
+    """A batched operator's structures are independent: one structure's huge panel leaves
+    the bits of the others alone."""
+    from paper_2609_04397_gb300 import VBCSR
+    w = syn.batched_uneven(6, 600, 900, seed=3)
+    offs = w.struct_brow_offsets
+    rows = w.pattern.block_rows()
+    local = w.pattern.block_col_idx - offs[np.searchsorted(offs, rows, side="right") - 1]
+    H = VBCSR.from_batched(offs, offs, w.pattern.row_bsize, w.pattern.col_bsize, w.pattern.block_row_ptr, local,
+                           w.values, torch.float64, "cuda:0")
+    X = np.random.default_rng(2).standard_normal((w.pattern.n_cols, 16))
+    Y = _check(H, w.pattern, w.values, X)
+    cut = int(w.pattern.row_bsize[:offs[1]].sum())
+    X2 = X.copy()
+    X2[:cut] *= 1e7
+    Y2 = _check(H, w.pattern, w.values, X2)
+    assert np.array_equal(Y[cut:], Y2[cut:])
+
+
+def test_tiles_follow_the_values():
+    """Eager and captured changes of the values reach eager and captured products."""
+    w = syn.amorphous(700, side=60.0 * (700 / 20000) ** (1 / 3))
+    pat, k = w.pattern, 16
+    rng = np.random.default_rng(1)
+    X = rng.standard_normal((pat.n_cols, k))
+    Xd = torch.from_numpy(X).cuda()
+    v = [syn.random_values(pat, s) for s in range(5)]
+    H = _handle(pat, v[0])
+    Y = torch.empty(pat.n_rows, k, dtype=torch.float64, device="cuda:0")
+    buf = torch.from_numpy(v[0]).cuda()
+
+    def same(i, y=None):
+        y = H.spmm(Xd) if y is None else y
+        ref = oracle.spmm(pat, v[i], X)
+        scale = oracle.spmm(pat, np.abs(v[i]), np.abs(X))
+        assert (np.abs(y.cpu().numpy() - ref) <= TOL * scale).all()
+
+    # a product captured before its tiles exist runs multiply-adds
+    first = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(first):
+        H.spmm(Xd, 1.0, 0.0, Y)
+    first.replay()
+    same(0, Y)
+    same(0)
+    H.set_values(torch.from_numpy(v[1]).cuda())
+    same(1)
+    first.replay()
+    same(1, Y)
+    H.set_values(torch.from_numpy(v[2]).cuda())          # stale tiles at capture
+    prod = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(prod):
+        H.spmm(Xd, 1.0, 0.0, Y)
+    same(2)
+    prod.replay()
+    same(2, Y)
+    H.set_values(torch.from_numpy(v[3]).cuda())
+    prod.replay()
+    same(3, Y)
+    setv = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(setv):
+        H.set_values(buf)
+    same(3)
+    buf.copy_(torch.from_numpy(v[4]))
+    setv.replay()
+    prod.replay()
+    same(4, Y)
+    same(4)
+    # values changed by a capture before the adjoint's tiles exist
+    G = rng.standard_normal((pat.n_rows, k))
+    _check(H, pat, v[4], G, transpose=True)
+    buf.copy_(torch.from_numpy(v[1]))
+    setv.replay()
+    _check(H, pat, v[1], G, transpose=True)
