@@ -154,6 +154,9 @@ struct vbcsr_matrix {
     std::vector<int64_t> struct_row, struct_col;   // first scalar row / column of every structure
     uint64_t *xdig = nullptr;
     size_t xdig_elems = 0;
+    uint64_t *sdpan = nullptr;   // fixed-point rows of A and B of the sliced pattern-sampled product
+    size_t sdpan_elems = 0;
+    bool sd_no_room = false;
     uint32_t *stab = nullptr;
     size_t stab_elems = 0;
     WorkItem *fwd_items = nullptr, *adj_items = nullptr;   // bucketed by row count
@@ -1449,6 +1452,9 @@ static int run_product(vbcsr_t *A, bool trans, int64_t k, double alpha, const vo
         sa.struct_rows = p.struct_rows;
         sa.struct_nnz = p.struct_nnz;
         sa.ldp = ldp8;
+        int ae = 0;
+        sa.alpha_pow2 = std::frexp(alpha, &ae) == 0.5 && std::abs(ae) < 128;
+        sa.alpha_exp = sa.alpha_pow2 ? ae - 1 : 0;
         a.queue = reinterpret_cast<long long *>(A->stab);
         per_item_dot = true;
         rc = launch(0, trans ? A->adj_lpt : A->fwd_lpt, n_all, 4, slice_kernel_ptr(trans, k), slice_smem_bytes());
@@ -1561,6 +1567,40 @@ static SddmmArgs sddmm_args(vbcsr_t *A) {
     return a;
 }
 
+// FP64 pattern-sampled product: sliced when it has enough work (below kSliceMinWork
+// the extra launch costs more than the multiply-adds), at k >= 2 (one column needs
+// half a clock an entry on the FP64 pipe, as much as the tensor-core tile) and up to
+// the widths whose level sums stay exact; else by multiply-adds, as on a stream that
+// is being captured before the buffers exist.
+static int run_sddmm_f64(vbcsr_t *A, const SddmmArgs &a, cudaStream_t s) {
+    bool sliced = a.k >= 2 && a.k <= kSliceKMax && a.alpha != 0.0 && A->nnz * a.k >= kSliceMinWork && !A->debug_checks;
+    if (sliced) {
+        const int64_t kp = (a.k + 15) / 16 * 16, rows = A->n_rows + A->n_cols;
+        const size_t need = (size_t)(rows * kp + (rows + 1) / 2);
+        if (need > A->sdpan_elems) {
+            if (A->sd_no_room || capturing(s)) {
+                sliced = false;
+            } else {
+                const int rc = grow(A, &A->sdpan, &A->sdpan_elems, need, s, "alloc fixed-point panels");
+                if (rc == VBCSR_ERR_NO_MEMORY) {
+                    A->sd_no_room = true;
+                    sliced = false;
+                } else if (rc) {
+                    return rc;
+                }
+            }
+        }
+        if (sliced) {
+            uint64_t *fa = A->sdpan, *fb = fa + A->n_rows * kp;
+            int32_t *ea = reinterpret_cast<int32_t *>(fb + A->n_cols * kp), *eb = ea + A->n_rows;
+            CUDA_TRY(launch_sddmm_sliced(a, A->n_rows, A->n_cols, fa, fb, ea, eb, s), "sddmm launch");
+            return VBCSR_OK;
+        }
+    }
+    CUDA_TRY(launch_sddmm(true, a, s), "sddmm launch");
+    return VBCSR_OK;
+}
+
 extern "C" int vbcsr_sddmm(vbcsr_t *A, int64_t k, double alpha, const void *Aop, int64_t lda, const void *Bop,
                            int64_t ldb, double beta, void *D, void *stream) {
     if (!A) return fail(VBCSR_ERR_INVALID_ARG, "handle is NULL");
@@ -1581,7 +1621,8 @@ extern "C" int vbcsr_sddmm(vbcsr_t *A, int64_t k, double alpha, const void *Aop,
     a.B = Bop;
     a.ldb = ldb;
     a.D = D;
-    CUDA_TRY(launch_sddmm(A->dtype == VBCSR_F64, a, (cudaStream_t)stream), "sddmm launch");
+    if (A->dtype == VBCSR_F64) return run_sddmm_f64(A, a, (cudaStream_t)stream);
+    CUDA_TRY(launch_sddmm(false, a, (cudaStream_t)stream), "sddmm launch");
     return VBCSR_OK;
 }
 
@@ -1754,7 +1795,7 @@ extern "C" int vbcsr_chebyshev_backward(vbcsr_t *A, int64_t k, const double *R, 
         a.B = T;
         a.ldb = wide;
         a.D = dvalues;
-        if (A->nnz) CUDA_TRY(launch_sddmm(true, a, s), "sddmm");
+        if (A->nnz && (rc = run_sddmm_f64(A, a, s))) return rc;
         first = false;
     }
     return VBCSR_OK;

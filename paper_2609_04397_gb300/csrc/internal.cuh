@@ -170,6 +170,7 @@ struct SliceArgs {
     const int32_t *struct_rows;   // X rows of every structure
     const int64_t *struct_nnz;    // stored entries of every structure
     int ldp;                      // k rounded up to 8
+    int alpha_pow2, alpha_exp;    // alpha = 2^alpha_exp: goes into the result's exponent
 };
 cudaError_t launch_slice_product(bool trans, const ProdArgs &a, const SliceArgs &q, cudaStream_t s);
 cudaError_t launch_slice_panel(const SliceChunk *chunks, int64_t n_chunks, const double *X, int64_t ldx, int k, int ldp,
@@ -282,6 +283,10 @@ struct SddmmArgs {
     void *D;
 };
 cudaError_t launch_sddmm(bool f64, const SddmmArgs &a, cudaStream_t s);
+// the same of FP64 operands on the FP16 tensor cores (sddmm_sliced.cu); fa, fb: rows x (k rounded
+// up to 16) words, ea, eb: one word a row
+cudaError_t launch_sddmm_sliced(const SddmmArgs &a, int64_t rows_a, int64_t rows_b, uint64_t *fa, uint64_t *fb, int32_t *ea,
+                                int32_t *eb, cudaStream_t s);
 
 // scatter (to_panel = true) or gather packed-order values <-> panels
 // reciprocal-space sampling (Eq. 4) of a k-space handle into packed complex values

@@ -66,21 +66,23 @@ __device__ __forceinline__ uint32_t slice_mag(double x) {
     return hi ? hi : ((uint32_t)b ? 1u : 0u);
 }
 
-// x at scale exponent E as a fixed-point integer plus 128 in every byte of the
-// low 7: byte b holds digit (6 - b) + 128. Integer arithmetic throughout (the
-// FP64 pipe is the scarce unit).
-constexpr uint64_t kSliceBias = 0x80808080808080ull;
+// x at scale exponent E as a fixed-point integer of D = 7 or 8 base-256 digits
+// plus 128 in every byte: byte b holds digit (D - 1 - b) + 128. Integer
+// arithmetic throughout (the FP64 pipe is the scarce unit).
+template <int D = kSliceDigits>
 __device__ __forceinline__ uint64_t slice_bytes(double x, int E) {
+    constexpr uint64_t kBias = D == 8 ? 0x8080808080808080ull : 0x80808080808080ull;
+    constexpr int kTop = D == 8 ? 10 : 2;          // shift of a 53-bit mantissa at the scale's own exponent
     const uint64_t b = (uint64_t)__double_as_longlong(x);
     const int eb = (int)((b >> 52) & 0x7ff);
     uint64_t m = b & 0xfffffffffffffull;
     if (eb) m |= 1ull << 52;
-    const int sh = 2 - (E - (eb ? eb : 1));        // value = m * 2^sh units, |.| < 2^55
+    const int sh = kTop - (E - (eb ? eb : 1));     // value = m * 2^sh units, |.| < 2^(8 D - 1)
     uint64_t v;
     if (sh >= 0) v = m << sh;
     else if (sh > -54) v = (m + (1ull << (-sh - 1))) >> -sh;
     else v = 0;
-    return (b >> 63) ? kSliceBias - v : kSliceBias + v;
+    return (b >> 63) ? kBias - v : kBias + v;
 }
 
 // two biased bytes as the f16 pair of their digits: 0x6400 | byte is 1024 + byte
@@ -90,22 +92,80 @@ __device__ __forceinline__ uint32_t slice_half2(uint32_t bytes, uint32_t sel) {
     return r;
 }
 
-// sum over levels of c[L] * 256^(7 - L) (each an integer below 2^24 in FP32),
-// rounded to FP64 once, times 2^e2
-__device__ __forceinline__ double slice_value(const float (&c)[kSliceLevels], int e2) {
-    int i[kSliceLevels];
+// The digits of four elements (K order) as f16 pairs: f[i][0] digit i of (v0, v1), f[i][1] of (v2, v3)
+template <int D>
+__device__ __forceinline__ void slice_pairs(const uint2 (&v)[4], uint32_t (&f)[D][2]) {
 #pragma unroll
-    for (int L = 0; L < kSliceLevels; ++L) i[L] = __float2int_rn(c[L]);
+    for (int h = 0; h < 2; ++h) {
+        const uint2 a = v[2 * h], b = v[2 * h + 1];
+        const uint32_t p[4] = {__byte_perm(a.x, b.x, 0x5140), __byte_perm(a.x, b.x, 0x7362),
+                               __byte_perm(a.y, b.y, 0x5140), __byte_perm(a.y, b.y, 0x7362)};
+#pragma unroll
+        for (int i = 0; i < D; ++i) {
+            const int byte = D - 1 - i;
+            f[i][h] = slice_half2(p[byte >> 1], byte & 1 ? 0x4342 : 0x4140);
+        }
+    }
+}
+
+// sum over levels of c[L] * 256^(7 - L), rounded to FP64 once (to nearest, ties
+// to even), times 2^e2, in integer arithmetic: with the sum's two halves
+// converted and joined on the FP64 pipe (4 of its operations an output, 64
+// clocks of an SM for a warp), the pattern-sampled kernel spent 80 % of its time there.
+// BOUND22: every |c| is below 2^22 (at most 16 terms a pair).
+template <bool BOUND22 = false>
+__device__ __forceinline__ double slice_value(const float (&c)[kSliceLevels], int e2) {
     long long p[2];
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
-        p[h] = ((long long)i[4 * h] << 24) + ((long long)i[4 * h + 1] << 16) +
-               (((long long)i[4 * h + 2] << 8) + i[4 * h + 3]);
-    // both parts are below 2^53: the fused multiply-add rounds their sum once
-    const double r = fma((double)p[0], 4294967296.0, (double)p[1]);
-    const uint64_t b = (uint64_t)__double_as_longlong(r);
-    // |e2| keeps the result normal (kSliceExpMin .. kSliceExpMax): scale by the exponent field
-    return r == 0.0 ? 0.0 : __longlong_as_double((long long)(b + ((uint64_t)(int64_t)e2 << 52)));
+    for (int h = 0; h < 2; ++h) {
+        if (BOUND22) {
+            // c + 1.5 * 2^23 holds the integer in its low bits over the constant below (full
+            // rate; a float-to-integer conversion runs at an eighth of it); two levels make
+            // one 32-bit integer
+            constexpr uint32_t kM = 0x4b400000u;
+            uint32_t b[4];
+#pragma unroll
+            for (int L = 0; L < 4; ++L) b[L] = __float_as_uint(__fadd_rn(c[4 * h + L], 12582912.f));
+            const int q0 = (int)(b[0] * 256u + (b[1] - kM * 257u)), q1 = (int)(b[2] * 256u + (b[3] - kM * 257u));
+            p[h] = (long long)q0 * 65536 + q1;
+        } else {
+            p[h] = __float2int_rn(c[4 * h]);
+#pragma unroll
+            for (int L = 1; L < 4; ++L) p[h] = p[h] * 256 + __float2int_rn(c[4 * h + L]);
+        }
+    }
+    // T = s * 2^32 + lo, then its magnitude m * 2^32 + mlo
+    const long long s = p[0] + (p[1] >> 32);
+    const uint32_t lo = (uint32_t)p[1];
+    const bool neg = s < 0;
+    uint64_t m = neg ? ~(uint64_t)s + (lo == 0) : (uint64_t)s;
+    uint32_t mlo = neg ? 0u - lo : lo;
+    int e = 1023 + 63 + 32;
+    if (m == 0) {
+        m = mlo;
+        mlo = 0;
+        e -= 32;
+    }
+    if (m == 0) return 0.0;
+    const int sh = __clzll((long long)m);
+    e -= sh;
+    // top: the leading 64 bits, the rest only counts as a sticky bit
+    uint64_t top = m << sh;
+    uint32_t rest;
+    if (sh < 32) {
+        top |= (uint64_t)mlo >> (32 - sh);
+        rest = mlo << sh;
+    } else {
+        top |= (uint64_t)mlo << (sh - 32);
+        rest = 0;
+    }
+    const uint32_t low11 = (uint32_t)top & 0x7ffu;
+    const uint64_t mant = top >> 11;
+    const uint32_t up = (low11 & 0x400u) && ((low11 & 0x3ffu) | rest | ((uint32_t)mant & 1u));
+    // the leading bit of mant adds one to the exponent field; |e2| keeps the result
+    // normal (kSliceExpMin .. kSliceExpMax)
+    const uint64_t bits = ((uint64_t)(e + e2 - 1) << 52) + mant + up;
+    return __longlong_as_double((long long)(bits | (neg ? 1ull << 63 : 0ull)));
 }
 
 // Carry the upper part of every level into the one above (exact: integers below 2^24)

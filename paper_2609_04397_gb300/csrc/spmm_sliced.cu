@@ -296,20 +296,7 @@ __global__ void __launch_bounds__(128, NT == 1 ? 4 : 3) slice_product_kernel(Pro
                     // B fragments: digit i of virtual columns (0, 1) and (2, 3) of the lane
                     uint32_t b[NT][kSliceDigits][2];
 #pragma unroll
-                    for (int n = 0; n < NT; ++n)
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            const uint2 u = x[n][2 * h], v = x[n][2 * h + 1];
-                            const uint32_t p0 = __byte_perm(u.x, v.x, 0x5140), p1 = __byte_perm(u.x, v.x, 0x7362);
-                            const uint32_t p2 = __byte_perm(u.y, v.y, 0x5140), p3 = __byte_perm(u.y, v.y, 0x7362);
-                            b[n][6][h] = slice_half2(p0, 0x4140);
-                            b[n][5][h] = slice_half2(p0, 0x4342);
-                            b[n][4][h] = slice_half2(p1, 0x4140);
-                            b[n][3][h] = slice_half2(p1, 0x4342);
-                            b[n][2][h] = slice_half2(p2, 0x4140);
-                            b[n][1][h] = slice_half2(p2, 0x4342);
-                            b[n][0][h] = slice_half2(p3, 0x4140);
-                        }
+                    for (int n = 0; n < NT; ++n) slice_pairs<kSliceDigits>(x[n], b[n]);
                     if (s + 1 < nsteps) load_x(s + 1);
                     const unsigned char *st = ring + (s % S) * kStage + g * 16 + t4 * 4;
 #pragma unroll
@@ -374,8 +361,8 @@ __global__ void __launch_bounds__(128, NT == 1 ? 4 : 3) slice_product_kernel(Pro
                         float lv[kSliceLevels];
 #pragma unroll
                         for (int L = 0; L < kSliceLevels; ++L) lv[L] = acc[n][L][2 * h + e];
-                        double o = slice_value(lv, eh + ex[n][e] - 2114);
-                        if (a.alpha != 1.0) o *= a.alpha;
+                        double o = slice_value(lv, eh + ex[n][e] - 2114 + q.alpha_exp);
+                        if (!q.alpha_pow2) o *= a.alpha;
                         if (a.beta_nz) o += a.beta * yrow[c];
                         if (a.gamma_nz) o += a.gamma * zrow[c];
                         yrow[c] = o;

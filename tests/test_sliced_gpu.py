@@ -206,3 +206,38 @@ def test_tiles_follow_the_values():
     buf.copy_(torch.from_numpy(v[1]))
     setv.replay()
     _check(H, pat, v[1], G, transpose=True)
+
+
+@pytest.mark.parametrize("k", [2, 7, 16, 17, 40, 200])
+def test_sliced_sddmm_against_oracle(k):
+    """The pattern-sampled product, contracting over the panel columns: row heights 1 to 33,
+    rows wider than the 512-column window, ragged tiles, leading dimensions above k, graded
+    rows, rows whose large columns do not meet, zero rows, Inf and NaN."""
+    pat = syn.random_pattern(230, 225, (1, 4, 9, 13, 33), 0.35, k, empty_rows=2, unsorted=True)
+    assert pat.nnz * k >= 1 << 22
+    H = _handle(pat, syn.random_values(pat, k))
+    rng = np.random.default_rng(k)
+    A0, B0 = rng.standard_normal((pat.n_rows, k + 1)), rng.standard_normal((pat.n_cols, k + 2))
+    D0 = rng.standard_normal(pat.nnz)
+    grade = 10.0 ** -np.arange(k + 2)
+    for A, B in ((A0, B0), (A0 * 10.0 ** rng.uniform(-30, 30, (pat.n_rows, 1)), B0),
+                 (A0 * np.clip(grade[:k + 1], 1e-30, None), B0 * np.clip(grade[k - 1::-1].tolist() + [1.0, 1.0], 1e-30, None))):
+        A, B = A.copy(), B.copy()
+        A[5] = 0.0
+        B[7] = 0.0
+        for alpha, beta in ((1.0, 0.0), (1.5, -0.5)):
+            Ad, Bd = torch.from_numpy(A).cuda()[:, :k], torch.from_numpy(B).cuda()[:, :k]
+            Dd = torch.from_numpy(D0.copy()).cuda()
+            H.sddmm(Ad, Bd, alpha, beta, Dd)
+            got = Dd.cpu().numpy()
+            ref = oracle.sddmm(pat, A[:, :k], B[:, :k], alpha, beta, D0)
+            scale = oracle.sddmm(pat, np.abs(A[:, :k]), np.abs(B[:, :k]), abs(alpha), 0.0) + abs(beta) * np.abs(D0)
+            assert (np.abs(got - ref) <= TOL * scale).all(), np.max(np.abs(got - ref) / np.maximum(scale, 1e-300))
+    A, B = A0.copy(), B0.copy()
+    A[3, 0], A[40, 1], B[9, 1], B[5] = np.nan, np.inf, -np.inf, 0.0
+    with np.errstate(invalid="ignore"):
+        ref = oracle.sddmm(pat, A[:, :k], B[:, :k], 1.0, 0.0, None)
+    got = H.sddmm(torch.from_numpy(A).cuda()[:, :k], torch.from_numpy(B).cuda()[:, :k]).cpu().numpy()
+    assert np.array_equal(np.isnan(got), np.isnan(ref)) and np.array_equal(np.isinf(got), np.isinf(ref))
+    assert any("slice_sddmm" in n for n in _kernels(lambda: H.sddmm(torch.from_numpy(A0).cuda()[:, :k],
+                                                                    torch.from_numpy(B0).cuda()[:, :k])))
