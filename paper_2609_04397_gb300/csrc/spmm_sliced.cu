@@ -162,7 +162,8 @@ __global__ void __launch_bounds__(128) slice_values_kernel(const WorkItem *items
 // ---------------------------------------------------------------------------
 // the product
 
-constexpr int kSliceStages = 5;   // value tiles in flight per warp (16 columns, up to 1792 bytes each)
+constexpr int kSliceList = (kSliceKMax + 16) * sizeof(int32_t);   // X rows of an item and of one step more
+constexpr int kSliceStages = 4;   // value tiles in flight per warp (16 columns, up to 1792 bytes each)
 
 template <int B, bool TRANS>
 __device__ __noinline__ void fma_item_fallback(const ProdArgs &a, const WorkItem &w, int kc, int32_t *s_x,
@@ -196,46 +197,201 @@ __device__ __noinline__ void fma_columns(const ProdArgs &a, int64_t n0, const Wo
 #undef VBCSR_SLICE_CASE
 }
 
-// One warp per work item (up to 16 output rows), passes of 8 NT columns, steps
-// of 16 virtual columns. A step's value tile (7 digits x B rows x 16 bytes,
-// contiguous) comes through a ring of shared-memory stages by asynchronous
-// copies; the 16 gathered X rows (8 bytes a column) are loaded to registers one
-// step ahead. Lane t4 of a fragment owns virtual columns 4 t4 .. 4 t4 + 3 of the
-// step (an order the A and B fragments share, so it does not matter to the
-// sums): their bytes are one 32-bit word of the value tile and four X loads.
-template <bool TRANS, int NT>
-__global__ void __launch_bounds__(128, NT == 1 ? 4 : 3) slice_product_kernel(ProdArgs a, SliceArgs q) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    constexpr int S = kSliceStages;
-    constexpr int kStage = 16 * kSliceTile;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+// One pass of an item: up to 16 columns (WIDE) or up to 8, steps of 16 virtual
+// columns. A step's value tile (7 digits x B rows x 16 bytes, contiguous) comes
+// through a ring of shared-memory stages by asynchronous copies; the 16 gathered
+// X rows (8 bytes a column) are loaded to registers one step ahead. Lane t4 of a
+// fragment owns virtual columns 4 t4 .. 4 t4 + 3 of the step (an order the two
+// operands share, so it does not matter to the sums): their bytes are one 32-bit
+// word of the value tile and four X loads.
+//
+// WIDE passes put the 16 columns on the M side of the MMA and the rows, NR
+// groups of 8, on the N side, so that items of up to 8 rows take half the MMAs
+// (and the outputs of a store are 8 consecutive columns); narrow ones put the
+// (up to 16) rows on the M side and the 8 columns on the N side. Returns false,
+// with nothing written, when an output is not resolved by the fixed point.
+template <bool TRANS, bool WIDE, int NR>
+__device__ __forceinline__ bool slice_pass(const ProdArgs &a, const SliceArgs &q, const WorkItem &w,
+                                           const unsigned char *vsrc, int nsteps, int64_t n0, const uint32_t *cmax,
+                                           unsigned char *ring, const int32_t *s_x, int lane, double &dot) {
+    constexpr int S = kSliceStages, kStage = 16 * kSliceTile;
+    constexpr int NX = WIDE ? 2 : 1, NA = WIDE ? NR : 1;
     const int g = lane >> 2, t4 = lane & 3;
-    unsigned char *ring = smem_raw + (size_t)warp * (S * kStage + kSliceKMax * sizeof(int32_t));
-    int32_t *s_x = reinterpret_cast<int32_t *>(ring + S * kStage);
-    const bool want_dot = a.item_partials != nullptr;
+    float acc[NA][kSliceLevels][4], low[NA][4];
+#pragma unroll
+    for (int n = 0; n < NA; ++n)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            low[n][j] = 0.f;
+#pragma unroll
+            for (int L = 0; L < kSliceLevels; ++L) acc[n][L][j] = 0.f;
+        }
+    if (nsteps > 0) {
+        const uint64_t *xd = q.xdig + n0 + g;
+        const int tile = w.B * kSliceTile;
+        // this lane's 16-byte chunks of a tile: lane, lane + 32, ... below 7 B (at most 4)
+        constexpr int kChunks = (16 * kSliceTile / 16 + 31) / 32;
+        bool mine[kChunks];
+#pragma unroll
+        for (int u = 0; u < kChunks; ++u) mine[u] = 16 * (lane + 32 * u) < tile;
+        const unsigned char *src = vsrc + 16 * lane;
+        auto issue = [&](int s) {   // steps are issued in order
+            const bool in = s < nsteps;
+            unsigned char *dst = ring + (s % S) * kStage + 16 * lane;
+#pragma unroll
+            for (int u = 0; u < kChunks; ++u)
+                if (in && mine[u]) cp_async16(dst + 512 * u, src + 512 * u);
+            src += tile;
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        uint2 x[NX][4];
+        auto load_x = [&](int s) {
+            const int4 xi = *reinterpret_cast<const int4 *>(s_x + 16 * s + 4 * t4);
+            const int row[4] = {xi.x, xi.y, xi.z, xi.w};
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const uint2 *p = reinterpret_cast<const uint2 *>(xd + (int64_t)row[r] * q.ldp);
+#pragma unroll
+                for (int n = 0; n < NX; ++n) x[n][r] = __ldg(p + 8 * n);
+            }
+        };
+        load_x(0);
+#pragma unroll
+        for (int s = 0; s < S - 1; ++s) issue(s);
+        const int digit = w.B * 16;   // bytes from a digit's plane of a tile to the next
+        int carry = kSliceFlush;
+        for (int s = 0; s < nsteps; ++s) {
+            asm volatile("cp.async.wait_group %0;" ::"n"(S - 2) : "memory");
+            __syncwarp();
+            issue(s + S - 1);
+            uint32_t b[NX][kSliceDigits][2];
+#pragma unroll
+            for (int n = 0; n < NX; ++n) slice_pairs<kSliceDigits>(x[n], b[n]);
+            load_x(s + 1);   // the list has one step past the last
+            const unsigned char *st = ring + (s % S) * kStage + g * 16 + t4 * 4;
+#pragma unroll
+            for (int i = 0; i < kSliceDigits; ++i, st += digit) {
+                // digit i of rows g (and g + 8)
+                uint32_t v[NR][2];
+#pragma unroll
+                for (int n = 0; n < NR; ++n) {
+                    const uint32_t word = *reinterpret_cast<const uint32_t *>(st + 128 * n);
+                    v[n][0] = slice_half2(word, 0x4140);
+                    v[n][1] = slice_half2(word, 0x4342);
+                }
+                const uint32_t rows[4] = {v[0][0], v[NR - 1][0], v[0][1], v[NR - 1][1]};   // M side of a narrow pass
+#pragma unroll
+                for (int j = 0; j < kSliceDigits && i + j < kSliceLevels; ++j) {
+                    if (WIDE) {
+                        const uint32_t cols[4] = {b[0][j][0], b[NX - 1][j][0], b[0][j][1], b[NX - 1][j][1]};
+#pragma unroll
+                        for (int n = 0; n < NA; ++n) mma_f16(acc[n][i + j], cols, v[n % NR][0], v[n % NR][1]);
+                    } else {
+                        mma_f16(acc[0][i + j], rows, b[0][j][0], b[0][j][1]);
+                    }
+                }
+                if (i == 0) {   // magnitudes of the leading digits
+                    constexpr uint32_t kAbs = 0x7fff7fffu;
+                    if (WIDE) {
+                        const uint32_t cols[4] = {b[0][0][0] & kAbs, b[NX - 1][0][0] & kAbs, b[0][0][1] & kAbs,
+                                                  b[NX - 1][0][1] & kAbs};
+#pragma unroll
+                        for (int n = 0; n < NA; ++n) mma_f16(low[n], cols, v[n % NR][0] & kAbs, v[n % NR][1] & kAbs);
+                    } else {
+                        const uint32_t r[4] = {rows[0] & kAbs, rows[1] & kAbs, rows[2] & kAbs, rows[3] & kAbs};
+                        mma_f16(low[0], r, b[0][0][0] & kAbs, b[0][0][1] & kAbs);
+                    }
+                }
+            }
+            if (--carry == 0) {
+                carry = kSliceFlush;
+#pragma unroll
+                for (int n = 0; n < NA; ++n) slice_carry(acc[n]);
+            }
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncwarp();
+    }
+    // accumulator j = 2 h + e of tile n: row and column (relative to the item and the pass)
+    auto row_of = [&](int n, int h, int e) { return WIDE ? 8 * n + 2 * t4 + e : g + 8 * h; };
+    auto col_of = [&](int h, int e) { return WIDE ? g + 8 * h : 2 * t4 + e; };
+    int er[NA][4], ec[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int64_t c = n0 + col_of(j >> 1, j & 1);
+        const uint32_t M = c < a.k ? cmax[c] : 0u;
+        ec[j] = M ? slice_exp(M) : 0;
+#pragma unroll
+        for (int n = 0; n < NA; ++n) {
+            const int r = row_of(n, j >> 1, j & 1);
+            er[n][j] = r < w.B ? q.rexp[w.yrow + r] : 0;
+        }
+    }
+    // every output's terms must be resolved by the fixed point (or be exactly zero)
+    bool ok = true;
+#pragma unroll
+    for (int n = 0; n < NA; ++n)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) ok &= er[n][j] >= 0 && (er[n][j] == 0 || ec[j] == 0 || low[n][j] >= kSliceGuard);
+    if (!__all_sync(0xffffffffu, ok)) return false;
+#pragma unroll
+    for (int n = 0; n < NA; ++n)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (!WIDE && NR == 1 && j >= 2) continue;
+            const int r = row_of(n, j >> 1, j & 1);
+            const int64_t c = n0 + col_of(j >> 1, j & 1);
+            if (r >= w.B || c >= a.k) continue;
+            const int64_t row = w.yrow + r;
+            float lv[kSliceLevels];
+#pragma unroll
+            for (int L = 0; L < kSliceLevels; ++L) lv[L] = acc[n][L][j];
+            double o = slice_value(lv, er[n][j] + ec[j] - 2114 + q.alpha_exp);
+            double *y = static_cast<double *>(a.Y) + row * a.ldy + c;
+            if (!q.alpha_pow2) o *= a.alpha;
+            if (a.beta_nz) o += a.beta * *y;
+            if (a.gamma_nz) o += a.gamma * static_cast<const double *>(a.Z)[row * a.ldz + c];
+            *y = o;
+            if (a.item_partials) dot += static_cast<const double *>(a.R)[row * a.ldr + c] * o;
+        }
+    return true;
+}
+
+// One warp per work item (up to 16 output rows); KWIDE: k > 8, passes of 16
+// columns with a last one of 8 where that is enough.
+template <bool TRANS, bool KWIDE>
+__global__ void __launch_bounds__(128, KWIDE ? 3 : 4) slice_product_kernel(ProdArgs a, SliceArgs q) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr int kRing = kSliceStages * 16 * kSliceTile;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    unsigned char *ring = smem_raw + (size_t)warp * (kRing + kSliceList);
+    int32_t *s_x = reinterpret_cast<int32_t *>(ring + kRing);
     double dot = 0.0;
 
+    // the next item is claimed when an item starts (lane 0's value counts)
+    auto claim = [&](int64_t from) -> unsigned long long {
+        if (!a.queue) return (unsigned long long)(from + (int64_t)gridDim.x * 4);
+        return lane == 0 ? atomicAdd(reinterpret_cast<unsigned long long *>(a.queue), 1ull) : 0ull;
+    };
+    int last_strct = -1;
+    bool last_plain = false;
     int64_t it = (int64_t)blockIdx.x * 4 + warp;
-    for (;;) {
-        if (a.queue) {
-            unsigned long long t = 0;
-            if (lane == 0) t = atomicAdd(reinterpret_cast<unsigned long long *>(a.queue), 1ull);
-            it = (int64_t)__shfl_sync(0xffffffffu, t, 0);
-        }
-        if (it >= a.n_items) break;
+    if (a.queue) it = (int64_t)__shfl_sync(0xffffffffu, claim(0), 0);
+    while (it < a.n_items) {
+        const unsigned long long next = claim(it);
         const WorkItem w = a.items[it];
         const SliceItem si = q.sitems[it];
         const uint32_t *cmax = q.cmax + (int64_t)si.strct * q.ldp;
-        // rows g, g + 8: scale exponents (0: zero row, -1: not sliced)
-        const int e0 = g < w.B ? q.rexp[w.yrow + g] : 0, e1 = g + 8 < w.B ? q.rexp[w.yrow + g + 8] : 0;
-        bool plain = si.doff < 0 || e0 < 0 || e1 < 0 || q.struct_nnz[si.strct] * a.k < kSliceMinWork;
-        {
-            // a structure with a column outside the sliced range, or mostly tiny, is not sliced
+        if (si.strct != last_strct) {
+            // a small structure, or one with a column outside the sliced range or mostly tiny, is not sliced
+            last_strct = si.strct;
             const uint32_t most = (uint32_t)q.struct_rows[si.strct] >> 2;
+            bool p = q.struct_nnz[si.strct] * a.k < kSliceMinWork;
             for (int c = lane; c < (int)a.k; c += 32)
-                plain |= !slice_exp_ok(cmax[c]) || q.ccnt[(int64_t)si.strct * q.ldp + c] > most;
+                p |= !slice_exp_ok(cmax[c]) || q.ccnt[(int64_t)si.strct * q.ldp + c] > most;
+            last_plain = __any_sync(0xffffffffu, p);
         }
-        plain = __any_sync(0xffffffffu, plain);
+        const bool plain = last_plain || si.doff < 0;
         const int nsteps = (w.K + 15) >> 4;
         const unsigned char *vsrc = q.vdig + si.doff;
         int64_t n0 = 0;
@@ -249,145 +405,45 @@ __global__ void __launch_bounds__(128, NT == 1 ? 4 : 3) slice_product_kernel(Pro
                 const int wd = TRANS ? a.tl.bi[l] : a.fl.w[l];
                 for (int t = 0; t < wd; ++t) s_x[pc + t] = xr + t;
                 if (e == w.nlist - 1)
-                    for (int t = w.K; t < 16 * nsteps; ++t) s_x[t] = xr;
+                    for (int t = w.K; t < 16 * nsteps + 16; ++t) s_x[t] = xr;
             }
             __syncwarp();
         }
-        for (; !plain && n0 < a.k; n0 += 8 * NT) {
-            float acc[NT][kSliceLevels][4], low[NT][4];
-#pragma unroll
-            for (int n = 0; n < NT; ++n)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    low[n][j] = 0.f;
-#pragma unroll
-                    for (int L = 0; L < kSliceLevels; ++L) acc[n][L][j] = 0.f;
-                }
-            if (nsteps > 0) {
-                const uint64_t *xd = q.xdig + n0 + g;
-                const bool two = NT == 2 && n0 + 8 < a.k;
-                auto issue = [&](int s) {
-                    if (s < nsteps) {
-                        unsigned char *dst = ring + (s % S) * kStage;
-                        const unsigned char *src = vsrc + (int64_t)s * w.B * kSliceTile;
-                        for (int c = lane; c < w.B * (kSliceTile / 16); c += 32) cp_async16(dst + 16 * c, src + 16 * c);
-                    }
-                    asm volatile("cp.async.commit_group;" ::: "memory");
-                };
-                uint2 x[NT][4];
-                auto load_x = [&](int s) {
-                    const int4 xi = *reinterpret_cast<const int4 *>(s_x + 16 * s + 4 * t4);
-                    const int row[4] = {xi.x, xi.y, xi.z, xi.w};
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) {
-                        const uint2 *p = reinterpret_cast<const uint2 *>(xd + (int64_t)row[r] * q.ldp);
-                        x[0][r] = __ldg(p);
-                        if (two) x[NT - 1][r] = __ldg(p + 8);
-                    }
-                };
-                load_x(0);
-#pragma unroll
-                for (int s = 0; s < S - 1; ++s) issue(s);
-                int flush = kSliceFlush;
-                for (int s = 0; s < nsteps; ++s) {
-                    asm volatile("cp.async.wait_group %0;" ::"n"(S - 2) : "memory");
-                    __syncwarp();
-                    issue(s + S - 1);
-                    // B fragments: digit i of virtual columns (0, 1) and (2, 3) of the lane
-                    uint32_t b[NT][kSliceDigits][2];
-#pragma unroll
-                    for (int n = 0; n < NT; ++n) slice_pairs<kSliceDigits>(x[n], b[n]);
-                    if (s + 1 < nsteps) load_x(s + 1);
-                    const unsigned char *st = ring + (s % S) * kStage + g * 16 + t4 * 4;
-#pragma unroll
-                    for (int i = 0; i < kSliceDigits; ++i) {
-                        const uint32_t lo = *reinterpret_cast<const uint32_t *>(st + i * w.B * 16);
-                        const uint32_t hi = *reinterpret_cast<const uint32_t *>(st + i * w.B * 16 + 128);
-                        uint32_t f[4] = {slice_half2(lo, 0x4140), slice_half2(hi, 0x4140), slice_half2(lo, 0x4342),
-                                         slice_half2(hi, 0x4342)};
-#pragma unroll
-                        for (int j = 0; j < kSliceDigits && i + j < kSliceLevels; ++j) {
-                            mma_f16(acc[0][i + j], f, b[0][j][0], b[0][j][1]);
-                            if (two) mma_f16(acc[NT - 1][i + j], f, b[NT - 1][j][0], b[NT - 1][j][1]);
-                        }
-                        if (i == 0) {   // magnitudes of the leading digits
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) f[j] &= 0x7fff7fffu;
-                            mma_f16(low[0], f, b[0][0][0] & 0x7fff7fffu, b[0][0][1] & 0x7fff7fffu);
-                            if (two)
-                                mma_f16(low[NT - 1], f, b[NT - 1][0][0] & 0x7fff7fffu, b[NT - 1][0][1] & 0x7fff7fffu);
-                        }
-                    }
-                    if (--flush == 0) {
-                        flush = kSliceFlush;
-#pragma unroll
-                        for (int n = 0; n < NT; ++n) slice_carry(acc[n]);
-                    }
-                }
-                asm volatile("cp.async.wait_all;" ::: "memory");
-                __syncwarp();
-            }
-            // every output's terms must be resolved by the fixed point (or be exactly zero)
-            int ex[NT][2];
+        if (!plain) {
             bool ok = true;
-#pragma unroll
-            for (int n = 0; n < NT; ++n)
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const int64_t c = n0 + 8 * n + 2 * t4 + e;
-                    const uint32_t M = c < a.k ? cmax[c] : 0u;
-                    ex[n][e] = slice_exp(M);
-                    if (M) {
-                        ok &= e0 == 0 || low[n][e] >= kSliceGuard;
-                        ok &= e1 == 0 || low[n][2 + e] >= kSliceGuard;
-                    }
-                }
-            if (!__all_sync(0xffffffffu, ok)) break;
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int r = g + 8 * h;
-                if (r >= w.B) continue;
-                const int64_t row = w.yrow + r;
-                const int eh = h ? e1 : e0;
-                double *yrow = static_cast<double *>(a.Y) + row * a.ldy;
-                const double *zrow = static_cast<const double *>(a.Z) + row * a.ldz;
-                const double *rrow = static_cast<const double *>(a.R) + row * a.ldr;
-#pragma unroll
-                for (int n = 0; n < NT; ++n)
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const int64_t c = n0 + 8 * n + 2 * t4 + e;
-                        if (c >= a.k) continue;
-                        float lv[kSliceLevels];
-#pragma unroll
-                        for (int L = 0; L < kSliceLevels; ++L) lv[L] = acc[n][L][2 * h + e];
-                        double o = slice_value(lv, eh + ex[n][e] - 2114 + q.alpha_exp);
-                        if (!q.alpha_pow2) o *= a.alpha;
-                        if (a.beta_nz) o += a.beta * yrow[c];
-                        if (a.gamma_nz) o += a.gamma * zrow[c];
-                        yrow[c] = o;
-                        if (want_dot) dot += rrow[c] * o;
-                    }
+            if (KWIDE)
+                for (; ok && n0 + 8 < a.k; n0 += ok ? 16 : 0)
+                    ok = w.B <= 8 ? slice_pass<TRANS, true, 1>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot)
+                                  : slice_pass<TRANS, true, 2>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot);
+            if (ok && n0 < a.k) {
+                ok = w.B <= 8 ? slice_pass<TRANS, false, 1>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot)
+                              : slice_pass<TRANS, false, 2>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot);
+                n0 += ok ? 8 : 0;
             }
         }
-        if (n0 < a.k) fma_columns<TRANS>(a, n0, w, ring, lane, dot);
-        if (want_dot) {
+        if (n0 < a.k) {
+            const WorkItem wc = w;   // copies: the call takes addresses, which would keep w and dot in memory
+            double dc = dot;
+            fma_columns<TRANS>(a, n0, wc, ring, lane, dc);
+            dot = dc;
+        }
+        if (a.item_partials) {
             // the item's share of the fused dot at the item's index (summed in a fixed order afterwards)
             for (int m = 16; m > 0; m >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, m);
             if (lane == 0) a.item_partials[it] = dot;
             dot = 0.0;
         }
-        if (!a.queue) it += (int64_t)gridDim.x * 4;
+        it = a.queue ? (int64_t)__shfl_sync(0xffffffffu, next, 0) : (int64_t)next;
     }
 }
 
 }  // namespace
 
-size_t slice_smem_bytes() { return 4 * ((size_t)kSliceStages * 16 * kSliceTile + kSliceKMax * sizeof(int32_t)); }
+size_t slice_smem_bytes() { return 4 * ((size_t)kSliceStages * 16 * kSliceTile + kSliceList); }
 
 const void *slice_kernel_ptr(bool trans, int64_t k) {
-    if (trans) return k <= 8 ? (const void *)slice_product_kernel<true, 1> : (const void *)slice_product_kernel<true, 2>;
-    return k <= 8 ? (const void *)slice_product_kernel<false, 1> : (const void *)slice_product_kernel<false, 2>;
+    if (trans) return k <= 8 ? (const void *)slice_product_kernel<true, false> : (const void *)slice_product_kernel<true, true>;
+    return k <= 8 ? (const void *)slice_product_kernel<false, false> : (const void *)slice_product_kernel<false, true>;
 }
 
 cudaError_t launch_slice_product(bool trans, const ProdArgs &a, const SliceArgs &q, cudaStream_t s) {
@@ -396,11 +452,11 @@ cudaError_t launch_slice_product(bool trans, const ProdArgs &a, const SliceArgs 
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     if (trans) {
-        if (a.k <= 8) slice_product_kernel<true, 1><<<a.grid, 128, smem, s>>>(a, q);
-        else slice_product_kernel<true, 2><<<a.grid, 128, smem, s>>>(a, q);
+        if (a.k <= 8) slice_product_kernel<true, false><<<a.grid, 128, smem, s>>>(a, q);
+        else slice_product_kernel<true, true><<<a.grid, 128, smem, s>>>(a, q);
     } else {
-        if (a.k <= 8) slice_product_kernel<false, 1><<<a.grid, 128, smem, s>>>(a, q);
-        else slice_product_kernel<false, 2><<<a.grid, 128, smem, s>>>(a, q);
+        if (a.k <= 8) slice_product_kernel<false, false><<<a.grid, 128, smem, s>>>(a, q);
+        else slice_product_kernel<false, true><<<a.grid, 128, smem, s>>>(a, q);
     }
     return cudaGetLastError();
 }
