@@ -170,7 +170,8 @@ struct vbcsr_matrix {
     int64_t *prow_ptr = nullptr, *d_row_off = nullptr;
     int32_t *d_row_b = nullptr;
     double *partials = nullptr;
-    double *item_partials = nullptr;   // one dot share per work item (persistent launches)
+    double *item_partials = nullptr;   // one dot share per work item, or group of its rows (persistent launches)
+    int64_t item_partials_n = 0;
     double *dot_scratch = nullptr;     // first-stage sums of long fixed-order reductions
     int *err = nullptr;
     int64_t device_bytes = 0;
@@ -224,6 +225,8 @@ static cudaError_t upload(vbcsr_matrix *A, T **dst, const std::vector<T> &src, c
 // validation and planning
 
 static const int32_t kMaxBlockSize = 4096;
+static const int kMaxRowSplit = 8;
+static const int64_t kMinItemPartials = 8192;   // above the warps of one launch, so that groups of rows fit
 
 static int validate_pattern(int64_t n_brows, int64_t n_bcols, const int32_t *row_bsize,
                             const int32_t *col_bsize, const int64_t *block_row_ptr,
@@ -617,8 +620,8 @@ static int build(vbcsr_matrix *A, int64_t n_brows, int64_t n_bcols, const int32_
         CUDA_TRY(upload(A, &A->tl_xrow, tl_xrow, s), "upload");
         CUDA_TRY(upload(A, &A->tl_vcol, tl_vcol, s), "upload");
     }
-    CUDA_TRY(A->alloc(&A->item_partials, (size_t)std::max(A->n_fwd_items, A->n_adj_items)),
-             "alloc per-item dot shares");
+    A->item_partials_n = std::max<int64_t>(std::max(A->n_fwd_items, A->n_adj_items), kMinItemPartials);
+    CUDA_TRY(A->alloc(&A->item_partials, (size_t)A->item_partials_n), "alloc per-item dot shares");
 
     A->h_rowptr = prow_ptr;
     A->h_ucol.assign(block_col_idx, block_col_idx + nblk);
@@ -1433,6 +1436,7 @@ static int run_product(vbcsr_t *A, bool trans, int64_t k, double alpha, const vo
                    : fma_f32_on_f64_kernel(trans, persistent, B, ring);
     };
     const int64_t n_all = trans ? A->n_adj_items : A->n_fwd_items;
+    int64_t n_dot = n_all;   // per-item dot shares
     int rc = VBCSR_OK;
     if (sliced) {
         // FP64 on the tensor cores (sliced.cuh): the digits of X, then one launch over every
@@ -1509,13 +1513,30 @@ static int run_product(vbcsr_t *A, bool trans, int64_t k, double alpha, const vo
             while ((1 << l) < kc_for(B)) ++l;
             a.kc_log2_by_b |= (uint64_t)l << (3 * B);
         }
-        a.queue = A->queue;
         per_item_dot = true;
-        CUDA_TRY(cudaMemsetAsync(A->queue, 0, sizeof(long long), s), "reset work counter");
         const int warps = A->persist_warps ? A->persist_warps : 4;
-        rc = launch(0, trans ? A->adj_lpt : A->fwd_lpt, n_all, warps,
-                    split ? fma_split_kernel(mma_mode) : fma_kern(true, 0),
-                    fma_smem_bytes(trans, warps, a.value_ring != 0));
+        const void *kern = split ? fma_split_kernel(mma_mode) : fma_kern(true, 0);
+        const size_t smem = fma_smem_bytes(trans, warps, a.value_ring != 0);
+        const int cap = cached_cap(kern, warps, smem);
+        if (cap < 0) return cuda_fail(cudaGetLastError(), "occupancy query of the product kernel");
+        // a small FP64 operator leaves most of the chip idle behind the latency of a few
+        // warps: cut its items into groups of rows while the groups still all run at once
+        // (at most 8: one or two rows each)
+        int64_t units = n_all;
+        if (mode == VBCSR_PREC_NATIVE && f64) {
+            a.row_split = 1;
+            while (a.row_split < kMaxRowSplit && units * 2 <= (int64_t)cap * warps && units * 2 <= A->item_partials_n) {
+                a.row_split *= 2;
+                units *= 2;
+            }
+        }
+        // every unit has a warp of its own: no queue
+        if ((units + warps - 1) / warps > cap) {
+            a.queue = A->queue;
+            CUDA_TRY(cudaMemsetAsync(A->queue, 0, sizeof(long long), s), "reset work counter");
+        }
+        n_dot = units;
+        rc = launch(0, trans ? A->adj_lpt : A->fwd_lpt, units, warps, kern, smem);
     } else {
         const std::vector<Bucket> &buckets = trans ? A->adj_buckets : A->fwd_buckets;
         const WorkItem *items = trans ? A->adj_items : A->fwd_items;
@@ -1529,7 +1550,7 @@ static int run_product(vbcsr_t *A, bool trans, int64_t k, double alpha, const vo
     }
     if (rc) return rc;
     if (want_dot)
-        CUDA_TRY(launch_finalize_dot(per_item_dot ? A->item_partials : A->partials, per_item_dot ? n_all : used,
+        CUDA_TRY(launch_finalize_dot(per_item_dot ? A->item_partials : A->partials, per_item_dot ? n_dot : used,
                                      dot_scale, epi->dot_out, A->dot_scratch, s),
                  "dot finalize");
     return VBCSR_OK;

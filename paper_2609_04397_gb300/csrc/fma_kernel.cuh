@@ -345,7 +345,11 @@ __device__ __forceinline__ void process_item(const ProdArgs &a, const WorkItem &
                     // count, and a persistent launch that runs many row counts at once
                     // (measured: nine on a variable-block operator with b in [9, 20]) ran
                     // 1.4x slower with it, while one or two row counts ran 3-10 % faster.
+                    // FP64 items of few rows (groups of rows of a small operator) take several
+                    // steps' loads at once: nothing else hides their latency
                     constexpr int CPL = sizeof(TA) == 8 && alignof(TA) == 8 ? 2 : (WIDE && B <= 13 ? 4 : 2);
+                    constexpr int kUnroll = sizeof(TA) == 8 && alignof(TA) == 8 && B <= 4 ? 4 : 1;
+#pragma unroll kUnroll
                     for (int t = CPL * tg; t < tn; t += CPL * TG) {
                         TA x[CPL];
 #pragma unroll
@@ -473,7 +477,9 @@ __global__ void __launch_bounds__(256, 2) fma_product_kernel(ProdArgs a) {
 // One launch over items of every row count. Items come from a.items in
 // order (the planner sorts them by descending cost); warps take the next
 // item from a device counter (a.queue, zeroed before the launch) or, without
-// a queue, round-robin. a.kc_of(B) is the column tile of row count B.
+// a queue, round-robin. a.kc_of(B) is the column tile of row count B. With
+// a.row_split > 1 an item is cut into that many groups of rows, one warp each
+// (a.n_items counts the groups).
 template <bool TRANS, typename TV, typename TA, typename TX, typename TXI, bool WIDE = true, bool RING = false>
 __global__ void __launch_bounds__(256, 2) fma_persistent_kernel(ProdArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -494,8 +500,16 @@ __global__ void __launch_bounds__(256, 2) fma_persistent_kernel(ProdArgs a) {
             it = (int64_t)__shfl_sync(0xffffffffu, q, 0);
         }
         if (it >= a.n_items) break;
-        const WorkItem w = a.items[it];
+        WorkItem w = a.items[a.row_split > 1 ? it / a.row_split : it];
         const int kc = a.kc_of(w.B);
+        if (a.row_split > 1) {
+            // rows [p0, p1) of the item: the same sums in the same order, more warps
+            const int c = (int)(it % a.row_split), p0 = w.B * c / a.row_split, p1 = w.B * (c + 1) / a.row_split;
+            if (TRANS) w.Kp += p0;
+            else w.vbase += (int64_t)p0 * w.Kp;
+            w.yrow += p0;
+            w.B = p1 - p0;
+        }
 #define VBCSR_ITEM_CASE(NB) \
     case NB: process_item<NB, TRANS, TV, TA, TX, TXI, WIDE, RING>(a, w, kc, s_x, s_a, s_ring, lane, dot); break;
         switch (w.B) {

@@ -94,6 +94,7 @@ struct ProdArgs {
     int warps;              // warps per CTA
     // persistent launch only
     long long *queue;       // device work counter, zero at launch (NULL: round-robin)
+    int row_split;          // groups of rows an item is cut into, one warp each (0, 1: whole items)
     uint64_t kc_log2_by_b;  // 3 bits per row count B = 1..16: log2 of its column tile
     int mma_staged;         // tensor-core forward: 1 = value panels staged in shared memory
     int value_ring;         // CUDA-core forward, FP32 values, k >= 4: read them through the ring
