@@ -948,18 +948,16 @@ static int slices_changed(vbcsr_t *A, cudaStream_t s) {
     return VBCSR_OK;
 }
 
-// True when a native FP64 product of k columns runs sliced. From two columns:
-// at one column the multiply-add kernel needs 2 FP64 operations per 8 stored
-// bytes and the value tiles are 12 bytes per entry, so there is nothing to gain.
+// True when a native FP64 product of k columns runs sliced.
 static bool slice_applies(const vbcsr_t *A, bool trans, int64_t k) {
     const SlicePlan &p = A->slice[trans];
-    return p.applies && !p.untracked && k >= 2 && k <= (1 << 20) && p.max_nnz * k >= kSliceMinWork && !A->debug_checks;
+    return p.applies && !p.untracked && k <= (1 << 20) && p.max_nnz * k >= slice_min_work(k) && !A->debug_checks;
 }
 
 static size_t slice_tab_elems(const vbcsr_t *A, int64_t ldp) { return 4 + 2 * (size_t)A->n_structs * (size_t)ldp; }
 
 static bool slice_buffers_ready(const vbcsr_t *A, bool trans, int64_t k) {
-    const int64_t ldp = (k + 7) / 8 * 8, xrows = trans ? A->n_rows : A->n_cols;
+    const int64_t ldp = slice_ldp(k), xrows = trans ? A->n_rows : A->n_cols;
     return A->slice[trans].vdig && A->xdig_elems >= (size_t)(xrows * ldp) &&
            A->stab_elems >= slice_tab_elems(A, ldp);
 }
@@ -1198,7 +1196,7 @@ static int slice_prepare(vbcsr_t *A, bool trans, int64_t k, bool may_alloc, cuda
         return VBCSR_OK;
     }
     if (!may_alloc || p.no_room || cap) return VBCSR_OK;
-    const int64_t ldp = (k + 7) / 8 * 8, xrows = trans ? A->n_rows : A->n_cols;
+    const int64_t ldp = slice_ldp(k), xrows = trans ? A->n_rows : A->n_cols;
     int rc = VBCSR_OK;
     if (!p.vdig) {
         cudaError_t e = p.rexp ? cudaSuccess : A->alloc(&p.rexp, (size_t)(trans ? A->n_cols : A->n_rows));
@@ -1442,10 +1440,10 @@ static int run_product(vbcsr_t *A, bool trans, int64_t k, double alpha, const vo
         // FP64 on the tensor cores (sliced.cuh): the digits of X, then one launch over every
         // item; the CUDA-core schedule and tiles do not apply
         const SlicePlan &p = A->slice[trans];
-        const int ldp8 = (int)((k + 7) / 8 * 8);
-        uint32_t *cmax = A->stab + 4, *ccnt = cmax + (size_t)A->n_structs * ldp8;
-        CUDA_TRY(cudaMemsetAsync(A->stab, 0, slice_tab_elems(A, ldp8) * sizeof(uint32_t), s), "reset column maxima");
-        CUDA_TRY(launch_slice_panel(p.chunks, p.n_chunks, (const double *)X, ldx, (int)k, ldp8, cmax, ccnt, A->xdig, s),
+        const int xld = slice_ldp(k);
+        uint32_t *cmax = A->stab + 4, *ccnt = cmax + (size_t)A->n_structs * xld;
+        CUDA_TRY(cudaMemsetAsync(A->stab, 0, slice_tab_elems(A, xld) * sizeof(uint32_t), s), "reset column maxima");
+        CUDA_TRY(launch_slice_panel(p.chunks, p.n_chunks, (const double *)X, ldx, (int)k, xld, cmax, ccnt, A->xdig, s),
                  "slice X");
         sa.sitems = p.items;
         sa.vdig = p.vdig;
@@ -1455,7 +1453,7 @@ static int run_product(vbcsr_t *A, bool trans, int64_t k, double alpha, const vo
         sa.ccnt = ccnt;
         sa.struct_rows = p.struct_rows;
         sa.struct_nnz = p.struct_nnz;
-        sa.ldp = ldp8;
+        sa.ldp = xld;
         int ae = 0;
         sa.alpha_pow2 = std::frexp(alpha, &ae) == 0.5 && std::abs(ae) < 128;
         sa.alpha_exp = sa.alpha_pow2 ? ae - 1 : 0;
@@ -1588,13 +1586,13 @@ static SddmmArgs sddmm_args(vbcsr_t *A) {
     return a;
 }
 
-// FP64 pattern-sampled product: sliced when it has enough work (below kSliceMinWork
-// the extra launch costs more than the multiply-adds), at k >= 2 (one column needs
-// half a clock an entry on the FP64 pipe, as much as the tensor-core tile) and up to
-// the widths whose level sums stay exact; else by multiply-adds, as on a stream that
+// FP64 pattern-sampled product: sliced when it has enough work (below, the extra
+// launch costs more than the multiply-adds), at k >= 2 (one column needs half a
+// clock an entry on the FP64 pipe, as much as the tensor-core tile) and up to the
+// widths whose level sums stay exact; else by multiply-adds, as on a stream that
 // is being captured before the buffers exist.
 static int run_sddmm_f64(vbcsr_t *A, const SddmmArgs &a, cudaStream_t s) {
-    bool sliced = a.k >= 2 && a.k <= kSliceKMax && a.alpha != 0.0 && A->nnz * a.k >= kSliceMinWork && !A->debug_checks;
+    bool sliced = a.k >= 2 && a.k <= kSliceKMax && a.alpha != 0.0 && A->nnz * a.k >= slice_min_work(3) && !A->debug_checks;
     if (sliced) {
         const int64_t kp = (a.k + 15) / 16 * 16, rows = A->n_rows + A->n_cols;
         const size_t need = (size_t)(rows * kp + (rows + 1) / 2);

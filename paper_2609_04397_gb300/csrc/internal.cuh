@@ -158,7 +158,15 @@ struct SliceItem {
     int32_t strct;    // structure (of a batched operator) whose X columns the item reads
     int32_t pad;
 };
-constexpr int64_t kSliceMinWork = 1 << 22;   // stored entries x columns of a structure below which it is not sliced
+// Stored entries x columns of a structure from which it is sliced. Below, the passes over X
+// and the launches cost more than the multiply-adds: at k >= 3 that is a few microseconds
+// (700 atoms, k = 8: 45 against 86 us; 200 atoms: 26 against 16). One and two columns leave
+// the multiply-add kernel closer to the memory: k = 1 on the 50k-atom operator (1.7e8
+// entries) 0.32 against 0.37 ms, on 20k disordered atoms (3.8e7) 0.128 against 0.111; k = 2
+// there 0.157 against 0.196, on 2500 atoms (7.6e6) 0.060 against 0.054.
+__host__ __device__ constexpr int64_t slice_min_work(int64_t k) {
+    return k == 1 ? (int64_t)1 << 26 : k == 2 ? (int64_t)1 << 25 : (int64_t)1 << 22;
+}
 struct SliceChunk {   // X rows of one structure
     int32_t row0, nrows, strct;
 };
@@ -170,7 +178,7 @@ struct SliceArgs {
     const uint32_t *cmax, *ccnt;  // [structures, ldp]: high word of the column maxima, tiny elements
     const int32_t *struct_rows;   // X rows of every structure
     const int64_t *struct_nnz;    // stored entries of every structure
-    int ldp;                      // k rounded up to 8
+    int ldp;                      // slice_ldp(k)
     int alpha_pow2, alpha_exp;    // alpha = 2^alpha_exp: goes into the result's exponent
 };
 cudaError_t launch_slice_product(bool trans, const ProdArgs &a, const SliceArgs &q, cudaStream_t s);
@@ -180,6 +188,8 @@ cudaError_t launch_slice_values(bool trans, const WorkItem *items, const SliceIt
                                 const AdjList &tl, const double *panel, uint8_t *dig, int32_t *rexp, cudaStream_t s);
 const void *slice_kernel_ptr(bool trans, int64_t k);
 size_t slice_smem_bytes();
+constexpr int kSliceThin = 3;         // widest product with the digits of X on the N side
+int slice_ldp(int64_t k);             // columns of the fixed-point X
 
 // Scalar (all 1 x 1 blocks) operators: L lanes per row (2, 4 or 8 for the
 // FP64 and double-FP32 kinds, 4, 8, 16 or 32 for the FP32 ones; csr_lane_class

@@ -10,8 +10,8 @@ namespace {
 // ---------------------------------------------------------------------------
 // X: column maxima per structure, then the digits
 
-// One CTA per chunk of X rows (rows of one structure); thread tx of TX takes
-// columns tx, tx + TX, ..., threads ty stride the rows.
+// A CTA takes `per` consecutive chunks of X rows (each of one structure);
+// thread tx of TX takes columns tx, tx + TX, ..., threads ty stride the rows.
 struct ColWalk {
     int tx, ty, TX, TY;
     __device__ __forceinline__ ColWalk(int cols) {
@@ -23,17 +23,32 @@ struct ColWalk {
     }
 };
 
-__global__ void __launch_bounds__(256) slice_colmax_kernel(const SliceChunk *chunks, int64_t n_chunks, const double *X,
-                                                           int64_t ldx, int k, int ldp, uint32_t *cmax) {
+// f(row0, rows, structure, last) over the CTA's chunks; `last` marks the end of a
+// structure's run of chunks
+template <typename F>
+__device__ __forceinline__ void over_chunks(const SliceChunk *chunks, int64_t n_chunks, int per, F f) {
+    const int64_t q1 = min(n_chunks, ((int64_t)blockIdx.x + 1) * per);
+    for (int64_t q = (int64_t)blockIdx.x * per; q < q1; ++q) {
+        const SliceChunk c = chunks[q];
+        f(c, q + 1 == q1 || chunks[q + 1].strct != c.strct);
+    }
+}
+
+__global__ void __launch_bounds__(256) slice_colmax_kernel(const SliceChunk *chunks, int64_t n_chunks, int per,
+                                                           const double *__restrict__ X, int64_t ldx, int k, int ldp,
+                                                           uint32_t *cmax) {
     __shared__ uint32_t red[256];
     const ColWalk w(k);
-    for (int64_t q = blockIdx.x; q < n_chunks; q += gridDim.x) {
-        const SliceChunk c = chunks[q];
-        for (int c0 = 0; c0 < k; c0 += w.TX) {
-            const int col = c0 + w.tx;
-            uint32_t m = 0;
-            if (col < k)
-                for (int r = w.ty; r < c.nrows; r += w.TY) m = max(m, slice_mag(X[(int64_t)(c.row0 + r) * ldx + col]));
+    for (int c0 = 0; c0 < k; c0 += w.TX) {
+        const int col = c0 + w.tx;
+        uint32_t m = 0;
+        over_chunks(chunks, n_chunks, per, [&](const SliceChunk &c, bool last) {
+            if (col < k) {
+                const double *x = X + (int64_t)c.row0 * ldx + col;
+#pragma unroll 4
+                for (int r = w.ty; r < c.nrows; r += w.TY) m = max(m, slice_mag(x[(int64_t)r * ldx]));
+            }
+            if (!last) return;
             __syncthreads();
             red[threadIdx.x] = m;
             __syncthreads();
@@ -42,34 +57,38 @@ __global__ void __launch_bounds__(256) slice_colmax_kernel(const SliceChunk *chu
                 __syncthreads();
             }
             if (w.ty == 0 && col < k && red[w.tx]) atomicMax(cmax + (int64_t)c.strct * ldp + col, red[w.tx]);
-        }
+            m = 0;
+        });
     }
 }
 
 // X as biased fixed point [rows, ldp] (8 bytes an element, 7 of them digits);
 // columns k .. ldp - 1 are zero. ccnt counts the elements below 2^-10 of their
 // column's maximum.
-__global__ void __launch_bounds__(256) slice_panel_kernel(const SliceChunk *chunks, int64_t n_chunks, const double *X,
-                                                          int64_t ldx, int k, int ldp, const uint32_t *cmax,
-                                                          uint32_t *ccnt, uint64_t *out) {
+__global__ void __launch_bounds__(256) slice_panel_kernel(const SliceChunk *chunks, int64_t n_chunks, int per,
+                                                          const double *__restrict__ X, int64_t ldx, int k, int ldp,
+                                                          const uint32_t *__restrict__ cmax, uint32_t *ccnt,
+                                                          uint64_t *__restrict__ out) {
     __shared__ uint32_t red[256];
     const ColWalk w(ldp);
-    for (int64_t q = blockIdx.x; q < n_chunks; q += gridDim.x) {
-        const SliceChunk c = chunks[q];
-        for (int c0 = 0; c0 < ldp; c0 += w.TX) {
-            const int col = c0 + w.tx;
-            uint32_t tiny = 0;
+    for (int c0 = 0; c0 < ldp; c0 += w.TX) {
+        const int col = c0 + w.tx;
+        uint32_t tiny = 0;
+        over_chunks(chunks, n_chunks, per, [&](const SliceChunk &c, bool last) {
             if (col < ldp) {
                 const uint32_t M = col < k ? cmax[(int64_t)c.strct * ldp + col] : 0u;
                 const bool live = M != 0 && slice_exp_ok(M);
                 const int E = slice_exp(M);
+                const double *x = X + (int64_t)c.row0 * ldx + (live ? col : 0);
+                uint64_t *o = out + (int64_t)c.row0 * ldp + col;
+#pragma unroll 4
                 for (int r = w.ty; r < c.nrows; r += w.TY) {
-                    const double x = live ? X[(int64_t)(c.row0 + r) * ldx + col] : 0.0;
-                    tiny += (slice_mag(x) >> 20) + 10 < (M >> 20);
-                    out[(int64_t)(c.row0 + r) * ldp + col] = slice_bytes(x, E);
+                    const double v = live ? x[(int64_t)r * ldx] : 0.0;
+                    tiny += live && (slice_mag(v) >> 20) + 10 < (M >> 20);
+                    o[(int64_t)r * ldp] = slice_bytes(v, E);
                 }
-                if (!live) tiny = 0;
             }
+            if (!last) return;
             __syncthreads();
             red[threadIdx.x] = tiny;
             __syncthreads();
@@ -78,14 +97,69 @@ __global__ void __launch_bounds__(256) slice_panel_kernel(const SliceChunk *chun
                 __syncthreads();
             }
             if (w.ty == 0 && col < k && red[w.tx]) atomicAdd(ccnt + (int64_t)c.strct * ldp + col, red[w.tx]);
-        }
+            tiny = 0;
+        });
     }
 }
 
 // ---------------------------------------------------------------------------
 // values: one warp per work item; row maxima, then 16-column tiles of digits
 // [tile][digit][row][16 columns], two tiles at a time staged in shared memory
-// and stored 16 bytes a lane
+// and stored 16 bytes a lane. Forward items are read with the lanes along a row
+// of the page; adjoint ones (TRANS), whose rows are the columns of the pages'
+// blocks, with BP = 1, 2, 4, 8 or 16 lanes along the item's rows (consecutive in
+// the pages) and 32 / BP virtual columns a load: with a virtual column per lane
+// every load touched 32 sectors (0.47 ms for 3.8e7 entries, the forward
+// form 0.18).
+
+// the digits of element (row p, column t of the two staged tiles)
+__device__ __forceinline__ void stage_digits(uint8_t *stage, int B, int p, int t, double v, int E) {
+    const uint64_t u = slice_bytes(E > 0 ? v : 0.0, E);
+    uint8_t *o = stage + (t >> 4) * B * kSliceTile + p * 16 + (t & 15);
+#pragma unroll
+    for (int i = 0; i < kSliceDigits; ++i) o[i * B * 16] = (uint8_t)(u >> (8 * (6 - i)));
+}
+
+// 16 loads of an adjoint item at once: row q of virtual columns t0 + u * (32 / BP) + lane / BP, u < BP
+template <int BP>
+__device__ __forceinline__ void adj_columns(const double *panel, const int64_t *s_a, const WorkItem &w, int t0, int lane,
+                                            double (&v)[BP]) {
+    const int q = lane % BP;
+#pragma unroll
+    for (int u = 0; u < BP; ++u) {
+        const int t = t0 + u * (32 / BP) + lane / BP;
+        v[u] = t < w.K && q < w.B ? panel[s_a[t] + q] : 0.0;
+    }
+}
+
+template <int BP>
+__device__ __forceinline__ void adj_item_digits(const double *panel, const int64_t *s_a, const WorkItem &w, uint8_t *dst,
+                                                uint8_t *stage, int32_t *rexp, int lane) {
+    uint32_t m = 0;
+    for (int t0 = 0; t0 < w.K; t0 += 32) {
+        double v[BP];
+        adj_columns<BP>(panel, s_a, w, t0, lane, v);
+#pragma unroll
+        for (int u = 0; u < BP; ++u) m = max(m, slice_mag(v[u]));
+    }
+#pragma unroll
+    for (int h = BP; h < 32; h <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, h));
+    const int E = m == 0 ? 0 : (slice_exp_ok(m) ? slice_exp(m) : -1), q = lane % BP;
+    if (lane < w.B) rexp[w.yrow + lane] = E;
+    const int nt = (w.K + 15) >> 4;
+    for (int c = 0; c < nt; c += 2) {
+        double v[BP];
+        adj_columns<BP>(panel, s_a, w, 16 * c, lane, v);
+        if (q < w.B)
+#pragma unroll
+            for (int u = 0; u < BP; ++u) stage_digits(stage, w.B, q, u * (32 / BP) + lane / BP, v[u], E);
+        __syncwarp();
+        uint4 *d = reinterpret_cast<uint4 *>(dst + (int64_t)c * w.B * kSliceTile);
+        const int n = min(2, nt - c) * w.B * (kSliceTile / 16);
+        for (int e = lane; e < n; e += 32) d[e] = reinterpret_cast<uint4 *>(stage)[e];
+        __syncwarp();
+    }
+}
 
 template <bool TRANS>
 __global__ void __launch_bounds__(128) slice_values_kernel(const WorkItem *items, const SliceItem *sitems,
@@ -100,7 +174,7 @@ __global__ void __launch_bounds__(128) slice_values_kernel(const WorkItem *items
         const WorkItem w = items[it];
         const SliceItem si = sitems[it];
         if (si.doff < 0) continue;   // too wide: never sliced
-        if (TRANS) {
+        if constexpr (TRANS) {
             __syncwarp();
             for (int e = lane; e < w.nlist; e += 32) {
                 const int64_t l = w.lbegin + e;
@@ -109,52 +183,53 @@ __global__ void __launch_bounds__(128) slice_values_kernel(const WorkItem *items
                 for (int p = 0; p < bi; ++p) s_a[vc + p] = pb + (int64_t)p * kp + w.Kp;
             }
             __syncwarp();
-        }
-        const double *src = TRANS ? panel : panel + w.vbase;
-        const int64_t ps = TRANS ? 1 : w.Kp;                    // from a row to the next
-        auto load = [&](int t, double (&v)[16]) {               // column t of the item, all rows at once
-            const bool in = t < w.K;
-            const double *c = src + (in ? (TRANS ? s_a[t] : t) : 0);
+            uint8_t *dst = dig + si.doff;
+            if (w.B > 8) adj_item_digits<16>(panel, s_a, w, dst, stage, rexp, lane);
+            else if (w.B > 4) adj_item_digits<8>(panel, s_a, w, dst, stage, rexp, lane);
+            else if (w.B > 2) adj_item_digits<4>(panel, s_a, w, dst, stage, rexp, lane);
+            else adj_item_digits<2>(panel, s_a, w, dst, stage, rexp, lane);
+        } else {
+            const double *src = panel + w.vbase;
+            auto load = [&](int t, double (&v)[16]) {               // column t of the item, all rows at once
+                const bool in = t < w.K;
+                const double *c = src + (in ? t : 0);
 #pragma unroll
-            for (int p = 0; p < 16; ++p) v[p] = in && p < w.B ? c[p * ps] : 0.0;
-        };
-        uint32_t m[16];
+                for (int p = 0; p < 16; ++p) v[p] = in && p < w.B ? c[(int64_t)p * w.Kp] : 0.0;
+            };
+            uint32_t m[16];
 #pragma unroll
-        for (int p = 0; p < 16; ++p) m[p] = 0;
-        for (int t = lane; t < w.K; t += 32) {
-            double v[16];
-            load(t, v);
+            for (int p = 0; p < 16; ++p) m[p] = 0;
+            for (int t = lane; t < w.K; t += 32) {
+                double v[16];
+                load(t, v);
 #pragma unroll
-            for (int p = 0; p < 16; ++p) m[p] = max(m[p], slice_mag(v[p]));
-        }
-#pragma unroll
-        for (int p = 0; p < 16; ++p) {
-            const uint32_t r = __reduce_max_sync(0xffffffffu, m[p]);
-            const int e = r == 0 ? 0 : (slice_exp_ok(r) ? slice_exp(r) : -1);
-            if (lane == p) {
-                s_e[warp][p] = e;
-                if (p < w.B) rexp[w.yrow + p] = e;
+                for (int p = 0; p < 16; ++p) m[p] = max(m[p], slice_mag(v[p]));
             }
-        }
-        __syncwarp();
-        const int nt = (w.K + 15) >> 4;
-        for (int c = 0; c < nt; c += 2) {
-            double v[16];
-            load(16 * c + lane, v);
-            uint8_t *o = stage + (lane >> 4) * w.B * kSliceTile + (lane & 15);
 #pragma unroll
             for (int p = 0; p < 16; ++p) {
-                if (p >= w.B) break;
-                const int E = s_e[warp][p];
-                const uint64_t u = slice_bytes(E > 0 ? v[p] : 0.0, E);
-#pragma unroll
-                for (int i = 0; i < kSliceDigits; ++i) o[(i * w.B + p) * 16] = (uint8_t)(u >> (8 * (6 - i)));
+                const uint32_t r = __reduce_max_sync(0xffffffffu, m[p]);
+                const int e = r == 0 ? 0 : (slice_exp_ok(r) ? slice_exp(r) : -1);
+                if (lane == p) {
+                    s_e[warp][p] = e;
+                    if (p < w.B) rexp[w.yrow + p] = e;
+                }
             }
             __syncwarp();
-            uint4 *dst = reinterpret_cast<uint4 *>(dig + si.doff + (int64_t)c * w.B * kSliceTile);
-            const int n = min(2, nt - c) * w.B * (kSliceTile / 16);
-            for (int q = lane; q < n; q += 32) dst[q] = reinterpret_cast<uint4 *>(stage)[q];
-            __syncwarp();
+            const int nt = (w.K + 15) >> 4;
+            for (int c = 0; c < nt; c += 2) {
+                double v[16];
+                load(16 * c + lane, v);
+#pragma unroll
+                for (int p = 0; p < 16; ++p) {
+                    if (p >= w.B) break;
+                    stage_digits(stage, w.B, p, lane, v[p], s_e[warp][p]);
+                }
+                __syncwarp();
+                uint4 *dst = reinterpret_cast<uint4 *>(dig + si.doff + (int64_t)c * w.B * kSliceTile);
+                const int n = min(2, nt - c) * w.B * (kSliceTile / 16);
+                for (int q = lane; q < n; q += 32) dst[q] = reinterpret_cast<uint4 *>(stage)[q];
+                __syncwarp();
+            }
         }
     }
 }
@@ -357,10 +432,158 @@ __device__ __forceinline__ bool slice_pass(const ProdArgs &a, const SliceArgs &q
     return true;
 }
 
-// One warp per work item (up to 16 output rows); KWIDE: k > 8, passes of 16
-// columns with a last one of 8 where that is enough.
-template <bool TRANS, bool KWIDE>
-__global__ void __launch_bounds__(128, KWIDE ? 3 : 4) slice_product_kernel(ProdArgs a, SliceArgs q) {
+// Products of KC <= kSliceThin columns: the digits of X, not its columns, are the
+// N side (8 of them a tile, 7 used, one tile a column), so an MMA forms digit i of
+// the values times all digits of a column at once: 7 KC MMAs a step instead of 35.
+// Every digit pair has an accumulator of its own, so nothing is dropped and the
+// sums over up to kSliceKMax columns are exact without carries. X is [rows, KC].
+// Bound by reading the value tiles (7 bytes an entry) and cutting them into f16
+// pairs. 50k atoms, k = 1 / 2 / 3: 0.32 / 0.43 / 0.56 ms, multiply-adds 0.37 / 0.73 / 1.26.
+template <bool TRANS, int KC, int NR>
+__device__ __forceinline__ bool slice_thin(const ProdArgs &a, const SliceArgs &q, const WorkItem &w,
+                                           const unsigned char *vsrc, int nsteps, const uint32_t *cmax,
+                                           unsigned char *ring, const int32_t *s_x, int lane, double &dot) {
+    constexpr int S = kSliceStages, kStage = 16 * kSliceTile;
+    const int g = lane >> 2, t4 = lane & 3;
+    float acc[kSliceDigits][KC][4], low[KC][4];
+#pragma unroll
+    for (int n = 0; n < KC; ++n)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            low[n][j] = 0.f;
+#pragma unroll
+            for (int i = 0; i < kSliceDigits; ++i) acc[i][n][j] = 0.f;
+        }
+    if (nsteps > 0) {
+        const int tile = w.B * kSliceTile;
+        constexpr int kChunks = (16 * kSliceTile / 16 + 31) / 32;
+        bool mine[kChunks];
+#pragma unroll
+        for (int u = 0; u < kChunks; ++u) mine[u] = 16 * (lane + 32 * u) < tile;
+        const unsigned char *src = vsrc + 16 * lane;
+        auto issue = [&](int s) {
+            const bool in = s < nsteps;
+            unsigned char *dst = ring + (s % S) * kStage + 16 * lane;
+#pragma unroll
+            for (int u = 0; u < kChunks; ++u)
+                if (in && mine[u]) cp_async16(dst + 512 * u, src + 512 * u);
+            src += tile;
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        // digit g of the lane's four virtual columns: byte 6 - g (the eighth digit is zero)
+        const uint8_t *xd = reinterpret_cast<const uint8_t *>(q.xdig) + (g < 7 ? 6 - g : 0);
+        uint32_t x[KC][4];
+        auto load_x = [&](int s) {
+            const int4 xi = *reinterpret_cast<const int4 *>(s_x + 16 * s + 4 * t4);
+            const int row[4] = {xi.x, xi.y, xi.z, xi.w};
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int n = 0; n < KC; ++n) x[n][r] = __ldg(xd + ((int64_t)row[r] * KC + n) * 8);
+        };
+        load_x(0);
+#pragma unroll
+        for (int s = 0; s < S - 1; ++s) issue(s);
+        const int digit = w.B * 16;
+        for (int s = 0; s < nsteps; ++s) {
+            asm volatile("cp.async.wait_group %0;" ::"n"(S - 2) : "memory");
+            __syncwarp();
+            issue(s + S - 1);
+            uint32_t b[KC][2];
+#pragma unroll
+            for (int n = 0; n < KC; ++n)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    // 0x6400 | byte is 1024 + byte in f16; less 1152
+                    uint32_t p = (x[n][2 * h] + (x[n][2 * h + 1] << 16)) | 0x64006400u;
+                    asm("sub.f16x2 %0, %0, %1;" : "+r"(p) : "r"(0x64806480u));
+                    b[n][h] = g < 7 ? p : 0u;
+                }
+            load_x(s + 1);
+            const unsigned char *st = ring + (s % S) * kStage + g * 16 + t4 * 4;
+#pragma unroll
+            for (int i = 0; i < kSliceDigits; ++i, st += digit) {
+                uint32_t v[NR][2];
+#pragma unroll
+                for (int n = 0; n < NR; ++n) {
+                    const uint32_t word = *reinterpret_cast<const uint32_t *>(st + 128 * n);
+                    v[n][0] = slice_half2(word, 0x4140);
+                    v[n][1] = slice_half2(word, 0x4342);
+                }
+                const uint32_t rows[4] = {v[0][0], v[NR - 1][0], v[0][1], v[NR - 1][1]};
+#pragma unroll
+                for (int n = 0; n < KC; ++n) mma_f16(acc[i][n], rows, b[n][0], b[n][1]);
+                if (i == 0) {   // magnitudes of the leading digits (column 0 of the tile)
+                    constexpr uint32_t kAbs = 0x7fff7fffu;
+                    const uint32_t r[4] = {rows[0] & kAbs, rows[1] & kAbs, rows[2] & kAbs, rows[3] & kAbs};
+#pragma unroll
+                    for (int n = 0; n < KC; ++n) mma_f16(low[n], r, b[n][0] & kAbs, b[n][1] & kAbs);
+                }
+            }
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncwarp();
+    }
+    // accumulator 2 h + e: row g + 8 h, digit 2 t4 + e of X. Lanes t4 = 0 hold digit 0 and write.
+    int er[2], ec[KC];
+    bool ok = true;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) er[h] = g + 8 * h < w.B ? q.rexp[w.yrow + g + 8 * h] : 0;
+#pragma unroll
+    for (int n = 0; n < KC; ++n) {
+        const uint32_t M = cmax[n];
+        ec[n] = M ? slice_exp(M) : 0;
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            ok &= er[h] >= 0 && (er[h] == 0 || ec[n] == 0 || t4 != 0 || low[n][2 * h] >= kSliceGuard);
+    }
+    if (!__all_sync(0xffffffffu, ok)) return false;
+#pragma unroll
+    for (int h = 0; h < NR; ++h) {
+        const int r = g + 8 * h;
+#pragma unroll
+        for (int n = 0; n < KC; ++n) {
+            // sum over the digits of the values, in units of their last: hi * 2^24 + lo, for the
+            // lane's two digits of X together (hi below 2^57, lo below 2^49)
+            long long hi = 0, lo = 0;
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                long long p = __float2int_rn(acc[0][n][2 * h + e]), t = __float2int_rn(acc[4][n][2 * h + e]);
+#pragma unroll
+                for (int i = 1; i < 4; ++i) p = p * 256 + __float2int_rn(acc[i][n][2 * h + e]);
+#pragma unroll
+                for (int i = 5; i < 7; ++i) t = t * 256 + __float2int_rn(acc[i][n][2 * h + e]);
+                hi = hi * 256 + p;
+                lo = lo * 256 + t;
+            }
+            // a pair of digits weighs 2^-16 of the one before
+            double d = fma((double)hi, 16777216.0, (double)lo);
+            d *= t4 == 0 ? 1.0 : t4 == 1 ? 0x1p-16 : t4 == 2 ? 0x1p-32 : 0x1p-48;
+            d += __shfl_xor_sync(0xffffffffu, d, 2);
+            d += __shfl_xor_sync(0xffffffffu, d, 1);
+            if (t4 == 0 && r < w.B) {
+                // digits 0 and 1 of X in units of 256^5: the same exponent as the level sums of a pass
+                const uint64_t bits = (uint64_t)__double_as_longlong(d);
+                const int e2 = er[h] + ec[n] - 2114 + q.alpha_exp;
+                double o = (bits << 1) == 0 ? 0.0 : __longlong_as_double((long long)(bits + ((uint64_t)(int64_t)e2 << 52)));
+                const int64_t row = w.yrow + r;
+                double *y = static_cast<double *>(a.Y) + row * a.ldy + n;
+                if (!q.alpha_pow2) o *= a.alpha;
+                if (a.beta_nz) o += a.beta * *y;
+                if (a.gamma_nz) o += a.gamma * static_cast<const double *>(a.Z)[row * a.ldz + n];
+                *y = o;
+                if (a.item_partials) dot += static_cast<const double *>(a.R)[row * a.ldr + n] * o;
+            }
+        }
+    }
+    return true;
+}
+
+// One warp per work item (up to 16 output rows). FORM 0: k > 8, passes of 16
+// columns with a last one of 8 where that is enough; 8: one pass of up to 8
+// columns; 1 .. kSliceThin: that many columns.
+template <bool TRANS, int FORM>
+__global__ void __launch_bounds__(128, FORM == 0 || FORM == 3 ? 3 : FORM == 1 ? 5 : 4) slice_product_kernel(ProdArgs a, SliceArgs q) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int kRing = kSliceStages * 16 * kSliceTile;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -386,7 +609,7 @@ __global__ void __launch_bounds__(128, KWIDE ? 3 : 4) slice_product_kernel(ProdA
             // a small structure, or one with a column outside the sliced range or mostly tiny, is not sliced
             last_strct = si.strct;
             const uint32_t most = (uint32_t)q.struct_rows[si.strct] >> 2;
-            bool p = q.struct_nnz[si.strct] * a.k < kSliceMinWork;
+            bool p = q.struct_nnz[si.strct] * a.k < slice_min_work(a.k);
             for (int c = lane; c < (int)a.k; c += 32)
                 p |= !slice_exp_ok(cmax[c]) || q.ccnt[(int64_t)si.strct * q.ldp + c] > most;
             last_plain = __any_sync(0xffffffffu, p);
@@ -411,14 +634,21 @@ __global__ void __launch_bounds__(128, KWIDE ? 3 : 4) slice_product_kernel(ProdA
         }
         if (!plain) {
             bool ok = true;
-            if (KWIDE)
+            if constexpr (FORM == 0)
                 for (; ok && n0 + 8 < a.k; n0 += ok ? 16 : 0)
                     ok = w.B <= 8 ? slice_pass<TRANS, true, 1>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot)
                                   : slice_pass<TRANS, true, 2>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot);
-            if (ok && n0 < a.k) {
-                ok = w.B <= 8 ? slice_pass<TRANS, false, 1>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot)
-                              : slice_pass<TRANS, false, 2>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot);
-                n0 += ok ? 8 : 0;
+            if constexpr (FORM == 0 || FORM == 8) {
+                if (ok && n0 < a.k) {
+                    ok = w.B <= 8
+                             ? slice_pass<TRANS, false, 1>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot)
+                             : slice_pass<TRANS, false, 2>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot);
+                    n0 += ok ? 8 : 0;
+                }
+            } else {
+                ok = w.B <= 8 ? slice_thin<TRANS, FORM, 1>(a, q, w, vsrc, nsteps, cmax, ring, s_x, lane, dot)
+                              : slice_thin<TRANS, FORM, 2>(a, q, w, vsrc, nsteps, cmax, ring, s_x, lane, dot);
+                n0 = ok ? FORM : 0;
             }
         }
         if (n0 < a.k) {
@@ -441,32 +671,40 @@ __global__ void __launch_bounds__(128, KWIDE ? 3 : 4) slice_product_kernel(ProdA
 
 size_t slice_smem_bytes() { return 4 * ((size_t)kSliceStages * 16 * kSliceTile + kSliceList); }
 
+int slice_ldp(int64_t k) { return k <= kSliceThin ? (int)k : (int)((k + 7) / 8 * 8); }
+
+using SliceKernel = void (*)(ProdArgs, SliceArgs);
+template <bool TRANS>
+static SliceKernel slice_kernel(int64_t k) {
+    switch (k) {
+        case 1: return slice_product_kernel<TRANS, 1>;
+        case 2: return slice_product_kernel<TRANS, 2>;
+        case 3: return slice_product_kernel<TRANS, 3>;
+        default: return k <= 8 ? slice_product_kernel<TRANS, 8> : slice_product_kernel<TRANS, 0>;
+    }
+}
+
 const void *slice_kernel_ptr(bool trans, int64_t k) {
-    if (trans) return k <= 8 ? (const void *)slice_product_kernel<true, false> : (const void *)slice_product_kernel<true, true>;
-    return k <= 8 ? (const void *)slice_product_kernel<false, false> : (const void *)slice_product_kernel<false, true>;
+    return (const void *)(trans ? slice_kernel<true>(k) : slice_kernel<false>(k));
 }
 
 cudaError_t launch_slice_product(bool trans, const ProdArgs &a, const SliceArgs &q, cudaStream_t s) {
     const size_t smem = slice_smem_bytes();
-    const void *kern = slice_kernel_ptr(trans, a.k);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const SliceKernel kern = trans ? slice_kernel<true>(a.k) : slice_kernel<false>(a.k);
+    cudaError_t e = cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    if (trans) {
-        if (a.k <= 8) slice_product_kernel<true, false><<<a.grid, 128, smem, s>>>(a, q);
-        else slice_product_kernel<true, true><<<a.grid, 128, smem, s>>>(a, q);
-    } else {
-        if (a.k <= 8) slice_product_kernel<false, false><<<a.grid, 128, smem, s>>>(a, q);
-        else slice_product_kernel<false, true><<<a.grid, 128, smem, s>>>(a, q);
-    }
+    kern<<<a.grid, 128, smem, s>>>(a, q);
     return cudaGetLastError();
 }
 
 cudaError_t launch_slice_panel(const SliceChunk *chunks, int64_t n_chunks, const double *X, int64_t ldx, int k, int ldp,
                                uint32_t *cmax, uint32_t *ccnt, uint64_t *out, cudaStream_t s) {
     if (n_chunks == 0) return cudaSuccess;
-    const int grid = (int)(n_chunks < 65535 ? n_chunks : 65535);
-    slice_colmax_kernel<<<grid, 256, 0, s>>>(chunks, n_chunks, X, ldx, k, ldp, cmax);
-    slice_panel_kernel<<<grid, 256, 0, s>>>(chunks, n_chunks, X, ldx, k, ldp, cmax, ccnt, out);
+    // about 2048 elements a CTA: several chunks of narrow panels
+    const int per = k >= 8 ? 1 : 8 / k;
+    const unsigned grid = (unsigned)((n_chunks + per - 1) / per);
+    slice_colmax_kernel<<<grid, 256, 0, s>>>(chunks, n_chunks, per, X, ldx, k, ldp, cmax);
+    slice_panel_kernel<<<grid, 256, 0, s>>>(chunks, n_chunks, per, X, ldx, k, ldp, cmax, ccnt, out);
     return cudaGetLastError();
 }
 

@@ -241,3 +241,30 @@ def test_sliced_sddmm_against_oracle(k):
     assert np.array_equal(np.isnan(got), np.isnan(ref)) and np.array_equal(np.isinf(got), np.isinf(ref))
     assert any("slice_sddmm" in n for n in _kernels(lambda: H.sddmm(torch.from_numpy(A0).cuda()[:, :k],
                                                                     torch.from_numpy(B0).cuda()[:, :k])))
+
+
+def test_thin_sliced_products():
+    """One to three columns (the digits of X on the N side), forward and adjoint: every
+    row height of a random pattern at three columns, the sizes from which one and two
+    columns are sliced on a nanoparticle, outputs that are not resolved, an exact sum."""
+    pat = syn.random_pattern(270, 265, (1, 2, 4, 9, 13, 16, 33), 0.22, 3, empty_rows=2, unsorted=True)
+    assert 3 * pat.nnz >= 1 << 22
+    vals = syn.random_values(pat, 3)
+    H = _handle(pat, vals)
+    rng = np.random.default_rng(3)
+    X = rng.standard_normal((pat.n_cols, 3))
+    _check(H, pat, vals, X, alpha=-0.3, beta=2.0, Y0=rng.standard_normal((pat.n_rows, 3)))
+    _check(H, pat, vals, rng.standard_normal((pat.n_rows, 3)), transpose=True)
+    assert any("slice_product" in n for n in _kernels(lambda: H.spmm(torch.from_numpy(X).cuda())))
+    X[:, 1] *= np.exp(-np.arange(pat.n_cols) / 50.0)
+    X[9, 0] = np.inf
+    with np.errstate(invalid="ignore"):
+        _check(H, pat, vals, X)
+    w = syn.zincblende(21_000)
+    assert w.pattern.nnz >= 1 << 26
+    H = _handle(w.pattern, w.values)
+    for k in (1, 2):
+        X = rng.standard_normal((w.pattern.n_cols, k))
+        _check(H, w.pattern, w.values, X)
+        _check(H, w.pattern, w.values, X, transpose=True)
+        assert any("slice_product" in n for n in _kernels(lambda: H.spmm(torch.from_numpy(X).cuda())))
