@@ -183,10 +183,7 @@ struct vbcsr_matrix {
     double *ks_shift = nullptr;      // s_e = R [+ tau_j - tau_i] of every sorted edge (3 doubles)
     int64_t *ks_voff = nullptr;      // offset of every sorted edge's real block in ks_vals
     double *ks_vals = nullptr;       // the image blocks, row-major
-    int64_t *ks_uoff = nullptr;      // packed offset of every union block
-    int32_t *ks_ubn = nullptr;       // entries of every union block
     double2 *ks_phase = nullptr;     // phase of every sorted edge at the current k
-    double2 *ks_stage = nullptr;     // packed complex values at the current k
 
     ~vbcsr_matrix() {
         int cur = 0;
@@ -321,7 +318,8 @@ static void sort_by_cost(std::vector<WorkItem> &items) {
 // out_start / in_start: first scalar output / input row of every structure.
 static int plan_slices(vbcsr_matrix *A, SlicePlan *p, const std::vector<WorkItem> &items,
                        const std::vector<int64_t> &out_start, const std::vector<int64_t> &in_start, cudaStream_t s) {
-    if (A->dtype != VBCSR_F64 || A->backend == VBCSR_BACKEND_CSR || items.empty() || A->nblk == 0) return VBCSR_OK;
+    if (A->dtype == VBCSR_F32 || A->backend == VBCSR_BACKEND_CSR || items.empty() || A->nblk == 0) return VBCSR_OK;
+    const int cw = A->dtype == VBCSR_C128 ? 2 : 1;   // real virtual columns and X rows a complex one
     std::vector<SliceItem> si(items.size());
     std::vector<int64_t> nnz(out_start.size() - 1, 0);
     int64_t pos = 0;
@@ -332,13 +330,13 @@ static int plan_slices(vbcsr_matrix *A, SlicePlan *p, const std::vector<WorkItem
         si[t].pad = 0;
         si[t].strct = (int32_t)(std::upper_bound(out_start.begin(), out_start.end() - 1, w.yrow) - out_start.begin() - 1);
         all += (double)w.B * w.K;
-        nnz[si[t].strct] += (int64_t)w.B * w.K;
-        if (w.K > kSliceKMax) {
+        nnz[si[t].strct] += (int64_t)w.B * w.K * cw;
+        if (cw * w.K > kSliceKMax) {
             wide += (double)w.B * w.K;
             continue;
         }
         si[t].doff = pos;
-        pos += (int64_t)((w.K + 15) / 16) * w.B * (kSliceDigits * 16);
+        pos += (int64_t)((cw * w.K + 15) / 16) * w.B * (kSliceDigits * 16);
     }
     // the wide items run multiply-adds in a kernel with fewer resident warps than the
     // multiply-add kernels have: not for an operator with much of its work there
@@ -783,7 +781,7 @@ extern "C" int vbcsr_create_kspace(vbcsr_t **out, int64_t n_atoms, const int32_t
             return edge_i[x] != edge_i[y] ? edge_i[x] < edge_i[y] : edge_j[x] < edge_j[y];
         });
         std::vector<int64_t> rowptr(n_atoms + 1, 0), ks_ptr(1, 0), ks_voff(n_edges);
-        std::vector<int32_t> cols, ubn;
+        std::vector<int32_t> cols;
         std::vector<double> shift(3 * (size_t)n_edges);
         for (int64_t t = 0; t < n_edges; ++t) {
             const int64_t e = order[t];
@@ -791,7 +789,6 @@ extern "C" int vbcsr_create_kspace(vbcsr_t **out, int64_t n_atoms, const int32_t
             const bool fresh = t == 0 || edge_i[order[t - 1]] != i || edge_j[order[t - 1]] != j;
             if (fresh) {
                 cols.push_back(j);
-                ubn.push_back(bsize[i] * bsize[j]);
                 rowptr[i + 1] += 1;
                 if (t > 0) ks_ptr.push_back(t);
             }
@@ -801,7 +798,6 @@ extern "C" int vbcsr_create_kspace(vbcsr_t **out, int64_t n_atoms, const int32_t
         }
         if (n_edges > 0) ks_ptr.push_back(n_edges);
         for (int64_t a = 0; a < n_atoms; ++a) rowptr[a + 1] += rowptr[a];
-        const int64_t nblk = (int64_t)cols.size();
         int rc = create_common(out, n_atoms, n_atoms, bsize, bsize, rowptr.data(), cols.data(), nullptr, VBCSR_C128,
                                0, stream, 1, nullptr, nullptr, true);
         if (rc) return rc;
@@ -813,16 +809,12 @@ extern "C" int vbcsr_create_kspace(vbcsr_t **out, int64_t n_atoms, const int32_t
         };
         A->kspace = true;
         A->ks_edges = n_edges;
-        std::vector<int64_t> uo(A->uoff.begin(), A->uoff.begin() + nblk);
         std::vector<double> vals(edge_values, edge_values + evoff[n_edges]);
         cudaError_t e = upload(A, &A->ks_ptr, ks_ptr, s);
         if (e == cudaSuccess) e = upload(A, &A->ks_shift, shift, s);
         if (e == cudaSuccess) e = upload(A, &A->ks_voff, ks_voff, s);
         if (e == cudaSuccess) e = upload(A, &A->ks_vals, vals, s);
-        if (e == cudaSuccess) e = upload(A, &A->ks_uoff, uo, s);
-        if (e == cudaSuccess) e = upload(A, &A->ks_ubn, ubn, s);
         if (e == cudaSuccess) e = A->alloc(&A->ks_phase, (size_t)n_edges);
-        if (e == cudaSuccess) e = A->alloc(&A->ks_stage, (size_t)A->nnz);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return bail(cuda_fail(e, "upload the lattice images"));
     } catch (const std::bad_alloc &) {
@@ -835,17 +827,16 @@ extern "C" int vbcsr_create_kspace(vbcsr_t **out, int64_t n_atoms, const int32_t
     return VBCSR_OK;
 }
 
+static int slices_changed(vbcsr_t *A, cudaStream_t s);
+
 extern "C" int vbcsr_set_kpoint(vbcsr_t *A, const double *kfrac, void *stream) {
     if (!A || !kfrac) return fail(VBCSR_ERR_INVALID_ARG, "NULL argument");
     if (!A->kspace) return fail(VBCSR_ERR_INVALID_ARG, "not a handle made by vbcsr_create_kspace");
     cudaStream_t s = (cudaStream_t)stream;
-    CUDA_TRY(launch_ksample(A->nblk, A->ks_edges, A->ks_ptr, A->ks_shift, A->ks_voff, A->ks_vals, A->ks_uoff,
-                            A->ks_ubn, kfrac, A->ks_phase, A->ks_stage, s),
+    CUDA_TRY(launch_ksample(A->nblk, A->ks_edges, A->ks_ptr, A->ks_shift, A->ks_voff, A->ks_vals, A->fl_pbase, A->fl_kp,
+                            A->fl_bi, A->fl_w, kfrac, A->ks_phase, (double2 *)A->panel, s),
              "k-space sampling");
-    CUDA_TRY(launch_permute_values((int)A->esize, true, A->nblk, A->fl_uoff, A->fl_pbase, A->fl_kp, A->fl_bi,
-                                   A->fl_w, A->ks_stage, A->panel, s),
-             "scatter values");
-    return VBCSR_OK;
+    return slices_changed(A, s);
 }
 
 extern "C" int vbcsr_destroy(vbcsr_t *A) {
@@ -913,7 +904,7 @@ static int grow(vbcsr_t *A, T **buf, size_t *have, size_t need, cudaStream_t s, 
 static int refresh_slices(vbcsr_t *A, bool trans, cudaStream_t s) {
     SlicePlan &p = A->slice[trans];
     const AdjList tl = {A->tl_pbase, A->tl_kp, A->tl_bi, A->tl_xrow, A->tl_vcol};
-    CUDA_TRY(launch_slice_values(trans, trans ? A->adj_lpt : A->fwd_lpt, p.items,
+    CUDA_TRY(launch_slice_values(A->dtype == VBCSR_C128, trans, trans ? A->adj_lpt : A->fwd_lpt, p.items,
                                  trans ? A->n_adj_items : A->n_fwd_items, tl, (const double *)A->panel, p.vdig, p.rexp,
                                  s),
              "slice values");
@@ -954,12 +945,16 @@ static bool slice_applies(const vbcsr_t *A, bool trans, int64_t k) {
     return p.applies && !p.untracked && k <= (1 << 20) && p.max_nnz * k >= slice_min_work(k) && !A->debug_checks;
 }
 
+// k counts real columns here and below (two a column of a complex operator)
+static size_t slice_x_elems(const vbcsr_t *A, bool trans, int64_t k) {
+    return (size_t)((trans ? A->n_rows : A->n_cols) * slice_ldp(k)) * (A->dtype == VBCSR_C128 ? 2 : 1);
+}
+
 static size_t slice_tab_elems(const vbcsr_t *A, int64_t ldp) { return 4 + 2 * (size_t)A->n_structs * (size_t)ldp; }
 
 static bool slice_buffers_ready(const vbcsr_t *A, bool trans, int64_t k) {
-    const int64_t ldp = slice_ldp(k), xrows = trans ? A->n_rows : A->n_cols;
-    return A->slice[trans].vdig && A->xdig_elems >= (size_t)(xrows * ldp) &&
-           A->stab_elems >= slice_tab_elems(A, ldp);
+    return A->slice[trans].vdig && A->xdig_elems >= slice_x_elems(A, trans, k) &&
+           A->stab_elems >= slice_tab_elems(A, slice_ldp(k));
 }
 
 // Builds what a sliced product needs and is missing (*ready = true when it can
@@ -1196,7 +1191,6 @@ static int slice_prepare(vbcsr_t *A, bool trans, int64_t k, bool may_alloc, cuda
         return VBCSR_OK;
     }
     if (!may_alloc || p.no_room || cap) return VBCSR_OK;
-    const int64_t ldp = slice_ldp(k), xrows = trans ? A->n_rows : A->n_cols;
     int rc = VBCSR_OK;
     if (!p.vdig) {
         cudaError_t e = p.rexp ? cudaSuccess : A->alloc(&p.rexp, (size_t)(trans ? A->n_cols : A->n_rows));
@@ -1209,8 +1203,8 @@ static int slice_prepare(vbcsr_t *A, bool trans, int64_t k, bool may_alloc, cuda
         p.stale = rc != VBCSR_OK;
     }
     if (!rc)
-        rc = grow(A, &A->xdig, &A->xdig_elems, (size_t)(xrows * ldp), s, "alloc fixed-point X");
-    if (!rc) rc = grow(A, &A->stab, &A->stab_elems, slice_tab_elems(A, ldp), s, "alloc column maxima");
+        rc = grow(A, &A->xdig, &A->xdig_elems, slice_x_elems(A, trans, k), s, "alloc fixed-point X");
+    if (!rc) rc = grow(A, &A->stab, &A->stab_elems, slice_tab_elems(A, slice_ldp(k)), s, "alloc column maxima");
     if (rc == VBCSR_ERR_NO_MEMORY) {
         p.no_room = true;
         return VBCSR_OK;
@@ -1269,9 +1263,10 @@ static int run_product(vbcsr_t *A, bool trans, int64_t k, double alpha, const vo
         int rc = refresh_panelbp(A, s);
         if (rc) return rc;
     }
-    bool sliced = f64 && mode == VBCSR_PREC_NATIVE && alpha != 0.0 && slice_applies(A, trans, k);
+    const int64_t kr = cplx ? 2 * k : k;   // real columns
+    bool sliced = (f64 || cplx) && mode == VBCSR_PREC_NATIVE && alpha != 0.0 && slice_applies(A, trans, kr);
     if (sliced) {
-        int rc = slice_prepare(A, trans, k, may_alloc, s, &sliced);
+        int rc = slice_prepare(A, trans, kr, may_alloc, s, &sliced);
         if (rc) return rc;
     }
     const bool piped = mp.pipe || mp.pipe_tf;
@@ -1406,7 +1401,7 @@ static int run_product(vbcsr_t *A, bool trans, int64_t k, double alpha, const vo
         }
         cudaError_t e;
         if (sliced)
-            e = launch_slice_product(trans, a, sa, s);
+            e = cplx ? launch_slice_product_c128(trans, a, sa, s) : launch_slice_product(trans, a, sa, s);
         else if (fpipe)
             e = launch_fma32_pipe(f64, a, s);
         else if (mode == VBCSR_PREC_NATIVE)
@@ -1440,10 +1435,18 @@ static int run_product(vbcsr_t *A, bool trans, int64_t k, double alpha, const vo
         // FP64 on the tensor cores (sliced.cuh): the digits of X, then one launch over every
         // item; the CUDA-core schedule and tiles do not apply
         const SlicePlan &p = A->slice[trans];
-        const int xld = slice_ldp(k);
+        const int xld = slice_ldp(kr);
         uint32_t *cmax = A->stab + 4, *ccnt = cmax + (size_t)A->n_structs * xld;
         CUDA_TRY(cudaMemsetAsync(A->stab, 0, slice_tab_elems(A, xld) * sizeof(uint32_t), s), "reset column maxima");
-        CUDA_TRY(launch_slice_panel(p.chunks, p.n_chunks, (const double *)X, ldx, (int)k, xld, cmax, ccnt, A->xdig, s),
+        if (cplx) {
+            a.k = kr;
+            a.ldx = ldx * 2;
+            a.ldy *= 2;
+            a.ldz *= 2;
+            a.ldr *= 2;
+        }
+        CUDA_TRY(launch_slice_panel(cplx, p.chunks, p.n_chunks, (const double *)X, a.ldx, (int)kr, xld, cmax, ccnt,
+                                    A->xdig, s),
                  "slice X");
         sa.sitems = p.items;
         sa.vdig = p.vdig;
@@ -1459,7 +1462,8 @@ static int run_product(vbcsr_t *A, bool trans, int64_t k, double alpha, const vo
         sa.alpha_exp = sa.alpha_pow2 ? ae - 1 : 0;
         a.queue = reinterpret_cast<long long *>(A->stab);
         per_item_dot = true;
-        rc = launch(0, trans ? A->adj_lpt : A->fwd_lpt, n_all, 4, slice_kernel_ptr(trans, k), slice_smem_bytes());
+        rc = launch(0, trans ? A->adj_lpt : A->fwd_lpt, n_all, 4,
+                    cplx ? slice_c128_kernel_ptr(trans, kr) : slice_kernel_ptr(trans, kr), slice_smem_bytes());
     } else if (!fma && !split) {
         // tensor-core kernel: the row count is a runtime mask, one launch serves every item
         const bool staged = !trans && (A->schedule & VBCSR_SCHED_MMA_STAGED);

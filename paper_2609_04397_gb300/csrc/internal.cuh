@@ -182,11 +182,14 @@ struct SliceArgs {
     int alpha_pow2, alpha_exp;    // alpha = 2^alpha_exp: goes into the result's exponent
 };
 cudaError_t launch_slice_product(bool trans, const ProdArgs &a, const SliceArgs &q, cudaStream_t s);
-cudaError_t launch_slice_panel(const SliceChunk *chunks, int64_t n_chunks, const double *X, int64_t ldx, int k, int ldp,
-                               uint32_t *cmax, uint32_t *ccnt, uint64_t *out, cudaStream_t s);
-cudaError_t launch_slice_values(bool trans, const WorkItem *items, const SliceItem *sitems, int64_t n_items,
+// complex operators: k, ldx and the other leading dimensions count real columns (two a complex one)
+cudaError_t launch_slice_product_c128(bool trans, const ProdArgs &a, const SliceArgs &q, cudaStream_t s);
+cudaError_t launch_slice_panel(bool cplx, const SliceChunk *chunks, int64_t n_chunks, const double *X, int64_t ldx, int k,
+                               int ldp, uint32_t *cmax, uint32_t *ccnt, uint64_t *out, cudaStream_t s);
+cudaError_t launch_slice_values(bool cplx, bool trans, const WorkItem *items, const SliceItem *sitems, int64_t n_items,
                                 const AdjList &tl, const double *panel, uint8_t *dig, int32_t *rexp, cudaStream_t s);
 const void *slice_kernel_ptr(bool trans, int64_t k);
+const void *slice_c128_kernel_ptr(bool trans, int64_t k);
 size_t slice_smem_bytes();
 constexpr int kSliceThin = 3;         // widest product with the digits of X on the N side
 int slice_ldp(int64_t k);             // columns of the fixed-point X
@@ -300,10 +303,11 @@ cudaError_t launch_sddmm_sliced(const SddmmArgs &a, int64_t rows_a, int64_t rows
                                 int32_t *eb, cudaStream_t s);
 
 // scatter (to_panel = true) or gather packed-order values <-> panels
-// reciprocal-space sampling (Eq. 4) of a k-space handle into packed complex values
+// reciprocal-space sampling (Eq. 4) of a k-space handle into its pages (blocks in plan order)
 cudaError_t launch_ksample(int64_t nblk, int64_t n_edges, const int64_t *ks_ptr, const double *ks_shift,
-                           const int64_t *ks_voff, const double *ks_vals, const int64_t *uoff, const int32_t *ub_n,
-                           const double *kfrac, double2 *phase, double2 *out, cudaStream_t s);
+                           const int64_t *ks_voff, const double *ks_vals, const int64_t *pbase, const int32_t *kp,
+                           const int32_t *bi, const int32_t *bj, const double *kfrac, double2 *phase, double2 *panel,
+                           cudaStream_t s);
 // complex FP64 products (VBCSR_C128)
 cudaError_t launch_fma_c128(int B, bool trans, const ProdArgs &a, cudaStream_t s);
 const void *fma_c128_kernel(bool trans, bool persistent, int B);

@@ -212,8 +212,8 @@ cudaError_t launch_permute_values(int esize, bool to_panel, int64_t nblk, const 
 // tau_i] (one FP64 sincospi per edge: GB300's FP64 pipe is narrow, so it is not
 // repeated per entry); then block u of the union pattern sums its edges
 // ks_ptr[u] .. ks_ptr[u+1] (real b_i x b_j image blocks at ks_voff) times their
-// phases, written in packed order at uoff[u]: one warp per block, lanes over
-// its entries.
+// phases, written straight to the pages (the pattern is created with sorted
+// columns, so blocks lie in plan order): one warp per block, lanes over its entries.
 
 __global__ void kphase_kernel(int64_t n_edges, const double *ks_shift, double k0, double k1, double k2,
                               double2 *phase) {
@@ -225,13 +225,14 @@ __global__ void kphase_kernel(int64_t n_edges, const double *ks_shift, double k0
     }
 }
 
-__global__ void ksample_kernel(int64_t nblk, const int64_t *ks_ptr, const double2 *phase, const int64_t *ks_voff,
-                               const double *ks_vals, const int64_t *uoff, const int32_t *ub_n, double2 *out,
+__global__ void ksample_kernel(int64_t nblk, const int64_t *ks_ptr, const double2 *__restrict__ phase,
+                               const int64_t *ks_voff, const double *__restrict__ ks_vals, const int64_t *pbase,
+                               const int32_t *kp, const int32_t *bi, const int32_t *bj, double2 *__restrict__ panel,
                                int warps) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int64_t u = (int64_t)blockIdx.x * warps + warp; u < nblk; u += (int64_t)gridDim.x * warps) {
-        const int n = ub_n[u];
-        const int64_t e0 = ks_ptr[u], e1 = ks_ptr[u + 1], o = uoff[u];
+        const int w = bj[u], n = bi[u] * w;
+        const int64_t e0 = ks_ptr[u], e1 = ks_ptr[u + 1], o = pbase[u], stride = kp[u];
         for (int q = lane; q < n; q += 32) {
             double re = 0.0, im = 0.0;
             for (int64_t e = e0; e < e1; ++e) {
@@ -240,14 +241,16 @@ __global__ void ksample_kernel(int64_t nblk, const int64_t *ks_ptr, const double
                 re = fma(v, ph.x, re);
                 im = fma(v, ph.y, im);
             }
-            out[o + q] = make_double2(re, im);
+            const int p = q / w;
+            panel[o + p * stride + (q - p * w)] = make_double2(re, im);
         }
     }
 }
 
 cudaError_t launch_ksample(int64_t nblk, int64_t n_edges, const int64_t *ks_ptr, const double *ks_shift,
-                           const int64_t *ks_voff, const double *ks_vals, const int64_t *uoff, const int32_t *ub_n,
-                           const double *kfrac, double2 *phase, double2 *out, cudaStream_t s) {
+                           const int64_t *ks_voff, const double *ks_vals, const int64_t *pbase, const int32_t *kp,
+                           const int32_t *bi, const int32_t *bj, const double *kfrac, double2 *phase, double2 *panel,
+                           cudaStream_t s) {
     if (n_edges > 0) {
         int64_t need = (n_edges + 255) / 256;
         kphase_kernel<<<(int)(need < 65536 ? need : 65536), 256, 0, s>>>(n_edges, ks_shift, kfrac[0], kfrac[1],
@@ -259,7 +262,7 @@ cudaError_t launch_ksample(int64_t nblk, int64_t n_edges, const int64_t *ks_ptr,
     const int warps = 8;
     int64_t need = (nblk + warps - 1) / warps;
     int grid = (int)(need < 65536 ? need : 65536);
-    ksample_kernel<<<grid, warps * 32, 0, s>>>(nblk, ks_ptr, phase, ks_voff, ks_vals, uoff, ub_n, out, warps);
+    ksample_kernel<<<grid, warps * 32, 0, s>>>(nblk, ks_ptr, phase, ks_voff, ks_vals, pbase, kp, bi, bj, panel, warps);
     return cudaGetLastError();
 }
 

@@ -268,3 +268,40 @@ def test_thin_sliced_products():
         _check(H, w.pattern, w.values, X)
         _check(H, w.pattern, w.values, X, transpose=True)
         assert any("slice_product" in n for n in _kernels(lambda: H.spmm(torch.from_numpy(X).cuda())))
+
+
+@pytest.mark.parametrize("k", [1, 3, 8, 13])
+def test_sliced_complex_products(k):
+    """A complex operator as two real virtual columns a value, forward and
+    conjugate-transpose, at two k-points (the tiles follow the values), with the
+    fused epilogue, and on a panel that is not resolved."""
+    from paper_2609_04397_gb300 import VBCSR
+    w = syn.zincblende_crystal(4)
+    H = VBCSR.from_images(w.bsize, w.edge_i, w.edge_j, w.edge_R, w.edge_values, device="cuda:0")
+    rb, cb, rp, ci = H.pattern
+    pat = BlockPattern(rb, cb, rp, ci)
+    rng = np.random.default_rng(k)
+
+    def crandn(n):
+        return rng.standard_normal((n, k)) + 1j * rng.standard_normal((n, k))
+
+    X, Y0, Z, R = (crandn(pat.n_rows) for _ in range(4))
+    local = X * np.exp(-np.arange(pat.n_rows) / 9.0)[:, None]
+    for kp in ([0.13, -0.27, 0.41], [0.3, 0.2, -0.1]):
+        H.set_kpoint(kp)
+        vals = H.get_values().cpu().numpy()
+        for P in (X, local):
+            mag = oracle.spmm(pat, np.abs(vals), np.abs(P))
+            Yd, dot = torch.from_numpy(Y0.copy()).cuda(), torch.zeros(1, dtype=torch.float64, device="cuda:0")
+            H.spmm_ex(torch.from_numpy(P).cuda(), 2.0, -1.0, Yd, gamma=0.5, Z=torch.from_numpy(Z).cuda(),
+                      R=torch.from_numpy(R).cuda(), dot_out=dot)
+            ref = oracle.spmm_complex(pat, vals, P, 2.0, -1.0, Y0) + 0.5 * Z
+            got = Yd.cpu().numpy()
+            # four real products a complex one
+            assert (np.abs(got - ref) <= 2 * TOL * (2 * mag + np.abs(Y0) + np.abs(Z))).all()
+            assert abs(dot.item() - np.sum((np.conj(R) * got).real)) <= 1e-12 * np.sum(np.abs(R * got))
+            ref = oracle.spmm_adjoint_complex(pat, vals, P, 1.0, 0.0, Y0)
+            got = H.spmm_adjoint(torch.from_numpy(P).cuda()).cpu().numpy()
+            assert (np.abs(got - ref) <= 2 * TOL * oracle.spmm_adjoint(pat, np.abs(vals), np.abs(P))).all()
+    if k > 1:   # from this width the operator has enough work
+        assert any("slice_product" in n for n in _kernels(lambda: H.spmm(torch.from_numpy(X).cuda())))
