@@ -1591,12 +1591,12 @@ static SddmmArgs sddmm_args(vbcsr_t *A) {
 }
 
 // FP64 pattern-sampled product: sliced when it has enough work (below, the extra
-// launch costs more than the multiply-adds), at k >= 2 (one column needs half a
-// clock an entry on the FP64 pipe, as much as the tensor-core tile) and up to the
-// widths whose level sums stay exact; else by multiply-adds, as on a stream that
+// launch costs more than the multiply-adds), at k >= 3 (one and two columns need
+// half a clock and a clock an entry on the FP64 pipe, about what the tensor-core
+// tile takes) and up to the widths whose level sums stay exact; else by multiply-adds, as on a stream that
 // is being captured before the buffers exist.
 static int run_sddmm_f64(vbcsr_t *A, const SddmmArgs &a, cudaStream_t s) {
-    bool sliced = a.k >= 2 && a.k <= kSliceKMax && a.alpha != 0.0 && A->nnz * a.k >= slice_min_work(3) && !A->debug_checks;
+    bool sliced = a.k >= 3 && a.k <= kSliceKMax && a.alpha != 0.0 && A->nnz * a.k >= slice_min_work(3) && !A->debug_checks;
     if (sliced) {
         const int64_t kp = (a.k + 15) / 16 * 16, rows = A->n_rows + A->n_cols;
         const size_t need = (size_t)(rows * kp + (rows + 1) / 2);

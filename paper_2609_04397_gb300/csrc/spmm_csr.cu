@@ -26,6 +26,10 @@ __global__ void __launch_bounds__(256) csr_kernel(ProdArgs a) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int sub = lane / L, lr = lane % L;
     constexpr int RPW = 32 / L;   // rows per warp
+    // 16-byte pieces of an X row's tile (0: the tile is no multiple of 16 bytes), usable
+    // when every row of X starts on a 16-byte boundary
+    constexpr int kVec = CW * sizeof(TXI) % 16 == 0 ? CW * sizeof(TXI) / 16 : 0;
+    const bool vec = (reinterpret_cast<uintptr_t>(a.X) | (uintptr_t)(a.ldx * sizeof(TXI))) % 16 == 0;
     const TV *__restrict__ vals = static_cast<const TV *>(a.values);
     const TXI *__restrict__ X = static_cast<const TXI *>(a.X);
     TX *__restrict__ Y = static_cast<TX *>(a.Y);
@@ -49,7 +53,16 @@ __global__ void __launch_bounds__(256) csr_kernel(ProdArgs a) {
                 for (int e = lr; e < w.K; e += L) {
                     const TA v = TA(__ldg(vals + w.vbase + e));
                     const TXI *xp = X + (int64_t)__ldg(a.fl.xrow + w.lbegin + e) * a.ldx + c0;
-                    if (nc == CW) {
+                    if (kVec && vec && nc == CW) {
+                        // 16-byte loads: lanes gather unrelated rows, so every load instruction
+                        // costs a pass over 32 sectors whatever its width
+                        alignas(16) TXI x[CW];
+#pragma unroll
+                        for (int j = 0; j < kVec; ++j)
+                            reinterpret_cast<uint4 *>(x)[j] = __ldg(reinterpret_cast<const uint4 *>(xp) + j);
+#pragma unroll
+                        for (int j = 0; j < CW; ++j) acc[j] = fmat(v, TA(x[j]), acc[j]);
+                    } else if (nc == CW) {
 #pragma unroll
                         for (int j = 0; j < CW; ++j) acc[j] = fmat(v, TA(__ldg(xp + j)), acc[j]);
                     } else {
