@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(128, 4) mma_bf16_pipe_kernel(ProdArgs a) {
                             mma16816(acc[0], alo, bh[0], bh[1]);
                         } else {
 #pragma unroll
-                            for (int n = 0; n < NT; n += 2) {
+                            for (int n = 0; n + 1 < NT; n += 2) {
                                 const int bm = lane >> 3, br = (lane & 7) + 8 * (bm & 1), bc = n + (bm >> 1);
                                 uint32_t bh[4], bl[4];
                                 ldsm_x4_t(xs0 + x_off<NT>(br, bc), bh);
@@ -231,6 +231,15 @@ __global__ void __launch_bounds__(128, 4) mma_bf16_pipe_kernel(ProdArgs a) {
                                 mma16816(acc[n + 1], ahi, bh[2], bh[3]);
                                 mma16816(acc[n + 1], ahi, bl[2], bl[3]);
                                 mma16816(acc[n + 1], alo, bh[2], bh[3]);
+                            }
+                            if constexpr (NT % 2 == 1) {   // the last tile of an odd count
+                                const int br = lane & 15;
+                                uint32_t bh[2], bl[2];
+                                ldsm_x2_t(xs0 + x_off<NT>(br, NT - 1), bh);
+                                ldsm_x2_t(xs0 + St::kXPlane + x_off<NT>(br, NT - 1), bl);
+                                mma16816(acc[NT - 1], ahi, bh[0], bh[1]);
+                                mma16816(acc[NT - 1], ahi, bl[0], bl[1]);
+                                mma16816(acc[NT - 1], alo, bh[0], bh[1]);
                             }
                         }
                         issue(s + S - 1);
@@ -783,7 +792,10 @@ cudaError_t fpipe_launch(const ProdArgs &a, cudaStream_t s) {
 
 }  // namespace
 
-int pipe_nt(int64_t k) { return k <= 8 ? 1 : (k <= 16 ? 2 : 4); }
+// 8-column tiles of a pass. 17 to 24 columns take 3: the 4-tile pass computes 32 (tiles of
+// 3 need no swizzle: their X rows of 48 or 96 bytes already fall on distinct banks).
+static int pipe_nt(int64_t k) { return k <= 8 ? 1 : (k <= 16 ? 2 : (k <= 24 ? 3 : 4)); }
+static int fpipe_nt(int64_t k) { return k <= 8 ? 1 : (k <= 16 ? 2 : 4); }
 
 int64_t pipe_ldp(int64_t k) {
     const int64_t w = 8 * pipe_nt(k);
@@ -792,8 +804,8 @@ int64_t pipe_ldp(int64_t k) {
 
 size_t mma_pipe_smem_bytes(int mode, int64_t k, int warps) {
     const int nt = pipe_nt(k);
-    if (mode != kBF16X2) return nt == 1 ? tf_smem<1>(warps) : nt == 2 ? tf_smem<2>(warps) : tf_smem<4>(warps);
-    return nt == 1 ? pipe_smem<1>(warps) : nt == 2 ? pipe_smem<2>(warps) : pipe_smem<4>(warps);
+    if (mode != kBF16X2) return nt == 1 ? tf_smem<1>(warps) : nt == 2 ? tf_smem<2>(warps) : nt == 3 ? tf_smem<3>(warps) : tf_smem<4>(warps);
+    return nt == 1 ? pipe_smem<1>(warps) : nt == 2 ? pipe_smem<2>(warps) : nt == 3 ? pipe_smem<3>(warps) : pipe_smem<4>(warps);
 }
 
 const void *mma_pipe_kernel_ptr(int mode, int64_t k) {
@@ -801,33 +813,39 @@ const void *mma_pipe_kernel_ptr(int mode, int64_t k) {
     if (mode == kTF32)
         return nt == 1 ? (const void *)mma_tf32_pipe_kernel<1, kTF32>
                        : nt == 2 ? (const void *)mma_tf32_pipe_kernel<2, kTF32>
+                       : nt == 3 ? (const void *)mma_tf32_pipe_kernel<3, kTF32>
                                  : (const void *)mma_tf32_pipe_kernel<4, kTF32>;
     if (mode == kTF32X3)
         return nt == 1 ? (const void *)mma_tf32_pipe_kernel<1, kTF32X3>
                        : nt == 2 ? (const void *)mma_tf32_pipe_kernel<2, kTF32X3>
+                       : nt == 3 ? (const void *)mma_tf32_pipe_kernel<3, kTF32X3>
                                  : (const void *)mma_tf32_pipe_kernel<4, kTF32X3>;
     return nt == 1 ? (const void *)mma_bf16_pipe_kernel<1>
-                   : nt == 2 ? (const void *)mma_bf16_pipe_kernel<2> : (const void *)mma_bf16_pipe_kernel<4>;
+                   : nt == 2 ? (const void *)mma_bf16_pipe_kernel<2>
+                   : nt == 3 ? (const void *)mma_bf16_pipe_kernel<3> : (const void *)mma_bf16_pipe_kernel<4>;
 }
 
 cudaError_t launch_mma_pipe(int mode, const ProdArgs &a, cudaStream_t s) {
     const int nt = pipe_nt(a.k);
-    if (mode == kTF32) return nt == 1 ? tf_launch<1, kTF32>(a, s) : nt == 2 ? tf_launch<2, kTF32>(a, s)
-                                                                           : tf_launch<4, kTF32>(a, s);
-    if (mode == kTF32X3) return nt == 1 ? tf_launch<1, kTF32X3>(a, s) : nt == 2 ? tf_launch<2, kTF32X3>(a, s)
-                                                                               : tf_launch<4, kTF32X3>(a, s);
+    if (mode == kTF32)
+        return nt == 1 ? tf_launch<1, kTF32>(a, s) : nt == 2 ? tf_launch<2, kTF32>(a, s)
+             : nt == 3 ? tf_launch<3, kTF32>(a, s) : tf_launch<4, kTF32>(a, s);
+    if (mode == kTF32X3)
+        return nt == 1 ? tf_launch<1, kTF32X3>(a, s) : nt == 2 ? tf_launch<2, kTF32X3>(a, s)
+             : nt == 3 ? tf_launch<3, kTF32X3>(a, s) : tf_launch<4, kTF32X3>(a, s);
     if (nt == 1) return pipe_launch<1>(a, s);
     if (nt == 2) return pipe_launch<2>(a, s);
+    if (nt == 3) return pipe_launch<3>(a, s);
     return pipe_launch<4>(a, s);
 }
 
 size_t fma32_pipe_smem_bytes(int64_t k, int warps) {
-    const int nt = pipe_nt(k);
+    const int nt = fpipe_nt(k);
     return nt == 1 ? fpipe_smem<1>(warps) : nt == 2 ? fpipe_smem<2>(warps) : fpipe_smem<4>(warps);
 }
 
 const void *fma32_pipe_kernel_ptr(int64_t k, bool ydouble) {
-    const int nt = pipe_nt(k);
+    const int nt = fpipe_nt(k);
     if (ydouble)
         return nt == 1 ? (const void *)fma32_pipe_kernel<1, double>
                        : nt == 2 ? (const void *)fma32_pipe_kernel<2, double> : (const void *)fma32_pipe_kernel<4, double>;
@@ -836,7 +854,7 @@ const void *fma32_pipe_kernel_ptr(int64_t k, bool ydouble) {
 }
 
 cudaError_t launch_fma32_pipe(bool ydouble, const ProdArgs &a, cudaStream_t s) {
-    const int nt = pipe_nt(a.k);
+    const int nt = fpipe_nt(a.k);
     if (ydouble) return nt == 1 ? fpipe_launch<1, double>(a, s) : nt == 2 ? fpipe_launch<2, double>(a, s)
                                                                           : fpipe_launch<4, double>(a, s);
     return nt == 1 ? fpipe_launch<1, float>(a, s) : nt == 2 ? fpipe_launch<2, float>(a, s)
