@@ -62,14 +62,19 @@ __device__ __noinline__ void fma_columns(const ProdArgs &a, int64_t n0, const Wo
 // WIDE passes put the 16 columns on the M side of the MMA and the rows, NR
 // groups of 8, on the N side, so that items of up to 8 rows take half the MMAs
 // (and the outputs of a store are 8 consecutive columns); narrow ones put the
-// (up to 16) rows on the M side and the 8 columns on the N side. Returns false,
-// with nothing written, when an output is not resolved by the fixed point.
+// (up to 16) rows on the M side and the 8 columns on the N side. Narrow passes of
+// up to 8 rows (PAIR) fill the M side with two digits of the 8 columns, j and
+// j + 1: accumulator L then holds level L of the even digits and level L + 1 of
+// the odd ones, and 19 MMAs make the 34 digit pairs (35 with the rows on the M
+// side, half of it padding). Returns false, with nothing written, when an output
+// is not resolved by the fixed point.
 template <bool TRANS, bool WIDE, int NR>
 __device__ __forceinline__ bool slice_pass(const ProdArgs &a, const SliceArgs &q, const WorkItem &w,
                                            const unsigned char *vsrc, int nsteps, int64_t n0, const uint32_t *cmax,
                                            unsigned char *ring, const int32_t *s_x, int lane, double &dot) {
     constexpr int S = kSliceStages, kStage = 16 * kSliceTile;
     constexpr int NX = WIDE ? 2 : 1, NA = WIDE ? NR : 1;
+    constexpr bool PAIR = !WIDE && NR == 1;
     const int g = lane >> 2, t4 = lane & 3;
     float acc[NA][kSliceLevels][4], low[NA][4];
 #pragma unroll
@@ -136,7 +141,13 @@ __device__ __forceinline__ bool slice_pass(const ProdArgs &a, const SliceArgs &q
                 const uint32_t rows[4] = {v[0][0], v[NR - 1][0], v[0][1], v[NR - 1][1]};   // M side of a narrow pass
 #pragma unroll
                 for (int j = 0; j < kSliceDigits && i + j < kSliceLevels; ++j) {
-                    if (WIDE) {
+                    if (PAIR) {
+                        if (j % 2) continue;
+                        const int j1 = j + 1 < kSliceDigits ? j + 1 : j;
+                        const bool one = j + 1 < kSliceDigits;   // the eighth digit is zero
+                        const uint32_t cols[4] = {b[0][j][0], one ? b[0][j1][0] : 0u, b[0][j][1], one ? b[0][j1][1] : 0u};
+                        mma_f16(acc[0][i + j], cols, v[0][0], v[0][1]);
+                    } else if (WIDE) {
                         const uint32_t cols[4] = {b[0][j][0], b[NX - 1][j][0], b[0][j][1], b[NX - 1][j][1]};
 #pragma unroll
                         for (int n = 0; n < NA; ++n) mma_f16(acc[n][i + j], cols, v[n % NR][0], v[n % NR][1]);
@@ -146,7 +157,10 @@ __device__ __forceinline__ bool slice_pass(const ProdArgs &a, const SliceArgs &q
                 }
                 if (i == 0) {   // magnitudes of the leading digits
                     constexpr uint32_t kAbs = 0x7fff7fffu;
-                    if (WIDE) {
+                    if (PAIR) {
+                        const uint32_t cols[4] = {b[0][0][0] & kAbs, 0u, b[0][0][1] & kAbs, 0u};
+                        mma_f16(low[0], cols, v[0][0] & kAbs, v[0][1] & kAbs);
+                    } else if (WIDE) {
                         const uint32_t cols[4] = {b[0][0][0] & kAbs, b[NX - 1][0][0] & kAbs, b[0][0][1] & kAbs,
                                                   b[NX - 1][0][1] & kAbs};
 #pragma unroll
@@ -167,8 +181,9 @@ __device__ __forceinline__ bool slice_pass(const ProdArgs &a, const SliceArgs &q
         __syncwarp();
     }
     // accumulator j = 2 h + e of tile n: row and column (relative to the item and the pass)
-    auto row_of = [&](int n, int h, int e) { return WIDE ? 8 * n + 2 * t4 + e : g + 8 * h; };
-    auto col_of = [&](int h, int e) { return WIDE ? g + 8 * h : 2 * t4 + e; };
+    // (PAIR: row 2 t4 + e, column g; h = 1 holds the odd digits, of one level more)
+    auto row_of = [&](int n, int h, int e) { return PAIR ? 2 * t4 + e : WIDE ? 8 * n + 2 * t4 + e : g + 8 * h; };
+    auto col_of = [&](int h, int e) { return PAIR ? g : WIDE ? g + 8 * h : 2 * t4 + e; };
     int er[NA][4], ec[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -186,20 +201,21 @@ __device__ __forceinline__ bool slice_pass(const ProdArgs &a, const SliceArgs &q
 #pragma unroll
     for (int n = 0; n < NA; ++n)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) ok &= er[n][j] >= 0 && (er[n][j] == 0 || ec[j] == 0 || low[n][j] >= kSliceGuard);
+        for (int j = 0; j < 4; ++j) ok &= er[n][j] >= 0 && (er[n][j] == 0 || ec[j] == 0 || low[n][PAIR ? j & 1 : j] >= kSliceGuard);
     if (!__all_sync(0xffffffffu, ok)) return false;
 #pragma unroll
     for (int n = 0; n < NA; ++n)
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            if (!WIDE && NR == 1 && j >= 2) continue;
+            if (PAIR && j >= 2) continue;
             const int r = row_of(n, j >> 1, j & 1);
             const int64_t c = n0 + col_of(j >> 1, j & 1);
             if (r >= w.B || c >= a.k) continue;
             const int64_t row = w.yrow + r;
             float lv[kSliceLevels];
 #pragma unroll
-            for (int L = 0; L < kSliceLevels; ++L) lv[L] = acc[n][L][j];
+            for (int L = 0; L < kSliceLevels; ++L)
+                lv[L] = acc[n][L][j] + (PAIR && L > 0 ? acc[n][L > 0 ? L - 1 : 0][(j + 2) & 3] : 0.f);
             double o = slice_value(lv, er[n][j] + ec[j] - 2114 + q.alpha_exp);
             double *y = static_cast<double *>(a.Y) + row * a.ldy + c;
             if (!q.alpha_pow2) o *= a.alpha;
