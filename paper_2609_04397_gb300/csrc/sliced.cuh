@@ -176,6 +176,32 @@ __device__ __forceinline__ double slice_value(const float (&c)[kSliceLevels], in
     return __longlong_as_double((long long)(bits | (neg ? 1ull << 63 : 0ull)));
 }
 
+// Sum over digits of one operand in registers (t[e][d], integers below 2^24) and of
+// the other across the four lanes of a group, two a lane (e): sum over d and j =
+// 2 t4 + e of t * 256^(12 - d - j), times 2^e2 and in units of 2^40 (the units of
+// slice_value), on every lane of the group. Two conversions, a fused multiply-add and
+// two additions of the FP64 pipe, which little else uses here; the largest part
+// carries the rounding.
+__device__ __forceinline__ double slice_value_of_lanes(const float (&t)[2][8], int t4, int e2) {
+    long long hi = 0, lo = 0;
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        long long p = __float2int_rn(t[e][0]), r = __float2int_rn(t[e][4]);
+#pragma unroll
+        for (int d = 1; d < 4; ++d) p = p * 256 + __float2int_rn(t[e][d]);
+#pragma unroll
+        for (int d = 5; d < 7; ++d) r = r * 256 + __float2int_rn(t[e][d]);
+        hi = hi * 256 + p;   // below 2^57
+        lo = lo * 256 + r;   // below 2^49
+    }
+    double v = fma((double)hi, 16777216.0, (double)lo);
+    v *= t4 == 0 ? 1.0 : t4 == 1 ? 0x1p-16 : t4 == 2 ? 0x1p-32 : 0x1p-48;
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    const uint64_t bits = (uint64_t)__double_as_longlong(v);
+    return (bits << 1) == 0 ? 0.0 : __longlong_as_double((long long)(bits + ((uint64_t)(int64_t)e2 << 52)));
+}
+
 // Carry the upper part of every level into the one above (exact: integers below 2^24)
 __device__ __forceinline__ void slice_carry(float (&acc)[kSliceLevels][4]) {
 #pragma unroll

@@ -66,15 +66,27 @@ __device__ __noinline__ void fma_columns(const ProdArgs &a, int64_t n0, const Wo
 // up to 8 rows (PAIR) fill the M side with two digits of the 8 columns, j and
 // j + 1: accumulator L then holds level L of the even digits and level L + 1 of
 // the odd ones, and 19 MMAs make the 34 digit pairs (35 with the rows on the M
-// side, half of it padding). Returns false, with nothing written, when an output
+// side, half of it padding). NINTH: items of 9 rows (an sp3d5 basis), the ninth
+// alone with its digits as the N side, one more MMA per digit of X (PAIR: per two)
+// instead of another group of 8 rows: 44 MMAs a wide step instead of 72, 25 a
+// narrow one instead of 36 (50k zinc-blende atoms, k = 32: 1.43 ms against 1.56). Returns false, with nothing written, when an output
 // is not resolved by the fixed point.
-template <bool TRANS, bool WIDE, int NR>
+template <bool TRANS, bool WIDE, int NR, bool NINTH = false>
 __device__ __forceinline__ bool slice_pass(const ProdArgs &a, const SliceArgs &q, const WorkItem &w,
                                            const unsigned char *vsrc, int nsteps, int64_t n0, const uint32_t *cmax,
                                            unsigned char *ring, const int32_t *s_x, int lane, double &dot) {
     constexpr int S = kSliceStages, kStage = 16 * kSliceTile;
     constexpr int NX = WIDE ? 2 : 1, NA = WIDE ? NR : 1;
     constexpr bool PAIR = !WIDE && NR == 1;
+    // the ninth row: digit j of X (PAIR: j and j + 1) times all its digits, 2 t4 + e a lane
+    constexpr int NJ = NINTH ? (WIDE ? kSliceDigits : 4) : 1;
+    float ninth[NJ][4], nlow[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        nlow[r] = 0.f;
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) ninth[j][r] = 0.f;
+    }
     const int g = lane >> 2, t4 = lane & 3;
     float acc[NA][kSliceLevels][4], low[NA][4];
 #pragma unroll
@@ -128,6 +140,24 @@ __device__ __forceinline__ bool slice_pass(const ProdArgs &a, const SliceArgs &q
             for (int n = 0; n < NX; ++n) slice_pairs<kSliceDigits>(x[n], b[n]);
             load_x(s + 1);   // the list has one step past the last
             const unsigned char *st = ring + (s % S) * kStage + g * 16 + t4 * 4;
+            if constexpr (NINTH) {
+                constexpr uint32_t kAbs = 0x7fff7fffu;
+                // digit g of the ninth row (the eighth digit is zero)
+                const uint32_t word = g < kSliceDigits ? *reinterpret_cast<const uint32_t *>(
+                                                             ring + (s % S) * kStage + g * digit + 128 + t4 * 4)
+                                                       : 0x80808080u;
+                const uint32_t v0 = slice_half2(word, 0x4140), v1 = slice_half2(word, 0x4342);
+#pragma unroll
+                for (int j = 0; j < NJ; ++j) {
+                    const int a0 = WIDE ? j : 2 * j, a1 = WIDE || j == 3 ? a0 : a0 + 1;
+                    const uint32_t cols[4] = {b[0][a0][0], WIDE ? b[NX - 1][a0][0] : j == 3 ? 0u : b[0][a1][0],
+                                              b[0][a0][1], WIDE ? b[NX - 1][a0][1] : j == 3 ? 0u : b[0][a1][1]};
+                    mma_f16(ninth[j], cols, v0, v1);
+                }
+                const uint32_t cols[4] = {b[0][0][0] & kAbs, WIDE ? b[NX - 1][0][0] & kAbs : 0u, b[0][0][1] & kAbs,
+                                          WIDE ? b[NX - 1][0][1] & kAbs : 0u};
+                mma_f16(nlow, cols, v0 & kAbs, v1 & kAbs);
+            }
 #pragma unroll
             for (int i = 0; i < kSliceDigits; ++i, st += digit) {
                 // digit i of rows g (and g + 8)
@@ -202,7 +232,36 @@ __device__ __forceinline__ bool slice_pass(const ProdArgs &a, const SliceArgs &q
     for (int n = 0; n < NA; ++n)
 #pragma unroll
         for (int j = 0; j < 4; ++j) ok &= er[n][j] >= 0 && (er[n][j] == 0 || ec[j] == 0 || low[n][PAIR ? j & 1 : j] >= kSliceGuard);
+    const int e9 = NINTH ? q.rexp[w.yrow + 8] : 0;
+    if (NINTH) {
+        ok &= e9 >= 0;
+#pragma unroll
+        for (int h = 0; h < NX; ++h)   // lanes t4 = 0 hold digit 0
+            ok &= e9 == 0 || ec[2 * h] == 0 || t4 != 0 || nlow[2 * h] >= kSliceGuard;
+    }
     if (!__all_sync(0xffffffffu, ok)) return false;
+    auto store = [&](int64_t row, int64_t c, double o) {
+        double *y = static_cast<double *>(a.Y) + row * a.ldy + c;
+        if (!q.alpha_pow2) o *= a.alpha;
+        if (a.beta_nz) o += a.beta * *y;
+        if (a.gamma_nz) o += a.gamma * static_cast<const double *>(a.Z)[row * a.ldz + c];
+        *y = o;
+        if (a.item_partials) dot += static_cast<const double *>(a.R)[row * a.ldr + c] * o;
+    };
+    if constexpr (NINTH) {
+#pragma unroll
+        for (int h = 0; h < NX; ++h) {   // column g + 8 h
+            // the digits of X in units of their last, for the lane's digits 2 t4 and 2 t4 + 1 of the row
+            float t[2][8];
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+#pragma unroll
+                for (int d = 0; d < kSliceDigits; ++d)
+                    t[e][d] = WIDE ? ninth[d % NJ][2 * h + e] : ninth[d / 2 % NJ][2 * (d & 1) + e];
+            const double o = slice_value_of_lanes(t, t4, e9 + ec[2 * h] - 2114 + q.alpha_exp);
+            if (t4 == 0 && n0 + g + 8 * h < a.k) store(w.yrow + 8, n0 + g + 8 * h, o);
+        }
+    }
 #pragma unroll
     for (int n = 0; n < NA; ++n)
 #pragma unroll
@@ -210,19 +269,13 @@ __device__ __forceinline__ bool slice_pass(const ProdArgs &a, const SliceArgs &q
             if (PAIR && j >= 2) continue;
             const int r = row_of(n, j >> 1, j & 1);
             const int64_t c = n0 + col_of(j >> 1, j & 1);
-            if (r >= w.B || c >= a.k) continue;
+            if (r >= (NINTH ? 8 : w.B) || c >= a.k) continue;
             const int64_t row = w.yrow + r;
             float lv[kSliceLevels];
 #pragma unroll
             for (int L = 0; L < kSliceLevels; ++L)
                 lv[L] = acc[n][L][j] + (PAIR && L > 0 ? acc[n][L > 0 ? L - 1 : 0][(j + 2) & 3] : 0.f);
-            double o = slice_value(lv, er[n][j] + ec[j] - 2114 + q.alpha_exp);
-            double *y = static_cast<double *>(a.Y) + row * a.ldy + c;
-            if (!q.alpha_pow2) o *= a.alpha;
-            if (a.beta_nz) o += a.beta * *y;
-            if (a.gamma_nz) o += a.gamma * static_cast<const double *>(a.Z)[row * a.ldz + c];
-            *y = o;
-            if (a.item_partials) dot += static_cast<const double *>(a.R)[row * a.ldr + c] * o;
+            store(row, c, slice_value(lv, er[n][j] + ec[j] - 2114 + q.alpha_exp));
         }
     return true;
 }
@@ -338,29 +391,13 @@ __device__ __forceinline__ bool slice_thin(const ProdArgs &a, const SliceArgs &q
         const int r = g + 8 * h;
 #pragma unroll
         for (int n = 0; n < KC; ++n) {
-            // sum over the digits of the values, in units of their last: hi * 2^24 + lo, for the
-            // lane's two digits of X together (hi below 2^57, lo below 2^49)
-            long long hi = 0, lo = 0;
+            float t[2][8];
 #pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                long long p = __float2int_rn(acc[0][n][2 * h + e]), t = __float2int_rn(acc[4][n][2 * h + e]);
+            for (int e = 0; e < 2; ++e)
 #pragma unroll
-                for (int i = 1; i < 4; ++i) p = p * 256 + __float2int_rn(acc[i][n][2 * h + e]);
-#pragma unroll
-                for (int i = 5; i < 7; ++i) t = t * 256 + __float2int_rn(acc[i][n][2 * h + e]);
-                hi = hi * 256 + p;
-                lo = lo * 256 + t;
-            }
-            // a pair of digits weighs 2^-16 of the one before
-            double d = fma((double)hi, 16777216.0, (double)lo);
-            d *= t4 == 0 ? 1.0 : t4 == 1 ? 0x1p-16 : t4 == 2 ? 0x1p-32 : 0x1p-48;
-            d += __shfl_xor_sync(0xffffffffu, d, 2);
-            d += __shfl_xor_sync(0xffffffffu, d, 1);
+                for (int i = 0; i < kSliceDigits; ++i) t[e][i] = acc[i][n][2 * h + e];
+            double o = slice_value_of_lanes(t, t4, er[h] + ec[n] - 2114 + q.alpha_exp);
             if (t4 == 0 && r < w.B) {
-                // digits 0 and 1 of X in units of 256^5: the same exponent as the level sums of a pass
-                const uint64_t bits = (uint64_t)__double_as_longlong(d);
-                const int e2 = er[h] + ec[n] - 2114 + q.alpha_exp;
-                double o = (bits << 1) == 0 ? 0.0 : __longlong_as_double((long long)(bits + ((uint64_t)(int64_t)e2 << 52)));
                 const int64_t row = w.yrow + r;
                 double *y = static_cast<double *>(a.Y) + row * a.ldy + n;
                 if (!q.alpha_pow2) o *= a.alpha;
@@ -436,11 +473,15 @@ __global__ void __launch_bounds__(128, FORM == 0 || FORM == 3 ? 3 : FORM == 1 ? 
             if constexpr (FORM == 0)
                 for (; ok && n0 + 8 < a.k; n0 += ok ? 16 : 0)
                     ok = w.B <= 8 ? slice_pass<TRANS, true, 1>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot)
-                                  : slice_pass<TRANS, true, 2>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot);
+                         : w.B == 9
+                             ? slice_pass<TRANS, true, 1, true>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot)
+                             : slice_pass<TRANS, true, 2>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot);
             if constexpr (FORM == 0 || FORM == 8) {
                 if (ok && n0 < a.k) {
                     ok = w.B <= 8
                              ? slice_pass<TRANS, false, 1>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot)
+                         : w.B == 9
+                             ? slice_pass<TRANS, false, 1, true>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot)
                              : slice_pass<TRANS, false, 2>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot);
                     n0 += ok ? 8 : 0;
                 }

@@ -94,6 +94,36 @@ def test_exact_level_sums_at_the_widest_row():
             assert (got - exact).abs().max().item() <= 4e-16 * abs(exact)
 
 
+@pytest.mark.parametrize("k", [7, 8, 16, 19])   # from 7 columns on, an operator of this size is sliced
+def test_items_of_nine_rows(k):
+    """The ninth row's digits are the N side of its own products: the largest digit sums of
+    765 columns, and ninth rows that are zero, far smaller than the others or unresolved."""
+    b = 9
+    pat = BlockPattern(np.full(90, b), np.full(85, b), np.arange(91) * 85, np.tile(np.arange(85), 90))
+    h = float(0x7D808080808080 - 0x01010101010100) * 2.0 ** -54
+    H = _handle(pat, np.full(pat.nnz, h))
+    X = torch.full((765, k), -h, dtype=torch.float64, device="cuda:0")
+    from fractions import Fraction
+    exact = float(-765 * Fraction(h) * Fraction(h))
+    got = H.spmm(X)
+    assert (got - exact).abs().max().item() <= 4e-16 * abs(exact)
+    assert any("slice_product" in n for n in _kernels(lambda: H.spmm(X)))
+    rng = np.random.default_rng(k)
+    vals = rng.standard_normal(pat.nnz).reshape(90, 85, b, b)   # blocks of a block row are b x b
+    vals[0, :, 8] = 0.0
+    vals[1, :, 8] *= 1e-200
+    vals[2, :, 8, :] = 0.0
+    vals[2, 3, 8, 4] = 1.0
+    vals[3, :, 8] *= np.exp(-np.arange(85) / 3.0)[:, None]
+    vals = vals.reshape(-1)
+    X = rng.standard_normal((765, k))
+    X[:40, k // 2] = 0.0
+    H = _handle(pat, vals)
+    Y0 = rng.standard_normal((810, k))
+    _check(H, pat, vals, X, alpha=0.3, beta=2.0, Y0=Y0)
+    _check(H, pat, vals, rng.standard_normal((810, k)), transpose=True)
+
+
 def test_unresolved_outputs_take_multiply_adds():
     """Graded rows and columns, zero rows and columns, panels supported on a few
     rows, tiny and huge magnitudes, Inf and NaN: every output as accurate as the
