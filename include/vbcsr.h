@@ -72,7 +72,24 @@ typedef enum {
  * handle owns (allocated on first use and grown when a call needs more;
  * growing it synchronises the stream). Mixed-mode calls on one handle
  * therefore must not overlap on the GPU.
- *  NATIVE  products and accumulation in the matrix dtype (FP64 FMA / FP32 FMA)
+ *  NATIVE  products and accumulation in the matrix dtype's precision. FP32:
+ *          FMA. FP64 and complex FP64: block operators (not the CSR backend)
+ *          of at least 2^22 stored entries x columns per structure (2^26 /
+ *          2^25 for 1 / 2 columns), of whose work nine tenths lie in rows of
+ *          at most 768 entries (384 complex), run these rows on the tensor
+ *          cores: rows of H and columns of X as 56-bit fixed-point
+ *          integers in exact base-256 digits, their products summed exactly
+ *          and rounded once. An output that the fixed point does not resolve
+ *          (its terms far below its row's or column's largest), rows and
+ *          columns with Inf, NaN or extreme exponents, and everything smaller
+ *          is computed by FP64 FMA; either way the error is within that of an
+ *          FMA chain. The digits of the values (7 bytes an entry, one copy a
+ *          direction) and of X are buffers that the handle owns, allocated on
+ *          first use and grown like those of the mixed modes; while `stream`
+ *          is being captured, or when the device has no room, nothing is
+ *          allocated and such a call runs by FMA. Make one ordinary call
+ *          before a capture so that the graph gets the tensor-core form; a
+ *          graph stays valid when later calls need larger buffers.
  *  F32     values and X rounded to FP32, FP32 FMA, FP32 accumulation
  *  TF32    one TF32 tensor-core product per block product, FP32 accumulation
  *  TF32X3  v = hi + lo with hi = tf32(v), lo = tf32(v - hi) for values and X;
@@ -272,6 +289,10 @@ int vbcsr_spmm_ex(vbcsr_t *A, int transpose, int64_t k, double alpha, const void
  * for every stored block (i, j), written in packed order.
  *  Aop  device [n_rows, k], lda >= k;  Bop  device [n_cols, k], ldb >= k
  *  D    device, nnz elements of the matrix dtype; beta == 0: D is not read
+ * FP64 operators of at least 2^22 stored entries x columns, 3 <= k <= 768, form it on
+ * the tensor cores like the native products, with fixed-point copies of Aop and Bop in a
+ * buffer of the handle (8 bytes an element, columns rounded up to 16), allocated and
+ * grown on first use as theirs are, and by FMA where those would be.
  * (This operation has no counterpart in the paper.)
  */
 int vbcsr_sddmm(vbcsr_t *A, int64_t k, double alpha, const void *Aop, int64_t lda,
@@ -409,6 +430,8 @@ int vbcsr_shift_scale(vbcsr_t *A, double c, double d, void *stream);
  *         VBCSR_ERR_UNSUPPORTED and launch nothing.
  *  The first call on a device looks up the array's device address (with
  *  that device current); make that first call before any stream capture.
+ *  NATIVE products run on the tensor cores only when an earlier call on the
+ *  handle has built their buffers, else by FMA.
  *  All calls share the one array: calls whose work overlaps on the GPU (on
  *  different streams, or from several threads) race and give wrong moments.
  *  Nothing in the array needs to start at zero: each call writes every element
@@ -498,7 +521,8 @@ int vbcsr_shape_classes(const vbcsr_t *A, int32_t *bi, int32_t *bj, int64_t *cou
  *                           persistent launch (0 = 4)
  *  vbcsr_get_tuning         reads them back: kc_by_b[17], warps_by_b[17] (index = B;
  *                           any pointer may be NULL)
- * They apply to later calls on this handle. The tensor-core modes ignore them.
+ * They apply to later calls on this handle. The tensor-core modes and the native FP64
+ * products that run on the tensor cores ignore them.
  */
 int vbcsr_set_tuning(vbcsr_t *A, int32_t kc, int32_t warps_per_cta);
 int vbcsr_set_bucket_tuning(vbcsr_t *A, int32_t B, int32_t kc, int32_t warps_per_cta);
@@ -513,7 +537,8 @@ int vbcsr_get_tuning(const vbcsr_t *A, int32_t *kc_by_b, int32_t *warps_by_b, in
  * whichever schedule is faster (unless flags has VBCSR_TUNE_NO_PERSISTENT).
  * X and Y are device panels of the product's shapes; Y is overwritten. The
  * call synchronises `stream` repeatedly (a set-up step: do not capture it in
- * a CUDA graph). For the tensor-core precisions it only chooses, for the
+ * a CUDA graph). A native FP64 product that runs on the tensor cores takes the
+ * same time in every trial. For the tensor-core precisions it only chooses, for the
  * forward product, between the plain and the shared-memory-staged kernel.
  * (The per-shape-group tuning of tiles has no counterpart in the paper.)
  */

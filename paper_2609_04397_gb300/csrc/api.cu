@@ -156,6 +156,7 @@ struct vbcsr_matrix {
     size_t xdig_elems = 0;
     uint64_t *sdpan = nullptr;   // fixed-point rows of A and B of the sliced pattern-sampled product
     size_t sdpan_elems = 0;
+    bool xdig_captured = false, stab_captured = false, sdpan_captured = false;   // a graph holds the buffer
     bool sd_no_room = false;
     uint32_t *stab = nullptr;
     size_t stab_elems = 0;
@@ -900,6 +901,35 @@ static int grow(vbcsr_t *A, T **buf, size_t *have, size_t need, cudaStream_t s, 
     return VBCSR_OK;
 }
 
+// The same for a buffer of the native products, which need none without slicing: graphs
+// that hold the old one (*captured) stay valid, so it is kept until the handle goes, and
+// the new one is at least twice its size (what is kept stays below what is in use).
+// A capture on another thread is not disturbed by the allocation.
+template <typename T>
+static int grow_native(vbcsr_t *A, T **buf, size_t *have, size_t need, bool *captured, cudaStream_t s,
+                       const char *what) {
+    if (need <= *have) return VBCSR_OK;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    CUDA_TRY(cudaThreadExchangeStreamCaptureMode(&mode), "capture mode");
+    int rc = VBCSR_OK;
+    if (*captured) {
+        T *more = nullptr;
+        const size_t n = std::max(need, 2 * *have);
+        const cudaError_t e = A->alloc(&more, n);
+        if (e == cudaSuccess) {
+            *buf = more;
+            *have = n;
+            *captured = false;
+        } else {
+            rc = cuda_fail(e, what);
+        }
+    } else {
+        rc = grow(A, buf, have, need, s, what);
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    return rc;
+}
+
 // The digit tiles of one direction, from the values now in the pages
 static int refresh_slices(vbcsr_t *A, bool trans, cudaStream_t s) {
     SlicePlan &p = A->slice[trans];
@@ -1182,6 +1212,8 @@ static int slice_prepare(vbcsr_t *A, bool trans, int64_t k, bool may_alloc, cuda
     const bool cap = capturing(s);
     if (*ready) {
         p.captured |= cap;
+        A->xdig_captured |= cap;
+        A->stab_captured |= cap;
         if (p.stale) {
             // under capture the rebuild belongs to the graph: the tiles stay stale for eager calls
             int rc = refresh_slices(A, trans, s);
@@ -1193,8 +1225,11 @@ static int slice_prepare(vbcsr_t *A, bool trans, int64_t k, bool may_alloc, cuda
     if (!may_alloc || p.no_room || cap) return VBCSR_OK;
     int rc = VBCSR_OK;
     if (!p.vdig) {
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        CUDA_TRY(cudaThreadExchangeStreamCaptureMode(&mode), "capture mode");
         cudaError_t e = p.rexp ? cudaSuccess : A->alloc(&p.rexp, (size_t)(trans ? A->n_cols : A->n_rows));
         if (e == cudaSuccess) e = A->alloc(&p.vdig, (size_t)p.digit_bytes);
+        cudaThreadExchangeStreamCaptureMode(&mode);
         if (e != cudaSuccess) rc = cuda_fail(e, "alloc value digits");
         p.stale = p.vdig != nullptr;
     }
@@ -1203,8 +1238,11 @@ static int slice_prepare(vbcsr_t *A, bool trans, int64_t k, bool may_alloc, cuda
         p.stale = rc != VBCSR_OK;
     }
     if (!rc)
-        rc = grow(A, &A->xdig, &A->xdig_elems, slice_x_elems(A, trans, k), s, "alloc fixed-point X");
-    if (!rc) rc = grow(A, &A->stab, &A->stab_elems, slice_tab_elems(A, slice_ldp(k)), s, "alloc column maxima");
+        rc = grow_native(A, &A->xdig, &A->xdig_elems, slice_x_elems(A, trans, k), &A->xdig_captured, s,
+                         "alloc fixed-point X");
+    if (!rc)
+        rc = grow_native(A, &A->stab, &A->stab_elems, slice_tab_elems(A, slice_ldp(k)), &A->stab_captured, s,
+                         "alloc column maxima");
     if (rc == VBCSR_ERR_NO_MEMORY) {
         p.no_room = true;
         return VBCSR_OK;
@@ -1604,7 +1642,8 @@ static int run_sddmm_f64(vbcsr_t *A, const SddmmArgs &a, cudaStream_t s) {
             if (A->sd_no_room || capturing(s)) {
                 sliced = false;
             } else {
-                const int rc = grow(A, &A->sdpan, &A->sdpan_elems, need, s, "alloc fixed-point panels");
+                const int rc = grow_native(A, &A->sdpan, &A->sdpan_elems, need, &A->sdpan_captured, s,
+                                           "alloc fixed-point panels");
                 if (rc == VBCSR_ERR_NO_MEMORY) {
                     A->sd_no_room = true;
                     sliced = false;
@@ -1614,6 +1653,7 @@ static int run_sddmm_f64(vbcsr_t *A, const SddmmArgs &a, cudaStream_t s) {
             }
         }
         if (sliced) {
+            A->sdpan_captured |= capturing(s);
             uint64_t *fa = A->sdpan, *fb = fa + A->n_rows * kp;
             int32_t *ea = reinterpret_cast<int32_t *>(fb + A->n_cols * kp), *eb = ea + A->n_rows;
             CUDA_TRY(launch_sddmm_sliced(a, A->n_rows, A->n_cols, fa, fb, ea, eb, s), "sddmm launch");

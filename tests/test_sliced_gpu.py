@@ -238,6 +238,27 @@ def test_tiles_follow_the_values():
     _check(H, pat, v[1], G, transpose=True)
 
 
+def test_captured_products_outlive_larger_ones():
+    """A graph's buffers stay when a wider product, or a wider sampled one, needs larger ones."""
+    w = syn.amorphous(700, side=60.0 * (700 / 20000) ** (1 / 3))
+    pat = w.pattern
+    H = _handle(pat, w.values)
+    rng = np.random.default_rng(3)
+    X, Xw = (rng.standard_normal((pat.n_cols, k)) for k in (16, 90))
+    Xd, Xwd = torch.from_numpy(X).cuda(), torch.from_numpy(Xw).cuda()
+    A, Aw = torch.randn_like(Xd[:pat.n_rows]), torch.randn_like(Xwd[:pat.n_rows])
+    Y, D = H.spmm(Xd), H.sddmm(A, Xd)
+    Yg, Dg = torch.empty_like(Y), torch.empty_like(D)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        H.spmm(Xd, 1.0, 0.0, Yg)
+        H.sddmm(A, Xd, 1.0, 0.0, Dg)
+    _check(H, pat, w.values, Xw)
+    H.sddmm(Aw, Xwd)
+    graph.replay()
+    assert torch.equal(Yg, Y) and torch.equal(Dg, D)
+
+
 @pytest.mark.parametrize("k", [3, 7, 16, 17, 40, 200])
 def test_sliced_sddmm_against_oracle(k):
     """The pattern-sampled product, contracting over the panel columns: row heights 1 to 33,
