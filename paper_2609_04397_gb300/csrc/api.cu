@@ -1151,7 +1151,7 @@ static ModePlan plan_mode(const vbcsr_t *A, bool trans, int64_t k, int precision
     // to 16 columns (at 17-32 its 32-column tiles hold 4 CTAs per SM and the register-load
     // kernel is 3 % faster: 0.58 against 0.60 ms at k = 32 on the 50k-atom operator)
     p.pipe_tf = p.f64 && (p.mode == VBCSR_PREC_TF32 || p.mode == VBCSR_PREC_TF32X3) && !trans && !p.split &&
-                k <= 24 && !p.csr_kernel && !(A->schedule & VBCSR_SCHED_MMA_STAGED) &&
+                k <= 16 && !p.csr_kernel && !(A->schedule & VBCSR_SCHED_MMA_STAGED) &&
                 A->backend != VBCSR_BACKEND_CSR;
     p.presplit = p.f64 && p.mode == VBCSR_PREC_BF16X2 && !trans && !p.csr_kernel && !p.pipe &&
                  (p.split || !(A->schedule & VBCSR_SCHED_MMA_STAGED));

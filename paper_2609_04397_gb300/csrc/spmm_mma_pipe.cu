@@ -792,8 +792,10 @@ cudaError_t fpipe_launch(const ProdArgs &a, cudaStream_t s) {
 
 }  // namespace
 
-// 8-column tiles of a pass. 17 to 24 columns take 3: the 4-tile pass computes 32 (tiles of
-// 3 need no swizzle: their X rows of 48 or 96 bytes already fall on distinct banks).
+// 8-column tiles of a pass of the BF16X2 kernel, and of the others. There 17 to 24 columns
+// take 3 (the 4-tile pass computes 32; 364 against 406 us at k = 24 on the 50k-atom
+// operator; tiles of 3 need no swizzle: their X rows of 48 bytes already fall on
+// distinct banks).
 static int pipe_nt(int64_t k) { return k <= 8 ? 1 : (k <= 16 ? 2 : (k <= 24 ? 3 : 4)); }
 static int fpipe_nt(int64_t k) { return k <= 8 ? 1 : (k <= 16 ? 2 : 4); }
 
@@ -803,22 +805,20 @@ int64_t pipe_ldp(int64_t k) {
 }
 
 size_t mma_pipe_smem_bytes(int mode, int64_t k, int warps) {
-    const int nt = pipe_nt(k);
-    if (mode != kBF16X2) return nt == 1 ? tf_smem<1>(warps) : nt == 2 ? tf_smem<2>(warps) : nt == 3 ? tf_smem<3>(warps) : tf_smem<4>(warps);
+    const int nt = mode == kBF16X2 ? pipe_nt(k) : fpipe_nt(k);
+    if (mode != kBF16X2) return nt == 1 ? tf_smem<1>(warps) : nt == 2 ? tf_smem<2>(warps) : tf_smem<4>(warps);
     return nt == 1 ? pipe_smem<1>(warps) : nt == 2 ? pipe_smem<2>(warps) : nt == 3 ? pipe_smem<3>(warps) : pipe_smem<4>(warps);
 }
 
 const void *mma_pipe_kernel_ptr(int mode, int64_t k) {
-    const int nt = pipe_nt(k);
+    const int nt = mode == kBF16X2 ? pipe_nt(k) : fpipe_nt(k);
     if (mode == kTF32)
         return nt == 1 ? (const void *)mma_tf32_pipe_kernel<1, kTF32>
                        : nt == 2 ? (const void *)mma_tf32_pipe_kernel<2, kTF32>
-                       : nt == 3 ? (const void *)mma_tf32_pipe_kernel<3, kTF32>
                                  : (const void *)mma_tf32_pipe_kernel<4, kTF32>;
     if (mode == kTF32X3)
         return nt == 1 ? (const void *)mma_tf32_pipe_kernel<1, kTF32X3>
                        : nt == 2 ? (const void *)mma_tf32_pipe_kernel<2, kTF32X3>
-                       : nt == 3 ? (const void *)mma_tf32_pipe_kernel<3, kTF32X3>
                                  : (const void *)mma_tf32_pipe_kernel<4, kTF32X3>;
     return nt == 1 ? (const void *)mma_bf16_pipe_kernel<1>
                    : nt == 2 ? (const void *)mma_bf16_pipe_kernel<2>
@@ -826,13 +826,11 @@ const void *mma_pipe_kernel_ptr(int mode, int64_t k) {
 }
 
 cudaError_t launch_mma_pipe(int mode, const ProdArgs &a, cudaStream_t s) {
-    const int nt = pipe_nt(a.k);
-    if (mode == kTF32)
-        return nt == 1 ? tf_launch<1, kTF32>(a, s) : nt == 2 ? tf_launch<2, kTF32>(a, s)
-             : nt == 3 ? tf_launch<3, kTF32>(a, s) : tf_launch<4, kTF32>(a, s);
-    if (mode == kTF32X3)
-        return nt == 1 ? tf_launch<1, kTF32X3>(a, s) : nt == 2 ? tf_launch<2, kTF32X3>(a, s)
-             : nt == 3 ? tf_launch<3, kTF32X3>(a, s) : tf_launch<4, kTF32X3>(a, s);
+    const int nt = mode == kBF16X2 ? pipe_nt(a.k) : fpipe_nt(a.k);
+    if (mode == kTF32) return nt == 1 ? tf_launch<1, kTF32>(a, s) : nt == 2 ? tf_launch<2, kTF32>(a, s)
+                                                                           : tf_launch<4, kTF32>(a, s);
+    if (mode == kTF32X3) return nt == 1 ? tf_launch<1, kTF32X3>(a, s) : nt == 2 ? tf_launch<2, kTF32X3>(a, s)
+                                                                               : tf_launch<4, kTF32X3>(a, s);
     if (nt == 1) return pipe_launch<1>(a, s);
     if (nt == 2) return pipe_launch<2>(a, s);
     if (nt == 3) return pipe_launch<3>(a, s);
