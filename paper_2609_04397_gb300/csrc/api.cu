@@ -970,9 +970,10 @@ static int slices_changed(vbcsr_t *A, cudaStream_t s) {
 }
 
 // True when a native FP64 product of k columns runs sliced.
-static bool slice_applies(const vbcsr_t *A, bool trans, int64_t k) {
+static bool slice_applies(const vbcsr_t *A, bool trans, int64_t k, bool repeated) {
     const SlicePlan &p = A->slice[trans];
-    return p.applies && !p.untracked && k <= (1 << 20) && p.max_nnz * k >= slice_min_work(k) && !A->debug_checks;
+    return p.applies && !p.untracked && k <= (1 << 20) && p.max_nnz >= slice_min_nnz(k, repeated) &&
+           !A->debug_checks;
 }
 
 // k counts real columns here and below (two a column of a complex operator)
@@ -1254,7 +1255,8 @@ static int slice_prepare(vbcsr_t *A, bool trans, int64_t k, bool may_alloc, cuda
 
 static int run_product(vbcsr_t *A, bool trans, int64_t k, double alpha, const void *X, int64_t ldx, double beta,
                        void *Y, int64_t ldy, const vbcsr_epilogue_t *epi, int precision, cudaStream_t s,
-                       double dot_scale = 1.0, const FusedX *fx = nullptr, bool may_alloc = true) {
+                       double dot_scale = 1.0, const FusedX *fx = nullptr, bool may_alloc = true,
+                       bool repeated = false) {
     if (!A) return fail(VBCSR_ERR_INVALID_ARG, "handle is NULL");
     if (k < 0) return fail(VBCSR_ERR_INVALID_ARG, "k = %lld", (long long)k);
     if (precision < VBCSR_PREC_NATIVE || precision > VBCSR_PREC_DF32)
@@ -1302,7 +1304,8 @@ static int run_product(vbcsr_t *A, bool trans, int64_t k, double alpha, const vo
         if (rc) return rc;
     }
     const int64_t kr = cplx ? 2 * k : k;   // real columns
-    bool sliced = (f64 || cplx) && mode == VBCSR_PREC_NATIVE && alpha != 0.0 && slice_applies(A, trans, kr);
+    bool sliced = (f64 || cplx) && mode == VBCSR_PREC_NATIVE && alpha != 0.0 &&
+                  slice_applies(A, trans, kr, repeated);
     if (sliced) {
         int rc = slice_prepare(A, trans, kr, may_alloc, s, &sliced);
         if (rc) return rc;
@@ -1494,6 +1497,7 @@ static int run_product(vbcsr_t *A, bool trans, int64_t k, double alpha, const vo
         sa.ccnt = ccnt;
         sa.struct_rows = p.struct_rows;
         sa.struct_nnz = p.struct_nnz;
+        sa.min_nnz = slice_min_nnz(kr, repeated);
         sa.ldp = xld;
         int ae = 0;
         sa.alpha_pow2 = std::frexp(alpha, &ae) == 0.5 && std::abs(ae) < 128;
@@ -1629,12 +1633,11 @@ static SddmmArgs sddmm_args(vbcsr_t *A) {
 }
 
 // FP64 pattern-sampled product: sliced when it has enough work (below, the extra
-// launch costs more than the multiply-adds), at k >= 3 (one and two columns need
-// half a clock and a clock an entry on the FP64 pipe, about what the tensor-core
-// tile takes) and up to the widths whose level sums stay exact; else by multiply-adds, as on a stream that
-// is being captured before the buffers exist.
+// launch costs more than the multiply-adds), from kSddmmMinCols columns and up to the
+// widths whose level sums stay exact; else by multiply-adds, as on a stream that is
+// being captured before the buffers exist.
 static int run_sddmm_f64(vbcsr_t *A, const SddmmArgs &a, cudaStream_t s) {
-    bool sliced = a.k >= 3 && a.k <= kSliceKMax && a.alpha != 0.0 && A->nnz * a.k >= slice_min_work(3) && !A->debug_checks;
+    bool sliced = a.k >= kSddmmMinCols && a.k <= kSliceKMax && a.alpha != 0.0 && A->nnz * a.k >= kSddmmMinWork && !A->debug_checks;
     if (sliced) {
         const int64_t kp = (a.k + 15) / 16 * 16, rows = A->n_rows + A->n_cols;
         const size_t need = (size_t)(rows * kp + (rows + 1) / 2);
@@ -1762,7 +1765,7 @@ static int run_chebyshev(vbcsr_t *A, int64_t k, const double *R, int64_t ldr, in
     // with the fused form, t_n is also kept converted in xs[n & 1]
     const FusedX fx0 = {nullptr, xs[1]};
     int rc = run_product(A, false, k, 1.0, R, ldr, 0.0, buf[1], k, &epi, precision, s, scale, xs[1] ? &fx0 : nullptr,
-                         may_alloc);
+                         may_alloc, true);
     if (rc) return rc;
     auto store_pair = [&](int64_t m, const double *tm, int64_t ldm, const double *tm1) -> int {
         if (!ckpt || m % ckpt_every) return VBCSR_OK;
@@ -1780,7 +1783,7 @@ static int run_chebyshev(vbcsr_t *A, int64_t k, const double *R, int64_t ldr, in
         epi.dot_out = moments + n + 1;
         const FusedX fx = {xs[n & 1], xs[(n + 1) & 1]};
         rc = run_product(A, false, k, 2.0, tn, k, -1.0, tprev, k, &epi, precision, s, scale, xs[0] ? &fx : nullptr,
-                         may_alloc);
+                         may_alloc, true);
         if (rc) return rc;
         if ((rc = store_pair(n, tn, k, tprev))) return rc;
     }
@@ -1833,7 +1836,8 @@ extern "C" int vbcsr_chebyshev_backward(vbcsr_t *A, int64_t k, const double *R, 
             epi.gamma = -1.0;
             epi.Z = T + (e - 1) * k;
             epi.ldz = wide;
-            rc = run_product(A, false, k, 2.0, T + e * k, wide, 0.0, T + (e + 1) * k, wide, &epi, precision, s);
+            rc = run_product(A, false, k, 2.0, T + e * k, wide, 0.0, T + (e + 1) * k, wide, &epi, precision, s, 1.0,
+                             nullptr, true, true);
             if (rc) return rc;
         }
         for (int64_t n = n_hi; n >= n_lo; --n) {
@@ -1844,7 +1848,7 @@ extern "C" int vbcsr_chebyshev_backward(vbcsr_t *A, int64_t k, const double *R, 
                 epi.gamma = gm[n] * scale;
                 epi.Z = R;
                 epi.ldz = ldr;
-                rc = run_product(A, true, k, 2.0, cur, k, -1.0, nxt, k, &epi, precision, s);
+                rc = run_product(A, true, k, 2.0, cur, k, -1.0, nxt, k, &epi, precision, s, 1.0, nullptr, true, true);
                 if (rc) return rc;
                 std::swap(cur, nxt);
             }
@@ -1900,7 +1904,7 @@ extern "C" int vbcsr_kpm_moments(vbcsr_t *A, int64_t k, const double *R, int64_t
     epi.dot_out = moments + 1;                                             // mu_1 = <t_1, t_0>
     const FusedX fx0 = {nullptr, xs[1]};
     if ((rc = run_product(A, false, k, 1.0, R, ldr, 0.0, buf[1], k, &epi, precision, s, scale,
-                          xs[1] ? &fx0 : nullptr)))
+                          xs[1] ? &fx0 : nullptr, true, true)))
         return rc;
     CUDA_TRY(launch_copy_panel(N, k * cw, R, ldr * cw, buf[0], k * cw, s), "copy R");
     // t_n in buf[n & 1]; raw dots <t_n, t_n> -> moments[2n], <t_{n+1}, t_n> -> moments[2n+1]
@@ -1913,7 +1917,7 @@ extern "C" int vbcsr_kpm_moments(vbcsr_t *A, int64_t k, const double *R, int64_t
         epi.dot_out = moments + 2 * n + 1;
         const FusedX fx = {xs[n & 1], xs[(n + 1) & 1]};
         if ((rc = run_product(A, false, k, 2.0, tn, k, -1.0, tprev, k, &epi, precision, s, scale,
-                              xs[0] ? &fx : nullptr)))
+                              xs[0] ? &fx : nullptr, true, true)))
             return rc;
     }
     CUDA_TRY(launch_kpm_fixup(moments, M, s), "moment fix-up");

@@ -500,9 +500,10 @@ __global__ void __launch_bounds__(256, 2) fma_persistent_kernel(ProdArgs a) {
             it = (int64_t)__shfl_sync(0xffffffffu, q, 0);
         }
         if (it >= a.n_items) break;
-        WorkItem w = a.items[a.row_split > 1 ? it / a.row_split : it];
+        constexpr bool kSplit = sizeof(TV) == 8 && alignof(TV) == 8 && sizeof(TA) == 8 && alignof(TA) == 8;   // FP64
+        WorkItem w = a.items[kSplit && a.row_split > 1 ? it / a.row_split : it];
         const int kc = a.kc_of(w.B);
-        if (a.row_split > 1) {
+        if (kSplit && a.row_split > 1) {
             // rows [p0, p1) of the item: the same sums in the same order, more warps
             const int c = (int)(it % a.row_split), p0 = w.B * c / a.row_split, p1 = w.B * (c + 1) / a.row_split;
             if (TRANS) w.Kp += p0;

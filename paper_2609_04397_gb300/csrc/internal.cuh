@@ -158,15 +158,26 @@ struct SliceItem {
     int32_t strct;    // structure (of a batched operator) whose X columns the item reads
     int32_t pad;
 };
-// Stored entries x columns of a structure from which it is sliced. Below, the passes over X
-// and the launches cost more than the multiply-adds: at k >= 3 that is a few microseconds
-// (700 atoms, k = 8: 45 against 86 us; 200 atoms: 26 against 16). One and two columns leave
-// the multiply-add kernel closer to the memory: k = 1 on the 50k-atom operator (1.7e8
-// entries) 0.32 against 0.37 ms, on 20k disordered atoms (3.8e7) 0.128 against 0.111; k = 2
-// there 0.157 against 0.196, on 2500 atoms (7.6e6) 0.060 against 0.054.
-__host__ __device__ constexpr int64_t slice_min_work(int64_t k) {
-    return k == 1 ? (int64_t)1 << 26 : k == 2 ? (int64_t)1 << 25 : (int64_t)1 << 22;
+// Stored entries from which a structure is sliced in products of k columns. `repeated`:
+// one of many products with the same values (a recurrence). There slicing pays from 3
+// columns and 2^22 entries x columns on; below, the passes over X and the launches cost
+// more than the multiply-adds (6000 atoms, k = 3, moments and gradient: 4.4 against 7.3 ms;
+// 687 atoms, k = 4: 2.5 against 2.7). A caller's single product may follow new values,
+// which first have to be cut into digits (about 0.45 ms for 1.7e8 entries): it is sliced
+// from 5 columns on, where the multiply-adds run tiles of 8, and 2^24 entries x tile
+// columns. Values set and one product, sliced against multiply-adds: k = 3, 3.8e7
+// entries 536 against 493 us; k = 8, 1.1e6 entries 75 against 60, 3.3e6 entries 130
+// against 141, 1.7e8 entries 1.69 against 2.88 ms; k = 16, 1.1e6 entries 85 against 97.
+inline int64_t slice_min_nnz(int64_t k, bool repeated) {
+    if (k < (repeated ? 3 : 5)) return INT64_MAX;
+    if (repeated) return (((int64_t)1 << 22) + k - 1) / k;
+    int64_t kc = 8;
+    while (kc < k) kc *= 2;
+    return (((int64_t)1 << 24) + kc - 1) / kc;
 }
+// The pattern-sampled product cuts its operands on every call; it takes about 1.5 ms for
+// 1.7e8 entries up to 8 columns, where the multiply-adds take 0.1 + 0.28 k ms
+constexpr int64_t kSddmmMinCols = 6, kSddmmMinWork = (int64_t)1 << 22;
 struct SliceChunk {   // X rows of one structure
     int32_t row0, nrows, strct;
 };
@@ -178,6 +189,7 @@ struct SliceArgs {
     const uint32_t *cmax, *ccnt;  // [structures, ldp]: high word of the column maxima, tiny elements
     const int32_t *struct_rows;   // X rows of every structure
     const int64_t *struct_nnz;    // stored entries of every structure
+    int64_t min_nnz;              // slice_min_nnz of this product
     int ldp;                      // slice_ldp(k)
     int alpha_pow2, alpha_exp;    // alpha = 2^alpha_exp: goes into the result's exponent
 };
@@ -191,7 +203,6 @@ cudaError_t launch_slice_values(bool cplx, bool trans, const WorkItem *items, co
 const void *slice_kernel_ptr(bool trans, int64_t k);
 const void *slice_c128_kernel_ptr(bool trans, int64_t k);
 size_t slice_smem_bytes();
-constexpr int kSliceThin = 3;         // widest product with the digits of X on the N side
 int slice_ldp(int64_t k);             // columns of the fixed-point X
 
 // Scalar (all 1 x 1 blocks) operators: L lanes per row (2, 4 or 8 for the

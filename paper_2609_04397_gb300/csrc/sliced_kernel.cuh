@@ -280,145 +280,14 @@ __device__ __forceinline__ bool slice_pass(const ProdArgs &a, const SliceArgs &q
     return true;
 }
 
-// Products of KC <= kSliceThin columns: the digits of X, not its columns, are the
-// N side (8 of them a tile, 7 used, one tile a column), so an MMA forms digit i of
-// the values times all digits of a column at once: 7 KC MMAs a step instead of 35.
-// Every digit pair has an accumulator of its own, so nothing is dropped and the
-// sums over up to kSliceKMax columns are exact without carries. X is [rows, KC].
-// Bound by reading the value tiles (7 bytes an entry) and cutting them into f16
-// pairs. 50k atoms, k = 1 / 2 / 3: 0.32 / 0.43 / 0.56 ms, multiply-adds 0.37 / 0.73 / 1.26.
-template <bool TRANS, int KC, int NR>
-__device__ __forceinline__ bool slice_thin(const ProdArgs &a, const SliceArgs &q, const WorkItem &w,
-                                           const unsigned char *vsrc, int nsteps, const uint32_t *cmax,
-                                           unsigned char *ring, const int32_t *s_x, int lane, double &dot) {
-    constexpr int S = kSliceStages, kStage = 16 * kSliceTile;
-    const int g = lane >> 2, t4 = lane & 3;
-    float acc[kSliceDigits][KC][4], low[KC][4];
-#pragma unroll
-    for (int n = 0; n < KC; ++n)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            low[n][j] = 0.f;
-#pragma unroll
-            for (int i = 0; i < kSliceDigits; ++i) acc[i][n][j] = 0.f;
-        }
-    if (nsteps > 0) {
-        const int tile = w.B * kSliceTile;
-        constexpr int kChunks = (16 * kSliceTile / 16 + 31) / 32;
-        bool mine[kChunks];
-#pragma unroll
-        for (int u = 0; u < kChunks; ++u) mine[u] = 16 * (lane + 32 * u) < tile;
-        const unsigned char *src = vsrc + 16 * lane;
-        auto issue = [&](int s) {
-            const bool in = s < nsteps;
-            unsigned char *dst = ring + (s % S) * kStage + 16 * lane;
-#pragma unroll
-            for (int u = 0; u < kChunks; ++u)
-                if (in && mine[u]) cp_async16(dst + 512 * u, src + 512 * u);
-            src += tile;
-            asm volatile("cp.async.commit_group;" ::: "memory");
-        };
-        // digit g of the lane's four virtual columns: byte 6 - g (the eighth digit is zero)
-        const uint8_t *xd = reinterpret_cast<const uint8_t *>(q.xdig) + (g < 7 ? 6 - g : 0);
-        uint32_t x[KC][4];
-        auto load_x = [&](int s) {
-            const int4 xi = *reinterpret_cast<const int4 *>(s_x + 16 * s + 4 * t4);
-            const int row[4] = {xi.x, xi.y, xi.z, xi.w};
-#pragma unroll
-            for (int r = 0; r < 4; ++r)
-#pragma unroll
-                for (int n = 0; n < KC; ++n) x[n][r] = __ldg(xd + ((int64_t)row[r] * KC + n) * 8);
-        };
-        load_x(0);
-#pragma unroll
-        for (int s = 0; s < S - 1; ++s) issue(s);
-        const int digit = w.B * 16;
-        for (int s = 0; s < nsteps; ++s) {
-            asm volatile("cp.async.wait_group %0;" ::"n"(S - 2) : "memory");
-            __syncwarp();
-            issue(s + S - 1);
-            uint32_t b[KC][2];
-#pragma unroll
-            for (int n = 0; n < KC; ++n)
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    // 0x6400 | byte is 1024 + byte in f16; less 1152
-                    uint32_t p = (x[n][2 * h] + (x[n][2 * h + 1] << 16)) | 0x64006400u;
-                    asm("sub.f16x2 %0, %0, %1;" : "+r"(p) : "r"(0x64806480u));
-                    b[n][h] = g < 7 ? p : 0u;
-                }
-            load_x(s + 1);
-            const unsigned char *st = ring + (s % S) * kStage + g * 16 + t4 * 4;
-#pragma unroll
-            for (int i = 0; i < kSliceDigits; ++i, st += digit) {
-                uint32_t v[NR][2];
-#pragma unroll
-                for (int n = 0; n < NR; ++n) {
-                    const uint32_t word = *reinterpret_cast<const uint32_t *>(st + 128 * n);
-                    v[n][0] = slice_half2(word, 0x4140);
-                    v[n][1] = slice_half2(word, 0x4342);
-                }
-                const uint32_t rows[4] = {v[0][0], v[NR - 1][0], v[0][1], v[NR - 1][1]};
-#pragma unroll
-                for (int n = 0; n < KC; ++n) mma_f16(acc[i][n], rows, b[n][0], b[n][1]);
-                if (i == 0) {   // magnitudes of the leading digits (column 0 of the tile)
-                    constexpr uint32_t kAbs = 0x7fff7fffu;
-                    const uint32_t r[4] = {rows[0] & kAbs, rows[1] & kAbs, rows[2] & kAbs, rows[3] & kAbs};
-#pragma unroll
-                    for (int n = 0; n < KC; ++n) mma_f16(low[n], r, b[n][0] & kAbs, b[n][1] & kAbs);
-                }
-            }
-        }
-        asm volatile("cp.async.wait_all;" ::: "memory");
-        __syncwarp();
-    }
-    // accumulator 2 h + e: row g + 8 h, digit 2 t4 + e of X. Lanes t4 = 0 hold digit 0 and write.
-    int er[2], ec[KC];
-    bool ok = true;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) er[h] = g + 8 * h < w.B ? q.rexp[w.yrow + g + 8 * h] : 0;
-#pragma unroll
-    for (int n = 0; n < KC; ++n) {
-        const uint32_t M = cmax[n];
-        ec[n] = M ? slice_exp(M) : 0;
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-            ok &= er[h] >= 0 && (er[h] == 0 || ec[n] == 0 || t4 != 0 || low[n][2 * h] >= kSliceGuard);
-    }
-    if (!__all_sync(0xffffffffu, ok)) return false;
-#pragma unroll
-    for (int h = 0; h < NR; ++h) {
-        const int r = g + 8 * h;
-#pragma unroll
-        for (int n = 0; n < KC; ++n) {
-            float t[2][8];
-#pragma unroll
-            for (int e = 0; e < 2; ++e)
-#pragma unroll
-                for (int i = 0; i < kSliceDigits; ++i) t[e][i] = acc[i][n][2 * h + e];
-            double o = slice_value_of_lanes(t, t4, er[h] + ec[n] - 2114 + q.alpha_exp);
-            if (t4 == 0 && r < w.B) {
-                const int64_t row = w.yrow + r;
-                double *y = static_cast<double *>(a.Y) + row * a.ldy + n;
-                if (!q.alpha_pow2) o *= a.alpha;
-                if (a.beta_nz) o += a.beta * *y;
-                if (a.gamma_nz) o += a.gamma * static_cast<const double *>(a.Z)[row * a.ldz + n];
-                *y = o;
-                if (a.item_partials) dot += static_cast<const double *>(a.R)[row * a.ldr + n] * o;
-            }
-        }
-    }
-    return true;
-}
-
-// One warp per work item (up to 16 output rows). FORM 0: k > 8, passes of 16
-// columns with a last one of 8 where that is enough; 8: one pass of up to 8
-// columns; 1 .. kSliceThin: that many columns.
+// One warp per work item (up to 16 output rows). WIDE: k > 8, passes of 16
+// columns with a last one of 8 where that is enough; otherwise one pass of up to 8
+// columns.
 // Complex operators (T = double2, TA its arithmetic): the kernel sees two real
 // columns a complex one and two virtual columns a complex value, re meeting the
 // X row x and im the row i x (slice_panel_kernel).
-template <bool TRANS, int FORM, typename T, typename TA>
-__global__ void __launch_bounds__(128, FORM == 0 || FORM == 3 ? 3 : FORM == 1 ? 5 : 4) slice_product_kernel(ProdArgs a, SliceArgs q) {
+template <bool TRANS, bool WIDE, typename T, typename TA>
+__global__ void __launch_bounds__(128, WIDE ? 3 : 4) slice_product_kernel(ProdArgs a, SliceArgs q) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int kRing = kSliceStages * 16 * kSliceTile;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -444,7 +313,7 @@ __global__ void __launch_bounds__(128, FORM == 0 || FORM == 3 ? 3 : FORM == 1 ? 
             // a small structure, or one with a column outside the sliced range or mostly tiny, is not sliced
             last_strct = si.strct;
             const uint32_t most = (uint32_t)q.struct_rows[si.strct] >> 2;
-            bool p = q.struct_nnz[si.strct] * a.k < slice_min_work(a.k);
+            bool p = q.struct_nnz[si.strct] < q.min_nnz;
             for (int c = lane; c < (int)a.k; c += 32)
                 p |= !slice_exp_ok(cmax[c]) || q.ccnt[(int64_t)si.strct * q.ldp + c] > most;
             last_plain = __any_sync(0xffffffffu, p);
@@ -470,25 +339,18 @@ __global__ void __launch_bounds__(128, FORM == 0 || FORM == 3 ? 3 : FORM == 1 ? 
         }
         if (!plain) {
             bool ok = true;
-            if constexpr (FORM == 0)
+            if constexpr (WIDE)
                 for (; ok && n0 + 8 < a.k; n0 += ok ? 16 : 0)
                     ok = w.B <= 8 ? slice_pass<TRANS, true, 1>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot)
                          : w.B == 9
                              ? slice_pass<TRANS, true, 1, true>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot)
                              : slice_pass<TRANS, true, 2>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot);
-            if constexpr (FORM == 0 || FORM == 8) {
-                if (ok && n0 < a.k) {
-                    ok = w.B <= 8
-                             ? slice_pass<TRANS, false, 1>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot)
-                         : w.B == 9
-                             ? slice_pass<TRANS, false, 1, true>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot)
-                             : slice_pass<TRANS, false, 2>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot);
-                    n0 += ok ? 8 : 0;
-                }
-            } else {
-                ok = w.B <= 8 ? slice_thin<TRANS, FORM, 1>(a, q, w, vsrc, nsteps, cmax, ring, s_x, lane, dot)
-                              : slice_thin<TRANS, FORM, 2>(a, q, w, vsrc, nsteps, cmax, ring, s_x, lane, dot);
-                n0 = ok ? FORM : 0;
+            if (ok && n0 < a.k) {
+                ok = w.B <= 8 ? slice_pass<TRANS, false, 1>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot)
+                     : w.B == 9
+                         ? slice_pass<TRANS, false, 1, true>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot)
+                         : slice_pass<TRANS, false, 2>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot);
+                n0 += ok ? 8 : 0;
             }
         }
         if (n0 < a.k) {
@@ -510,12 +372,7 @@ __global__ void __launch_bounds__(128, FORM == 0 || FORM == 3 ? 3 : FORM == 1 ? 
 using SliceKernel = void (*)(ProdArgs, SliceArgs);
 template <bool TRANS, typename T, typename TA>
 SliceKernel slice_kernel(int64_t k) {
-    switch (k) {
-        case 1: return slice_product_kernel<TRANS, 1, T, TA>;
-        case 2: return slice_product_kernel<TRANS, 2, T, TA>;
-        case 3: return slice_product_kernel<TRANS, 3, T, TA>;
-        default: return k <= 8 ? slice_product_kernel<TRANS, 8, T, TA> : slice_product_kernel<TRANS, 0, T, TA>;
-    }
+    return k <= 8 ? slice_product_kernel<TRANS, false, T, TA> : slice_product_kernel<TRANS, true, T, TA>;
 }
 
 template <typename T, typename TA>

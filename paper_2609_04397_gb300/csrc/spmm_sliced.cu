@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(128) slice_values_kernel(const WorkItem *items
 
 }  // namespace
 
-int slice_ldp(int64_t k) { return k <= kSliceThin ? (int)k : (int)((k + 7) / 8 * 8); }
+int slice_ldp(int64_t k) { return (int)((k + 7) / 8 * 8); }
 
 size_t slice_smem_bytes() { return kSliceSmem; }
 

@@ -66,7 +66,7 @@ def test_sliced_products_against_oracle(sizes, n, density, k):
     vals = syn.random_values(pat, k)
     H = _handle(pat, vals)
     rng = np.random.default_rng(k)
-    wide = max(k, -(-(1 << 22) // pat.nnz) + 1)        # columns from which this operator is sliced
+    wide = max(k, -(-(1 << 24) // pat.nnz) + 1)        # columns from which this operator is sliced
     for cols in sorted({k, wide}):
         X = rng.standard_normal((pat.n_cols, cols))
         Y0 = rng.standard_normal((pat.n_rows, cols))
@@ -94,12 +94,13 @@ def test_exact_level_sums_at_the_widest_row():
             assert (got - exact).abs().max().item() <= 4e-16 * abs(exact)
 
 
-@pytest.mark.parametrize("k", [7, 8, 16, 19])   # from 7 columns on, an operator of this size is sliced
+@pytest.mark.parametrize("k", [7, 8, 16, 19])
 def test_items_of_nine_rows(k):
     """The ninth row's digits are the N side of its own products: the largest digit sums of
     765 columns, and ninth rows that are zero, far smaller than the others or unresolved."""
     b = 9
-    pat = BlockPattern(np.full(90, b), np.full(85, b), np.arange(91) * 85, np.tile(np.arange(85), 90))
+    nr = 310
+    pat = BlockPattern(np.full(nr, b), np.full(85, b), np.arange(nr + 1) * 85, np.tile(np.arange(85), nr))
     h = float(0x7D808080808080 - 0x01010101010100) * 2.0 ** -54
     H = _handle(pat, np.full(pat.nnz, h))
     X = torch.full((765, k), -h, dtype=torch.float64, device="cuda:0")
@@ -109,7 +110,7 @@ def test_items_of_nine_rows(k):
     assert (got - exact).abs().max().item() <= 4e-16 * abs(exact)
     assert any("slice_product" in n for n in _kernels(lambda: H.spmm(X)))
     rng = np.random.default_rng(k)
-    vals = rng.standard_normal(pat.nnz).reshape(90, 85, b, b)   # blocks of a block row are b x b
+    vals = rng.standard_normal(pat.nnz).reshape(nr, 85, b, b)   # blocks of a block row are b x b
     vals[0, :, 8] = 0.0
     vals[1, :, 8] *= 1e-200
     vals[2, :, 8, :] = 0.0
@@ -119,17 +120,18 @@ def test_items_of_nine_rows(k):
     X = rng.standard_normal((765, k))
     X[:40, k // 2] = 0.0
     H = _handle(pat, vals)
-    Y0 = rng.standard_normal((810, k))
+    Y0 = rng.standard_normal((nr * b, k))
     _check(H, pat, vals, X, alpha=0.3, beta=2.0, Y0=Y0)
-    _check(H, pat, vals, rng.standard_normal((810, k)), transpose=True)
+    _check(H, pat, vals, rng.standard_normal((nr * b, k)), transpose=True)
 
 
 def test_unresolved_outputs_take_multiply_adds():
     """Graded rows and columns, zero rows and columns, panels supported on a few
     rows, tiny and huge magnitudes, Inf and NaN: every output as accurate as the
     multiply-add chain's, and NaN and Inf only where they belong."""
-    pat = _pattern((4, 9, 13), 90, 0.3, 5)
+    pat = _pattern((4, 9, 13), 260, 0.25, 5)
     rng = np.random.default_rng(0)
+    assert 32 * pat.nnz >= 1 << 24   # sliced
     vals = syn.random_values(pat, 5)
     k = 24
     X = rng.standard_normal((pat.n_cols, k))
@@ -259,7 +261,7 @@ def test_captured_products_outlive_larger_ones():
     assert torch.equal(Yg, Y) and torch.equal(Dg, D)
 
 
-@pytest.mark.parametrize("k", [3, 7, 16, 17, 40, 200])
+@pytest.mark.parametrize("k", [6, 7, 16, 17, 40, 200])
 def test_sliced_sddmm_against_oracle(k):
     """The pattern-sampled product, contracting over the panel columns: row heights 1 to 33,
     rows wider than the 512-column window, ragged tiles, leading dimensions above k, graded
@@ -294,31 +296,37 @@ def test_sliced_sddmm_against_oracle(k):
                                                                     torch.from_numpy(B0).cuda()[:, :k])))
 
 
-def test_thin_sliced_products():
-    """One to three columns (the digits of X on the N side), forward and adjoint: every
-    row height of a random pattern at three columns, the sizes from which one and two
-    columns are sliced on a nanoparticle, outputs that are not resolved, an exact sum."""
-    pat = syn.random_pattern(330, 325, (1, 2, 4, 9, 13, 16, 33), 0.13, 3, empty_rows=2, unsorted=True)
-    assert 3 * pat.nnz >= 1 << 22
+def test_fewest_columns():
+    """Five columns, forward and adjoint, over every row height of a random pattern, with
+    outputs that are not resolved; four are sliced in a recurrence only, two never."""
+    pat = syn.random_pattern(430, 425, (1, 2, 4, 9, 13, 16, 33), 0.13, 3, empty_rows=2, unsorted=True)
+    assert 8 * pat.nnz >= 1 << 24
     vals = syn.random_values(pat, 3)
     H = _handle(pat, vals)
     rng = np.random.default_rng(3)
-    X = rng.standard_normal((pat.n_cols, 3))
-    _check(H, pat, vals, X, alpha=-0.3, beta=2.0, Y0=rng.standard_normal((pat.n_rows, 3)))
-    _check(H, pat, vals, rng.standard_normal((pat.n_rows, 3)), transpose=True)
+    X = rng.standard_normal((pat.n_cols, 5))
+    _check(H, pat, vals, X, alpha=-0.3, beta=2.0, Y0=rng.standard_normal((pat.n_rows, 5)))
+    _check(H, pat, vals, rng.standard_normal((pat.n_rows, 5)), transpose=True)
     assert any("slice_product" in n for n in _kernels(lambda: H.spmm(torch.from_numpy(X).cuda())))
+    assert not any("slice" in n for n in _kernels(lambda: H.spmm(torch.from_numpy(X[:, :4].copy()).cuda())))
     X[:, 1] *= np.exp(-np.arange(pat.n_cols) / 50.0)
     X[9, 0] = np.inf
     with np.errstate(invalid="ignore"):
         _check(H, pat, vals, X)
-    w = syn.zincblende(21_000)
-    assert w.pattern.nnz >= 1 << 26
+    w = syn.amorphous(700, side=60.0 * (700 / 20000) ** (1 / 3))
     H = _handle(w.pattern, w.values)
-    for k in (1, 2):
-        X = rng.standard_normal((w.pattern.n_cols, k))
-        _check(H, w.pattern, w.values, X)
-        _check(H, w.pattern, w.values, X, transpose=True)
-        assert any("slice_product" in n for n in _kernels(lambda: H.spmm(torch.from_numpy(X).cuda())))
+    lo, hi = H.gershgorin()
+    H.shift_scale((lo + hi) / 2, 0.51 * (hi - lo))
+    for k in (2, 3, 4):
+        R = torch.randn(w.pattern.n_rows, k, dtype=torch.float64, device="cuda:0")
+        sliced = any("slice_product" in n for n in _kernels(lambda: H.chebyshev(R, 5)))
+        assert sliced == (k * w.pattern.nnz >= 1 << 22 and k > 2)
+        mu, _ = H.chebyshev(R, 5)
+        t = [R, H.spmm(R)]
+        for _ in range(3):
+            t.append(2.0 * H.spmm(t[-1]) - t[-2])
+        ref = torch.stack([(R * x).sum() for x in t]) / R.numel()
+        assert (mu - ref).abs().max().item() <= 1e-13 * ref[0].abs().item()
 
 
 @pytest.mark.parametrize("k", [1, 3, 8, 13])
