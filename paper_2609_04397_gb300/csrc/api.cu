@@ -88,8 +88,8 @@ struct SlicePlan {
     SliceItem *items = nullptr;     // parallel to the cost-ordered work items
     SliceChunk *chunks = nullptr;   // X rows, cut at the structures
     int32_t *struct_rows = nullptr; // X rows of every structure
-    int64_t *struct_nnz = nullptr;  // stored entries of every structure
-    int64_t max_nnz = 0;            // of the largest structure
+    int64_t *struct_nnz = nullptr;  // stored entries of every structure, 0 where its items are too small: [2][structures]
+    int64_t max_nnz[2] = {0, 0};    // of the largest structure (kSliceItemNnz[0], [1])
     uint8_t *vdig = nullptr;        // value tiles, built on first use
     int32_t *rexp = nullptr;        // scale exponent of every output row
     bool no_room = false;           // an allocation failed: keep to the multiply-add kernels
@@ -322,7 +322,8 @@ static int plan_slices(vbcsr_matrix *A, SlicePlan *p, const std::vector<WorkItem
     if (A->dtype == VBCSR_F32 || A->backend == VBCSR_BACKEND_CSR || items.empty() || A->nblk == 0) return VBCSR_OK;
     const int cw = A->dtype == VBCSR_C128 ? 2 : 1;   // real virtual columns and X rows a complex one
     std::vector<SliceItem> si(items.size());
-    std::vector<int64_t> nnz(out_start.size() - 1, 0);
+    const size_t n_str = out_start.size() - 1;
+    std::vector<int64_t> nnz(2 * n_str, 0), n_items(n_str, 0);
     int64_t pos = 0;
     double wide = 0.0, all = 0.0;
     for (size_t t = 0; t < items.size(); ++t) {
@@ -332,6 +333,7 @@ static int plan_slices(vbcsr_matrix *A, SlicePlan *p, const std::vector<WorkItem
         si[t].strct = (int32_t)(std::upper_bound(out_start.begin(), out_start.end() - 1, w.yrow) - out_start.begin() - 1);
         all += (double)w.B * w.K;
         nnz[si[t].strct] += (int64_t)w.B * w.K * cw;
+        ++n_items[si[t].strct];
         if (cw * w.K > kSliceKMax) {
             wide += (double)w.B * w.K;
             continue;
@@ -351,12 +353,17 @@ static int plan_slices(vbcsr_matrix *A, SlicePlan *p, const std::vector<WorkItem
             ch.push_back({(int32_t)r, (int32_t)std::min<int64_t>(kSliceChunkRows, in_start[t + 1] - r), (int32_t)t});
     }
     p->n_chunks = (int64_t)ch.size();
+    for (size_t t = 0; t < n_str; ++t)
+        for (int h = 1; h >= 0; --h) {
+            nnz[h * n_str + t] = nnz[t] >= kSliceItemNnz[h] * n_items[t] ? nnz[t] : 0;
+            p->max_nnz[h] = std::max(p->max_nnz[h], nnz[h * n_str + t]);
+        }
+    if (p->max_nnz[1] == 0) return VBCSR_OK;
+    p->applies = true;
     CUDA_TRY(upload(A, &p->items, si, s), "upload sliced items");
     CUDA_TRY(upload(A, &p->chunks, ch, s), "upload");
     CUDA_TRY(upload(A, &p->struct_rows, rows, s), "upload");
     CUDA_TRY(upload(A, &p->struct_nnz, nnz, s), "upload");
-    p->max_nnz = *std::max_element(nnz.begin(), nnz.end());
-    p->applies = true;
     return VBCSR_OK;
 }
 
@@ -972,8 +979,8 @@ static int slices_changed(vbcsr_t *A, cudaStream_t s) {
 // True when a native FP64 product of k columns runs sliced.
 static bool slice_applies(const vbcsr_t *A, bool trans, int64_t k, bool repeated) {
     const SlicePlan &p = A->slice[trans];
-    return p.applies && !p.untracked && k <= (1 << 20) && p.max_nnz >= slice_min_nnz(k, repeated) &&
-           !A->debug_checks;
+    return p.applies && !p.untracked && k <= (1 << 20) &&
+           p.max_nnz[slice_small_items(k, repeated)] >= slice_min_nnz(k, repeated) && !A->debug_checks;
 }
 
 // k counts real columns here and below (two a column of a complex operator)
@@ -1496,7 +1503,7 @@ static int run_product(vbcsr_t *A, bool trans, int64_t k, double alpha, const vo
         sa.cmax = cmax;
         sa.ccnt = ccnt;
         sa.struct_rows = p.struct_rows;
-        sa.struct_nnz = p.struct_nnz;
+        sa.struct_nnz = p.struct_nnz + (slice_small_items(kr, repeated) ? A->n_structs : 0);
         sa.min_nnz = slice_min_nnz(kr, repeated);
         sa.ldp = xld;
         int ae = 0;
@@ -1637,7 +1644,8 @@ static SddmmArgs sddmm_args(vbcsr_t *A) {
 // widths whose level sums stay exact; else by multiply-adds, as on a stream that is
 // being captured before the buffers exist.
 static int run_sddmm_f64(vbcsr_t *A, const SddmmArgs &a, cudaStream_t s) {
-    bool sliced = a.k >= kSddmmMinCols && a.k <= kSliceKMax && a.alpha != 0.0 && A->nnz * a.k >= kSddmmMinWork && !A->debug_checks;
+    bool sliced = a.k >= kSddmmMinCols && a.k <= kSliceKMax && a.alpha != 0.0 && A->nnz * a.k >= kSddmmMinWork &&
+                  A->nnz >= (a.k < 16 ? kSddmmItemNnz : kSliceItemNnz[1]) * A->n_fwd_items && !A->debug_checks;
     if (sliced) {
         const int64_t kp = (a.k + 15) / 16 * 16, rows = A->n_rows + A->n_cols;
         const size_t need = (size_t)(rows * kp + (rows + 1) / 2);

@@ -175,6 +175,20 @@ inline int64_t slice_min_nnz(int64_t k, bool repeated) {
     while (kc < k) kc *= 2;
     return (((int64_t)1 << 24) + kc - 1) / kc;
 }
+// Entries a work item has on average from which a structure is sliced: [1] in recurrences
+// and from 9 columns on, [0] in single products of up to 8. Items of fewer waste the MMA's
+// rows and spend their time on starting and ending. Multiply-adds against sliced at k = 8,
+// product alone / after new values: 108 entries (b = 2, 27 blocks) 429 / 1023 against 399 /
+// 1233 us, 96 (b = 4, 6 blocks) 258 / 372 against 236 / 472, 243 (b = 3) 291 / 553 against
+// 206 / 613, 432 (b = 4) 417 / 686 against 227 / 696, 845 (b = 13, 5 blocks) 608 / 731
+// against 191 / 493; at k = 16, 28 entries (b = 2, 7 blocks) 288 against 478, 225 (b = 5, 9
+// blocks) 453 / 565 against 265 / 502.
+constexpr int64_t kSliceItemNnz[2] = {400, 200};
+inline int slice_small_items(int64_t k, bool repeated) { return repeated || k > 8 ? 1 : 0; }
+// The pattern-sampled product's, below 16 columns: 503 entries (b = 1 and 9) 518 against
+// 589 us at k = 8, 845 708 against 449; from 16 on kSliceItemNnz[1]: 243 entries 537
+// against 467 us, 108 entries 602 against 838
+constexpr int64_t kSddmmItemNnz = 800;
 // The pattern-sampled product cuts its operands on every call; it takes about 1.5 ms for
 // 1.7e8 entries up to 8 columns, where the multiply-adds take 0.1 + 0.28 k ms
 constexpr int64_t kSddmmMinCols = 6, kSddmmMinWork = (int64_t)1 << 22;

@@ -69,8 +69,9 @@ __device__ __noinline__ void fma_columns(const ProdArgs &a, int64_t n0, const Wo
 // side, half of it padding). NINTH: items of 9 rows (an sp3d5 basis), the ninth
 // alone with its digits as the N side, one more MMA per digit of X (PAIR: per two)
 // instead of another group of 8 rows: 44 MMAs a wide step instead of 72, 25 a
-// narrow one instead of 36 (50k zinc-blende atoms, k = 32: 1.43 ms against 1.56). Returns false, with nothing written, when an output
-// is not resolved by the fixed point.
+// narrow one instead of 36 (50k zinc-blende atoms, k = 32: 1.43 ms against 1.56).
+// Returns false, with nothing written, when an output is not resolved by the
+// fixed point.
 template <bool TRANS, bool WIDE, int NR, bool NINTH = false>
 __device__ __forceinline__ bool slice_pass(const ProdArgs &a, const SliceArgs &q, const WorkItem &w,
                                            const unsigned char *vsrc, int nsteps, int64_t n0, const uint32_t *cmax,

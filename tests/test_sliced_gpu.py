@@ -329,6 +329,20 @@ def test_fewest_columns():
         assert (mu - ref).abs().max().item() <= 1e-13 * ref[0].abs().item()
 
 
+def test_small_items_are_not_sliced():
+    """2 x 2 blocks, 40 a row: 160 entries a work item, too few for the digit products."""
+    n = 14_000
+    cols = np.sort((np.arange(n)[:, None] + 3 * np.arange(40)) % n, axis=1)
+    pat = BlockPattern(np.full(n, 2), np.full(n, 2), np.arange(n + 1) * 40, cols.reshape(-1))
+    assert 8 * pat.nnz >= 1 << 24
+    vals = syn.random_values(pat, 1)
+    H = _handle(pat, vals)
+    X = np.random.default_rng(1).standard_normal((pat.n_cols, 8))
+    _check(H, pat, vals, X)
+    Xd = torch.from_numpy(X).cuda()
+    assert not any("slice" in k for k in _kernels(lambda: (H.spmm(Xd), H.spmm_adjoint(Xd), H.sddmm(Xd, Xd))))
+
+
 @pytest.mark.parametrize("k", [1, 3, 8, 13])
 def test_sliced_complex_products(k):
     """A complex operator as two real virtual columns a value, forward and
