@@ -8,8 +8,9 @@ synthetic, shifted and scaled on the GPU to H~ = (H - c) / d with its spectrum
 inside [-1, 1] (Gershgorin bounds). One step is one step of the Chebyshev
 recurrence of the kernel polynomial method (Sec. V) on 16 Rademacher vectors:
 t_{n+1} = 2 H~ t_n - t_{n-1} with the moment <R, t_{n+1}> fused into the
-product's epilogue, FP64 block products. The values (27.5 GB) are far larger
-than the 129 MB L2, so no flush is needed.
+product's epilogue, FP64 block products (exact digit products on the FP16
+tensor cores, one FP64 rounding an output). The values (27.5 GB, 24 GB as
+digits) are far larger than the 129 MB L2, so no flush is needed.
 
 `value` is GFLOP/s = 2 * nnz * k per step over the device-timed steps, summed
 over ranks (replicas) with the max time. `mixed` times the full 50-step
@@ -73,20 +74,23 @@ def _peaks():
 
 
 # FP64 ALU peak from unit counts and clock: 152 SMs x 2 FP64 FMA per clock x
-# 2 flop x 2.07 GHz (the nominal 1.25 TFLOP/s); the self-written DFMA probe
-# measured 1.19 TFLOP/s on this machine's GB300.
+# 2 flop x 2.07 GHz (the nominal 1.25 TFLOP/s). The products on the tensor
+# cores go beyond it: `fp64_alu_frac` is their rate over that of FP64 FMAs.
 FP64_SMS, FP64_FMA_PER_CLK, SM_MAX_GHZ = 152, 2, 2.07
 FP64_PEAK_TFLOPS = FP64_SMS * FP64_FMA_PER_CLK * 2 * SM_MAX_GHZ / 1e3
-FP64_PROBE_TFLOPS = 1.19
+# multiply-adds a clock and SM of mma.sync m16n8k16 with FP16 operands and FP32
+# accumulators (self-written probe)
+MMA_F16_MAC_PER_CLK = 955
 
 
 # DRAM bytes (read + write) per stored entry of one FP64 Chebyshev step
-# (k = 16): ncu's dram__bytes_read.sum + dram__bytes_write.sum of the FP64
-# forward product with the recurrence epilogue on the ~100k-atom nanoparticle
-# (3.770 GB per launch, mean of two launches, 336,743,405 entries), scaled by
-# the stored entries to the headline operator (values, X, Y and R all grow
-# with the atom count). The summary is under profiles/.
-TRAFFIC_F64_PER_ENTRY = 11.197
+# (k = 16): ncu's dram__bytes_read.sum + dram__bytes_write.sum of the sliced
+# product with the recurrence epilogue (3.381 GB) and of the two passes over
+# t_n before it (0.141 and 0.234 GB) on the ~100k-atom nanoparticle
+# (336,743,405 entries), scaled by the stored entries to the headline operator
+# (values, X, Y and R all grow with the atom count). The summary is under
+# profiles/.
+TRAFFIC_F64_PER_ENTRY = 11.154
 
 
 def _workload(n_atoms=N_ATOMS):
@@ -115,6 +119,18 @@ def _alg_bytes(pat, k, value_bytes=8):
     indices and row pointers once, X read once, Y written once."""
     return (value_bytes * pat.nnz + 4 * pat.nblk + 8 * (pat.n_brows + 1)
             + 8 * k * (pat.n_cols + pat.n_rows))
+
+
+def _sliced_mmas(pat, k):
+    """m16n8k16 products of one sliced FP64 product of k > 8 columns: per work
+    item of up to 16 rows, per 16 stored columns of its block row and per 16
+    columns of X, 36 for up to 8 rows, 44 for 9, 72 above."""
+    width = np.add.reduceat(np.asarray(pat.col_bsize, np.int64)[pat.block_col_idx], pat.block_row_ptr[:-1])
+    width[np.diff(pat.block_row_ptr) == 0] = 0
+    b = np.asarray(pat.row_bsize, np.int64)
+    per = lambda h: np.select([h <= 0, h <= 8, h == 9], [0, 36, 44], 72)
+    mmas = (b // 16) * 72 + per(b % 16)
+    return int(np.sum((width + 15) // 16 * mmas) * ((k + 15) // 16))
 
 
 class ClockSampler:
@@ -697,11 +713,13 @@ def run_ours(args):
     N = pat.n_rows
     R = torch.from_numpy(syn.rademacher_panel(N, k, 0)).to(dev)
     flops_step = 2.0 * pat.nnz * k
-    # launches of one step: the product, then the dot's fixed-order sum (one launch up to
-    # 16384 work items, a chunk pass and a final pass beyond); a work item is up to 16
-    # rows of one block row
+    # launches of one step: the column maxima and the fixed-point form of t_n (operators of
+    # at least 2^24 entries x columns), the product, then the dot's fixed-order sum (one
+    # launch up to 16384 work items, a chunk pass and a final pass beyond); a work item is
+    # up to 16 rows of one block row
     n_items = int(np.sum((np.asarray(pat.row_bsize, np.int64) + 15) // 16))
-    launches_step = 1 + (2 if n_items > 16384 else 1)
+    sliced = pat.nnz * k >= 1 << 24
+    launches_step = (3 if sliced else 1) + (2 if n_items > 16384 else 1)
     n_warm = max(3, args.warmup)
     mu = torch.zeros(n_warm + args.steps + 2, dtype=torch.float64, device=dev)
 
@@ -743,17 +761,20 @@ def run_ours(args):
                                     dist if world > 1 else None)
     step_ms = sum(a.elapsed_time(b) for a, b in ev) / args.steps
     by_step = _step_bytes(pat, k, "native")
-    roofline = {"bound": "alu", "achieved": flops_step / step_ms / 1e9, "peak": FP64_PEAK_TFLOPS,
-                "unit": "TFLOP/s", "frac": flops_step / step_ms / 1e9 / FP64_PEAK_TFLOPS,
+    mma_tflops = 2 * 2048.0 * _sliced_mmas(pat, k) / step_ms / 1e9 if sliced else 0.0
+    mma_peak = 2e-3 * MMA_F16_MAC_PER_CLK * FP64_SMS * SM_MAX_GHZ
+    roofline = {"bound": "hbm", "achieved": by_step / step_ms / 1e6, "peak": hbm_peak,
+                "unit": "GB/s", "frac": by_step / step_ms / 1e6 / hbm_peak, "peak_source": peak_src,
                 "traffic": int(TRAFFIC_F64_PER_ENTRY * pat.nnz),
                 "traffic_source": "ncu DRAM bytes per stored entry on the ~100k-atom operator, scaled by the entries",
                 "algorithmic_bytes": by_step,
-                "kernel": "fma_persistent_kernel<false, double, double, double, double> (FP64 forward product "
-                          f"with the recurrence epilogue), k = {k}",
-                "frac_of_dfma_probe": flops_step / step_ms / 1e9 / FP64_PROBE_TFLOPS,
-                "peak_source": "unit counts x clock (152 SM x 2 FP64 FMA/clk x 2.07 GHz)",
-                "hbm_gbs": by_step / step_ms / 1e6, "hbm_frac": by_step / step_ms / 1e6 / hbm_peak,
-                "hbm_peak": hbm_peak, "hbm_peak_source": peak_src}
+                "kernel": "slice_product_kernel<false, true, double, double> (FP64 forward product on the FP16 tensor "
+                          f"cores, with the recurrence epilogue), k = {k}",
+                "tensor": {"achieved": mma_tflops, "peak": mma_peak, "unit": "FP16 TFLOP/s of mma.sync",
+                           "frac": mma_tflops / mma_peak,
+                           "peak_source": "self-written mma.sync m16n8k16 probe: 955 multiply-adds a clock and SM"},
+                "fp64_tflops": flops_step / step_ms / 1e9,
+                "vs_fp64_alu_peak": flops_step / step_ms / 1e9 / FP64_PEAK_TFLOPS}
 
     # ---- the full 50-step recurrence in FP64 and in each reduced-precision form ----
     mixed = {}

@@ -78,7 +78,8 @@ typedef enum {
  *          complex) run these rows on the tensor cores, from 2^24 stored
  *          entries x columns per structure and 5 columns on, inside a
  *          recurrence from 2^22 and 3 (a complex column counts as two, a
- *          complex entry too; 5 to 7 columns count as 8): rows of H and columns of X as 56-bit fixed-point
+ *          complex entry too; 5 to 7 columns count as 8) and work items of a
+ *          few hundred entries: rows of H and columns of X as 56-bit fixed-point
  *          integers in exact base-256 digits, their products summed exactly
  *          and rounded once. An output that the fixed point does not resolve
  *          (its terms far below its row's or column's largest), rows and
@@ -290,7 +291,8 @@ int vbcsr_spmm_ex(vbcsr_t *A, int transpose, int64_t k, double alpha, const void
  * for every stored block (i, j), written in packed order.
  *  Aop  device [n_rows, k], lda >= k;  Bop  device [n_cols, k], ldb >= k
  *  D    device, nnz elements of the matrix dtype; beta == 0: D is not read
- * FP64 operators of at least 2^22 stored entries x columns, 6 <= k <= 768, form it on
+ * FP64 operators of at least 2^22 stored entries x columns, 6 <= k <= 768, and work items
+ * of a few hundred entries form it on
  * the tensor cores like the native products, with fixed-point copies of Aop and Bop in a
  * buffer of the handle (8 bytes an element, columns rounded up to 16), allocated and
  * grown on first use as theirs are, and by FMA where those would be.
