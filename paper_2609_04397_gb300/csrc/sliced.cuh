@@ -30,7 +30,10 @@
 // computed with FP64 multiply-adds by the same warp: what remains has an error
 // of at most a few dozen 2^-53 of sum |h x|, inside the K 2^-53 of a K-term
 // multiply-add chain. Rows and columns with Inf, NaN or extreme exponents and
-// panels with mostly tiny entries take the multiply-adds as well.
+// panels with mostly tiny entries (one-hot or localised columns) take the
+// multiply-adds as well, and lose the two passes over X (3 to 6 % at k = 16 and 8
+// on 20k atoms); columns that fall by 10^3 from end to end, with part of the
+// outputs unresolved, still run 1.5 to 1.9 times as fast as multiply-adds.
 //
 // (The FP8 form of the same scheme, 12 base-32 digits in e4m3, needs no carries
 // and is as exact, but mma.sync runs e4m3 operands converted on the f16
