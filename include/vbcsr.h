@@ -84,14 +84,16 @@ typedef enum {
  *          and rounded once. An output that the fixed point does not resolve
  *          (its terms far below its row's or column's largest), rows and
  *          columns with Inf, NaN or extreme exponents, and everything smaller
- *          is computed by FP64 FMA; either way the error is within that of an
- *          FMA chain. The digits of the values (7 bytes an entry, one copy a
- *          direction) and of X are buffers that the handle owns, allocated on
- *          first use and grown like those of the mixed modes; while `stream`
- *          is being captured, or when the device has no room, nothing is
- *          allocated and such a call runs by FMA. Make one ordinary call
- *          before a capture so that the graph gets the tensor-core form; a
- *          graph stays valid when later calls need larger buffers.
+ *          is computed by FP64 FMA; either way the error of an output of K
+ *          terms is within the bound of an FMA chain, K 2^-53 of sum |h x|
+ *          and the rounding of the result. The digits of the values (7 bytes
+ *          an entry, one copy a direction) and of X are buffers that the handle
+ *          owns, allocated on first use and grown like those of the mixed
+ *          modes; while `stream` is being captured, or when the device has no
+ *          room, nothing is allocated and such a call runs by FMA. Make one
+ *          ordinary call before a capture so that the graph gets the
+ *          tensor-core form; a graph stays valid when later calls need larger
+ *          buffers.
  *  F32     values and X rounded to FP32, FP32 FMA, FP32 accumulation
  *  TF32    one TF32 tensor-core product per block product, FP32 accumulation
  *  TF32X3  v = hi + lo with hi = tf32(v), lo = tf32(v - hi) for values and X;

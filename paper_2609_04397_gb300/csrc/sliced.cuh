@@ -20,20 +20,18 @@
 //  * the levels 0 .. 7 (34 digit pairs) are added as integers and rounded to
 //    FP64 once. What is dropped is about 2^-58 of (row scale) x (column scale).
 //
-// An FP64 multiply-add chain instead rounds at every step; on the operators
-// and panels of this repository the sliced product is the nearer one to the
-// exact result. The scales make its error an absolute one, though: an output
-// whose terms are all far below the row's and the column's largest would lose
-// digits. So every output also carries an estimate of sum |h x| (the products
-// of the leading digits' magnitudes, one more MMA in 35), and the remaining
-// columns of an item with an output whose estimate is below kSliceGuard are
-// computed with FP64 multiply-adds by the same warp: what remains has an error
-// of at most a few dozen 2^-53 of sum |h x|, inside the K 2^-53 of a K-term
-// multiply-add chain. Rows and columns with Inf, NaN or extreme exponents and
-// panels with mostly tiny entries (one-hot or localised columns) take the
-// multiply-adds as well, and lose the two passes over X (3 to 6 % at k = 16 and 8
-// on 20k atoms); columns that fall by 10^3 from end to end, with part of the
-// outputs unresolved, still run 1.5 to 1.9 times as fast as multiply-adds.
+// An FP64 multiply-add chain instead rounds at every step; on panels of entries of
+// like size the sliced product is the nearer one to the exact result. The scales
+// make its error an absolute one, though: an output whose terms are all far below
+// the row's and the column's largest would lose digits. So every output also
+// carries an estimate of sum |h x| (the products of the leading digits'
+// magnitudes, one more MMA in 35), and an output whose estimate is too low
+// (kSliceGuard, slice_guard) is computed with FP64 multiply-adds by the same
+// warp, alone or with its pass of 16 columns. What remains is within K 2^-53 of
+// sum |h x|, the bound of a K-term multiply-add chain, and the one rounding. Rows
+// and columns with Inf, NaN or extreme exponents and panels with mostly tiny
+// entries (one-hot or localised columns) take the multiply-adds as well, and lose
+// the two passes over X (2 to 6 % at k = 8 to 32 on 50k and 20k atoms).
 //
 // (The FP8 form of the same scheme, 12 base-32 digits in e4m3, needs no carries
 // and is as exact, but mma.sync runs e4m3 operands converted on the f16
@@ -45,7 +43,23 @@
 
 namespace vbcsr {
 
-constexpr float kSliceGuard = 512.f;   // least sum of |leading digit| products of an output
+// Least sum of |leading digit| products of an output. In units of the last place (2^-55
+// of a scale) every element is rounded by up to 1/2, which costs an output up to
+// (sum |h| + sum |x|) / 2 <= 2^54 K (1 + sum |h x| / 2^110); the levels left out and the
+// FP32 sums past 2^24 in the levels 5 to 7 add less than 2 % of 2^54 K. Leading digits d
+// and e stand for magnitudes of at least (d - 0.502) 2^48 and (e - 0.502) 2^48. The least
+// sum |h x| for a given estimate and room for K roundings is that of products 1 x 128:
+// 0.496 of the estimate times 2^96, and 2^54 K <= K 2^-53 (0.496 G 2^96) from G = 4129 on,
+// whatever K is. (At 512 products of K = 764 were off by up to 2300 2^-53 of sum |h x|.)
+constexpr float kSliceGuard = 4352.f;
+// The same with the sum of the leading digits' magnitudes of the row and of the column over
+// the K terms at hand: sum |h| + sum |x| <= (digits + 1.004 K) 2^48, the levels left out
+// are below 2^48.4 K, sum |h x| is at least 0.248 of the estimate times 2^96. Panels whose
+// column maxima lie far above most entries stay resolved by it (Student's t with 3 degrees
+// of freedom, 20k disordered atoms, k = 8: 886 us by kSliceGuard alone, 546 by multiply-adds).
+__device__ __forceinline__ float slice_guard(int digits, int K) {
+    return fminf(kSliceGuard, 66.f * ((float)digits / (float)K + 3.7f));
+}
 constexpr int kSliceLevels = 8;
 constexpr int kSliceFlush = 12;        // 16-column steps between carries: 5 products x 192 columns x 2^14 < 2^24
 constexpr int kSliceTile = kSliceDigits * 16;   // bytes of one row of a 16-column value tile

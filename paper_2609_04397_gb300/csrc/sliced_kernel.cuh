@@ -10,7 +10,16 @@ namespace vbcsr {
 namespace {
 
 constexpr int kSliceList = (kSliceKMax + 16) * sizeof(int32_t);   // X rows of an item and of one step more
+constexpr int kSliceState = 16;   // bytes that a warp keeps from item to item
+constexpr int kSliceSingles = 32; // unresolved outputs of a pass computed one by one
 constexpr int kSliceStages = 4;   // value tiles in flight per warp (16 columns, up to 1792 bytes each)
+
+// What a warp keeps from item to item, behind its list: [0] the structure of the last item,
+// [1] its passes that run multiply-adds: bit p for the 16 columns of pass p, bit 31 for pass
+// 31 and all after it; [2] whether the last pass had outputs below kSliceGuard
+__device__ __forceinline__ volatile uint32_t *slice_state(unsigned char *ring) {
+    return reinterpret_cast<volatile uint32_t *>(ring + kSliceStages * 16 * kSliceTile + kSliceList);
+}
 
 // the operator's own arithmetic, for what is not sliced
 template <int B, bool TRANS, typename T, typename TA>
@@ -19,14 +28,14 @@ __device__ __noinline__ void fma_item_fallback(const ProdArgs &a, const WorkItem
     process_item<B, TRANS, T, TA, T, T>(a, w, kc, s_x, s_a, nullptr, lane, dot);
 }
 
-// Columns [n0, k) of item w by FP64 multiply-adds (complex T: two real columns of the
+// Columns [n0, n1) of item w by FP64 multiply-adds (complex T: two real columns of the
 // sliced panels make one)
 template <bool TRANS, typename T, typename TA>
-__device__ __noinline__ void fma_columns(const ProdArgs &a, int64_t n0, const WorkItem &w, unsigned char *smem, int lane,
+__device__ __noinline__ void fma_columns(const ProdArgs &a, int64_t n0, int64_t n1, const WorkItem &w, unsigned char *smem, int lane,
                                          double &dot) {
     ProdArgs b = a;
     constexpr int cw = sizeof(T) / sizeof(double);
-    b.k = (a.k - n0) / cw;
+    b.k = (n1 - n0) / cw;
     b.ldx = a.ldx / cw;
     b.ldy = a.ldy / cw;
     b.ldz = a.ldz / cw;
@@ -51,6 +60,56 @@ __device__ __noinline__ void fma_columns(const ProdArgs &a, int64_t n0, const Wo
 #undef VBCSR_SLICE_CASE
 }
 
+// Output (row r of the item, real column c) by FP64 multiply-adds: the whole warp, four
+// lanes a stored block, so a chain has a few terms a block and at most K / 4. Items that
+// need it are small and come last, where their latency shows. Complex T: the real column
+// is one component of a complex one.
+template <bool TRANS, typename T>
+__device__ __noinline__ double slice_one_output(const ProdArgs &a, const WorkItem &w, int r, int64_t c, int lane) {
+    constexpr int cw = sizeof(T) / sizeof(double);
+    const double *V = static_cast<const double *>(a.values), *X = static_cast<const double *>(a.X) + c;
+    double acc = 0.0;
+    for (int e = lane >> 2; e < w.nlist; e += 8) {
+        const int64_t l = w.lbegin + e;
+        const double *v = V + cw * (TRANS ? a.tl.pbase[l] + w.Kp + r : w.vbase + (int64_t)r * w.Kp + a.fl.pcol[l]);
+        const int64_t step = TRANS ? cw * (int64_t)a.tl.kp[l] : cw;
+        const double *x = X + (int64_t)(TRANS ? a.tl.xrow[l] : a.fl.xrow[l]) * a.ldx;
+        const int n = TRANS ? a.tl.bi[l] : a.fl.w[l];
+#pragma unroll 4
+        for (int t = lane & 3; t < n; t += 4) {
+            const double *vt = v + t * step, *xt = x + t * a.ldx;
+            acc = fma(vt[0], xt[0], acc);
+            // re: - im(v) im(x); im: + im(v) re(x); the adjoint conjugates v
+            if (cw == 2) acc = fma(((c & 1) != 0) != TRANS ? vt[1] : -vt[1], xt[c & 1 ? -1 : 1], acc);
+        }
+    }
+    for (int m = 16; m > 0; m >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, m);
+    return acc;
+}
+
+// Sums of the magnitudes of the leading digits: sum[r] of row r of the item's value tiles,
+// sum[16 + c] of column n0 + c of the X rows in s_x (sum in shared memory)
+__device__ __noinline__ void slice_digit_sums(const unsigned char *tiles, int B, int K, const uint64_t *xdig, int ldp,
+                                              int64_t n0, const int32_t *s_x, int *sum, int lane) {
+    const int i = lane & 15, h = lane >> 4;
+    unsigned rows = 0, cols = 0;
+    if (i < B)
+        for (int t = h; 16 * t < K; t += 2) {
+            const uint4 v = __ldg(reinterpret_cast<const uint4 *>(tiles + (int64_t)t * B * kSliceTile + 16 * i));
+            const uint32_t zero = 0x80808080u;
+            rows += __vsadu4(v.x, zero) + __vsadu4(v.y, zero) + __vsadu4(v.z, zero) + __vsadu4(v.w, zero);
+        }
+    if (n0 + i < ldp)
+#pragma unroll 8
+        for (int t = h; t < K; t += 2)
+            cols += abs((int)(__ldg(xdig + (int64_t)s_x[t] * ldp + n0 + i) >> 48 & 0xff) - 128);
+    rows += __shfl_xor_sync(0xffffffffu, rows, 16);
+    cols += __shfl_xor_sync(0xffffffffu, cols, 16);
+    __syncwarp();
+    sum[lane] = (int)(h ? cols : rows);
+    __syncwarp();
+}
+
 // One pass of an item: up to 16 columns (WIDE) or up to 8, steps of 16 virtual
 // columns. A step's value tile (7 digits x B rows x 16 bytes, contiguous) comes
 // through a ring of shared-memory stages by asynchronous copies; the 16 gathered
@@ -70,13 +129,20 @@ __device__ __noinline__ void fma_columns(const ProdArgs &a, int64_t n0, const Wo
 // alone with its digits as the N side, one more MMA per digit of X (PAIR: per two)
 // instead of another group of 8 rows: 44 MMAs a wide step instead of 72, 25 a
 // narrow one instead of 36 (50k zinc-blende atoms, k = 32: 1.43 ms against 1.56).
-// Returns false, with nothing written, when an output is not resolved by the
-// fixed point.
-template <bool TRANS, bool WIDE, int NR, bool NINTH = false>
+// Returns false, with nothing written, when an output is below kSliceGuard. Such a pass is
+// made a second time with CAREFUL (code that would cost the first one registers): outputs
+// below kSliceGuard are looked at with the sums that their error really depends on
+// (slice_guard), and those that the fixed point does not resolve are computed by
+// slice_one_output, up to kSliceSingles of them (rows of few entries have one now and
+// then: corners of a cluster, 40 to 120 columns; without this the k = 32 product on 50k
+// zinc-blende atoms took 1.52 ms, all 16 columns of such items by multiply-adds). It
+// returns false when there are more or a row has no scale.
+template <bool TRANS, bool WIDE, int NR, bool NINTH, bool CAREFUL, typename T>
 __device__ __forceinline__ bool slice_pass(const ProdArgs &a, const SliceArgs &q, const WorkItem &w,
-                                           const unsigned char *vsrc, int nsteps, int64_t n0, const uint32_t *cmax,
+                                           const unsigned char *vsrc, int K, int64_t n0, const uint32_t *cmax,
                                            unsigned char *ring, const int32_t *s_x, int lane, double &dot) {
     constexpr int S = kSliceStages, kStage = 16 * kSliceTile;
+    const int nsteps = (K + 15) >> 4;
     constexpr int NX = WIDE ? 2 : 1, NA = WIDE ? NR : 1;
     constexpr bool PAIR = !WIDE && NR == 1;
     // the ninth row: digit j of X (PAIR: j and j + 1) times all its digits, 2 t4 + e a lane
@@ -240,7 +306,29 @@ __device__ __forceinline__ bool slice_pass(const ProdArgs &a, const SliceArgs &q
         for (int h = 0; h < NX; ++h)   // lanes t4 = 0 hold digit 0
             ok &= e9 == 0 || ec[2 * h] == 0 || t4 != 0 || nlow[2 * h] >= kSliceGuard;
     }
-    if (!__all_sync(0xffffffffu, ok)) return false;
+    if (!CAREFUL && !__all_sync(0xffffffffu, ok)) return false;
+    uint32_t bad = 0;   // those for slice_one_output: bit 4 n + j, 8 + h for the ninth row's column g + 8 h
+    if (CAREFUL) {
+        const bool again = !__all_sync(0xffffffffu, ok);
+        if (lane == 0) slice_state(ring)[2] = again;
+        int *sum = reinterpret_cast<int *>(ring);
+        slice_digit_sums(vsrc, w.B, K, q.xdig, q.ldp, n0, s_x, sum, lane);
+        bool scaled = e9 >= 0;
+#pragma unroll
+        for (int n = 0; n < NA; ++n)
+#pragma unroll
+            for (int j = 0; j < (PAIR ? 2 : 4); ++j) {
+                scaled &= er[n][j] >= 0;
+                const float guard = slice_guard(sum[row_of(n, j >> 1, j & 1)] + sum[16 + col_of(j >> 1, j & 1)], K);
+                if (er[n][j] != 0 && ec[j] != 0 && low[n][j] < guard) bad |= 1u << (4 * n + j);
+            }
+        if (NINTH && t4 == 0)
+#pragma unroll
+            for (int h = 0; h < NX; ++h)
+                if (e9 != 0 && ec[2 * h] != 0 && nlow[2 * h] < slice_guard(sum[8] + sum[16 + g + 8 * h], K)) bad |= 256u << h;
+        if (!__all_sync(0xffffffffu, scaled) || __reduce_add_sync(0xffffffffu, __popc(bad)) > kSliceSingles) return false;
+        __syncwarp();   // before the next pass's tiles go where the sums were
+    }
     auto store = [&](int64_t row, int64_t c, double o) {
         double *y = static_cast<double *>(a.Y) + row * a.ldy + c;
         if (!q.alpha_pow2) o *= a.alpha;
@@ -260,7 +348,7 @@ __device__ __forceinline__ bool slice_pass(const ProdArgs &a, const SliceArgs &q
                 for (int d = 0; d < kSliceDigits; ++d)
                     t[e][d] = WIDE ? ninth[d % NJ][2 * h + e] : ninth[d / 2 % NJ][2 * (d & 1) + e];
             const double o = slice_value_of_lanes(t, t4, e9 + ec[2 * h] - 2114 + q.alpha_exp);
-            if (t4 == 0 && n0 + g + 8 * h < a.k) store(w.yrow + 8, n0 + g + 8 * h, o);
+            if (t4 == 0 && n0 + g + 8 * h < a.k && !(bad & (256u << h))) store(w.yrow + 8, n0 + g + 8 * h, o);
         }
     }
 #pragma unroll
@@ -270,7 +358,7 @@ __device__ __forceinline__ bool slice_pass(const ProdArgs &a, const SliceArgs &q
             if (PAIR && j >= 2) continue;
             const int r = row_of(n, j >> 1, j & 1);
             const int64_t c = n0 + col_of(j >> 1, j & 1);
-            if (r >= (NINTH ? 8 : w.B) || c >= a.k) continue;
+            if (r >= (NINTH ? 8 : w.B) || c >= a.k || (bad & (1u << (4 * n + j)))) continue;
             const int64_t row = w.yrow + r;
             float lv[kSliceLevels];
 #pragma unroll
@@ -278,7 +366,37 @@ __device__ __forceinline__ bool slice_pass(const ProdArgs &a, const SliceArgs &q
                 lv[L] = acc[n][L][j] + (PAIR && L > 0 ? acc[n][L > 0 ? L - 1 : 0][(j + 2) & 3] : 0.f);
             store(row, c, slice_value(lv, er[n][j] + ec[j] - 2114 + q.alpha_exp));
         }
+    if (CAREFUL)
+        for (unsigned lanes; (lanes = __ballot_sync(0xffffffffu, bad != 0)) != 0;) {
+            const int src = __ffs(lanes) - 1, bit = __ffs(bad) - 1, j = bit & 3;
+            const bool last = bit >= 8;
+            const int r = __shfl_sync(0xffffffffu, last ? 8 : row_of(bit >> 2, j >> 1, j & 1), src);
+            const int c = __shfl_sync(0xffffffffu, last ? g + 8 * j : col_of(j >> 1, j & 1), src);
+            double o = slice_one_output<TRANS, T>(a, w, r, n0 + c, lane);
+            if (q.alpha_pow2) o *= a.alpha;
+            if (lane != src) continue;
+            store(w.yrow + r, n0 + c, o);
+            bad &= bad - 1;
+        }
     return true;
+}
+
+template <bool TRANS, bool WIDE, bool CAREFUL, typename T>
+__device__ __forceinline__ bool slice_pass_rows(const ProdArgs &a, const SliceArgs &q, const WorkItem &w,
+                                                const unsigned char *vsrc, int K, int64_t n0, const uint32_t *cmax,
+                                                unsigned char *ring, const int32_t *s_x, int lane, double &dot) {
+    return w.B <= 8 ? slice_pass<TRANS, WIDE, 1, false, CAREFUL, T>(a, q, w, vsrc, K, n0, cmax, ring, s_x, lane, dot)
+           : w.B == 9 ? slice_pass<TRANS, WIDE, 1, true, CAREFUL, T>(a, q, w, vsrc, K, n0, cmax, ring, s_x, lane, dot)
+                      : slice_pass<TRANS, WIDE, 2, false, CAREFUL, T>(a, q, w, vsrc, K, n0, cmax, ring, s_x, lane, dot);
+}
+
+// The second attempt at a pass, or the only one where the warp's last pass needed two
+// (panels of a few large entries; the outputs are the same bits either way)
+template <bool TRANS, bool WIDE, typename T>
+__device__ __noinline__ bool slice_pass_again(const ProdArgs &a, const SliceArgs &q, const WorkItem &w,
+                                              const unsigned char *vsrc, int K, int64_t n0, const uint32_t *cmax,
+                                              unsigned char *ring, const int32_t *s_x, int lane, double &dot) {
+    return slice_pass_rows<TRANS, WIDE, true, T>(a, q, w, vsrc, K, n0, cmax, ring, s_x, lane, dot);
 }
 
 // One warp per work item (up to 16 output rows). WIDE: k > 8, passes of 16
@@ -287,13 +405,22 @@ __device__ __forceinline__ bool slice_pass(const ProdArgs &a, const SliceArgs &q
 // Complex operators (T = double2, TA its arithmetic): the kernel sees two real
 // columns a complex one and two virtual columns a complex value, re meeting the
 // X row x and im the row i x (slice_panel_kernel).
+// (The arguments are grid constants: the calls take their addresses, and a copy on the
+// stack cost the loop registers, 1.45 against 1.48 ms at k = 32 on 50k zinc-blende atoms.)
 template <bool TRANS, bool WIDE, typename T, typename TA>
-__global__ void __launch_bounds__(128, WIDE ? 3 : 4) slice_product_kernel(ProdArgs a, SliceArgs q) {
+__global__ void __launch_bounds__(128, WIDE ? 3 : 4) slice_product_kernel(const __grid_constant__ ProdArgs a,
+                                                                            const __grid_constant__ SliceArgs q) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int kRing = kSliceStages * 16 * kSliceTile;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    unsigned char *ring = smem_raw + (size_t)warp * (kRing + kSliceList);
+    unsigned char *ring = smem_raw + (size_t)warp * (kRing + kSliceList + kSliceState);
     int32_t *s_x = reinterpret_cast<int32_t *>(ring + kRing);
+    volatile uint32_t *state = slice_state(ring);
+    if (lane == 0) {
+        state[0] = ~0u;
+        state[2] = 0;
+    }
+    __syncwarp();
     double dot = 0.0;
 
     // the next item is claimed when an item starts (lane 0's value counts)
@@ -301,8 +428,6 @@ __global__ void __launch_bounds__(128, WIDE ? 3 : 4) slice_product_kernel(ProdAr
         if (!a.queue) return (unsigned long long)(from + (int64_t)gridDim.x * 4);
         return lane == 0 ? atomicAdd(reinterpret_cast<unsigned long long *>(a.queue), 1ull) : 0ull;
     };
-    int last_strct = -1;
-    bool last_plain = false;
     int64_t it = (int64_t)blockIdx.x * 4 + warp;
     if (a.queue) it = (int64_t)__shfl_sync(0xffffffffu, claim(0), 0);
     while (it < a.n_items) {
@@ -310,21 +435,28 @@ __global__ void __launch_bounds__(128, WIDE ? 3 : 4) slice_product_kernel(ProdAr
         const WorkItem w = a.items[it];
         const SliceItem si = q.sitems[it];
         const uint32_t *cmax = q.cmax + (int64_t)si.strct * q.ldp;
-        if (si.strct != last_strct) {
+        if ((uint32_t)si.strct != state[0]) {
             // a small structure, or one with a column outside the sliced range or mostly tiny, is not sliced
-            last_strct = si.strct;
             const uint32_t most = (uint32_t)q.struct_rows[si.strct] >> 2;
-            bool p = q.struct_nnz[si.strct] < q.min_nnz;
-            for (int c = lane; c < (int)a.k; c += 32)
-                p |= !slice_exp_ok(cmax[c]) || q.ccnt[(int64_t)si.strct * q.ldp + c] > most;
-            last_plain = __any_sync(0xffffffffu, p);
+            uint32_t plain = q.struct_nnz[si.strct] < q.min_nnz ? ~0u : 0u;
+            for (int c0 = 0; c0 < (int)a.k; c0 += 32) {
+                const int c = c0 + lane;
+                const unsigned m = __ballot_sync(
+                    0xffffffffu, c < (int)a.k && (!slice_exp_ok(cmax[c]) || q.ccnt[(int64_t)si.strct * q.ldp + c] > most));
+                if (m) plain = ~0u;
+            }
+            __syncwarp();
+            if (lane == 0) {
+                state[0] = (uint32_t)si.strct;
+                state[1] = plain;
+            }
+            __syncwarp();
         }
-        const bool plain = last_plain || si.doff < 0;
+        uint32_t skip = si.doff < 0 ? ~0u : state[1];   // this item's passes that are not tried
         constexpr int cw = sizeof(T) / sizeof(double);
         const int K = cw * w.K, nsteps = (K + 15) >> 4;
         const unsigned char *vsrc = q.vdig + si.doff;
-        int64_t n0 = 0;
-        if (!plain && nsteps > 0) {
+        if (skip != ~0u && nsteps > 0) {
             // X row of every virtual column (a valid row past the last one: its digits meet zeros)
             __syncwarp();
             for (int e = lane; e < w.nlist; e += 32) {
@@ -338,27 +470,53 @@ __global__ void __launch_bounds__(128, WIDE ? 3 : 4) slice_product_kernel(ProdAr
             }
             __syncwarp();
         }
-        if (!plain) {
-            bool ok = true;
-            if constexpr (WIDE)
-                for (; ok && n0 + 8 < a.k; n0 += ok ? 16 : 0)
-                    ok = w.B <= 8 ? slice_pass<TRANS, true, 1>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot)
-                         : w.B == 9
-                             ? slice_pass<TRANS, true, 1, true>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot)
-                             : slice_pass<TRANS, true, 2>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot);
-            if (ok && n0 < a.k) {
-                ok = w.B <= 8 ? slice_pass<TRANS, false, 1>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot)
-                     : w.B == 9
-                         ? slice_pass<TRANS, false, 1, true>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot)
-                         : slice_pass<TRANS, false, 2>(a, q, w, vsrc, nsteps, n0, cmax, ring, s_x, lane, dot);
-                n0 += ok ? 8 : 0;
+        if constexpr (!WIDE) {   // one pass
+            const bool tried = skip == 0;
+            if (!tried || state[2] || !slice_pass_rows<TRANS, false, false, T>(a, q, w, vsrc, K, 0, cmax, ring, s_x, lane, dot)) {
+                const WorkItem wc = w;   // copies: the calls take addresses, which would keep w and dot in memory
+                double dc = dot;
+                if (!tried || !slice_pass_again<TRANS, false, T>(a, q, wc, vsrc, K, 0, cmax, ring, s_x, lane, dc))
+                    fma_columns<TRANS, T, TA>(a, 0, a.k, wc, ring, lane, dc);
+                __syncwarp();
+                dot = dc;
             }
-        }
-        if (n0 < a.k) {
-            const WorkItem wc = w;   // copies: the call takes addresses, which would keep w and dot in memory
-            double dc = dot;
-            fma_columns<TRANS, T, TA>(a, n0, wc, ring, lane, dc);
-            dot = dc;
+        } else {
+            int64_t n0 = 0;
+            while (n0 < a.k) {
+                // sliced up to the next pass that is not tried
+                const uint32_t left = skip >> min((int)(n0 >> 4), 31);
+                const int64_t stop = left ? min(a.k, n0 + 16 * (int64_t)(__ffs(left) - 1)) : a.k;
+                bool ok = n0 >= stop || !state[2];
+                for (; ok && n0 + 8 < stop; n0 += ok ? 16 : 0)
+                    ok = slice_pass_rows<TRANS, true, false, T>(a, q, w, vsrc, K, n0, cmax, ring, s_x, lane, dot);
+                if (ok && n0 < stop) {
+                    ok = slice_pass_rows<TRANS, false, false, T>(a, q, w, vsrc, K, n0, cmax, ring, s_x, lane, dot);
+                    n0 += ok ? 8 : 0;
+                }
+                if (n0 >= a.k) break;
+                const WorkItem wc = w;   // copies: the calls take addresses, which would keep w and dot in memory
+                double dc = dot;
+                const bool wide = n0 + 8 < a.k;
+                if (!ok)
+                    ok = wide ? slice_pass_again<TRANS, WIDE, T>(a, q, wc, vsrc, K, n0, cmax, ring, s_x, lane, dc)
+                              : slice_pass_again<TRANS, false, T>(a, q, wc, vsrc, K, n0, cmax, ring, s_x, lane, dc);
+                else
+                    ok = false;   // not tried
+                int64_t n1 = n0 + (wide ? 16 : 8);
+                if (!ok) {
+                    // by multiply-adds, with the passes after it that are not tried: after two with
+                    // unresolved outputs none of the item's are
+                    const uint32_t self = 1u << min((int)(n0 >> 4), 31);
+                    if (!(skip & self)) skip = skip == state[1] ? skip | self : ~0u;
+                    if (skip == ~0u) n1 = a.k;
+                    while (n1 < a.k && (skip >> min((int)(n1 >> 4), 31) & 1u)) n1 += 16;
+                    n1 = min(n1, a.k);
+                    fma_columns<TRANS, T, TA>(a, n0, n1, wc, ring, lane, dc);
+                    __syncwarp();   // before the next pass's tiles go where the multiply-adds kept their lists
+                }
+                dot = dc;
+                n0 = n1;
+            }
         }
         if (a.item_partials) {
             // the item's share of the fused dot at the item's index (summed in a fixed order afterwards)
@@ -381,7 +539,7 @@ const void *slice_kernel_of(bool trans, int64_t k) {
     return (const void *)(trans ? slice_kernel<true, T, TA>(k) : slice_kernel<false, T, TA>(k));
 }
 
-constexpr size_t kSliceSmem = 4 * ((size_t)kSliceStages * 16 * kSliceTile + kSliceList);
+constexpr size_t kSliceSmem = 4 * ((size_t)kSliceStages * 16 * kSliceTile + kSliceList + kSliceState);
 
 template <typename T, typename TA>
 cudaError_t launch_slice(bool trans, const ProdArgs &a, const SliceArgs &q, cudaStream_t s) {

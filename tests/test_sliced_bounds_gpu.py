@@ -1,0 +1,188 @@
+"""Error bounds of the sliced FP64 products: an output of K terms within
+(K + 2) 2^-53 of sum |h x| (the bound of a K-term multiply-add chain, and the
+epilogue), on operands that sit just above the kernels' checks and on panels whose
+entries fall over many orders of magnitude."""
+from fractions import Fraction
+
+import numpy as np
+import pytest
+import torch
+
+from synthetic.structures import BlockPattern
+
+pytestmark = pytest.mark.gpu
+U = 2.0 ** -53
+
+
+def _handle(pat, vals):
+    from paper_2609_04397_gb300 import VBCSR
+    return VBCSR.from_pattern(pat, vals, torch.float64, "cuda:0")
+
+
+def _kernels(fn):
+    """Names of the library's kernels that fn launches (never empty)."""
+    from torch.profiler import ProfilerActivity, profile
+    for _ in range(5):   # a trace can come back before its buffers fill
+        with profile(activities=[ProfilerActivity.CUDA]) as prof:
+            fn()
+            torch.cuda.synchronize()
+        names = [e.name for e in prof.events() if "vbcsr" in e.name]
+        if names:
+            return names
+    raise AssertionError("no trace of the launches")
+
+
+def _uniform(rows, K, b=16):
+    """rows block rows of b x b blocks, all over the same K / b block columns."""
+    n = K // b
+    return BlockPattern(np.full(rows, b), np.full(n, b), np.arange(rows + 1) * n, np.tile(np.arange(n), rows))
+
+
+def _block_values(h, rows, b=16):
+    """The same stored row h everywhere."""
+    blocks = np.broadcast_to(h.reshape(-1, 1, b), (len(h) // b, b, b))
+    return np.tile(blocks.reshape(-1), rows)
+
+
+def _sums(h, x):
+    terms = [Fraction(a) * Fraction(b) for a, b in zip(h.tolist(), x.tolist())]
+    return sum(terms), sum(abs(t) for t in terms)
+
+
+def _products(K):
+    """(h, x) of K terms: large entries of one side meet entries of the other that the
+    fixed point rounds by half a unit, and the sum rests on a few products."""
+    half = 0.99 * 2.0 ** -55   # 0.495 of the last place at a scale of 1.97
+    h, x = np.full(K, half), np.full(K, 1.97)
+    h[0], x[0] = 1.97, 4.6 * 2.0 ** -6
+    yield "one product", h, x
+    for n in (9, 33, 35, 60):   # n products of leading digits 126 x 1
+        h, x = np.full(K, half), np.full(K, 1.97)
+        h[:n], x[:n] = 1.97, 0.504 * 2.0 ** -6
+        yield f"{n} products", h, x
+
+
+@pytest.mark.parametrize("K", [64, 320, 768])
+@pytest.mark.parametrize("k", [5, 16])
+def test_products_just_above_the_check(K, k):
+    rows = -(-(1 << 24) // (16 * K * (8 if k < 8 else k)))
+    pat = _uniform(rows, K)
+    for name, h, x in _products(K):
+        H = _handle(pat, _block_values(h, rows))
+        sign = np.where(np.arange(k) % 2, -1.0, 1.0)
+        X = torch.from_numpy(x[:, None] * sign).cuda()
+        exact, mag = _sums(h, x)
+        got = H.spmm(X).cpu().numpy()
+        bound = float((K + 2) * U * mag)
+        for s in (1, -1):
+            err = max(abs(Fraction(v) - s * exact) for v in np.unique(got[:, sign == s]).tolist())
+            assert err <= bound, (name, float(err / mag) / U)
+    assert any("slice_product" in n for n in _kernels(lambda: H.spmm(X)))
+
+
+@pytest.mark.parametrize("K", [128, 320, 752])
+@pytest.mark.parametrize("fall", [3.0, 7.0, 14.0])
+def test_falling_panels(K, fall, monkeypatch):
+    """Columns of X that fall by e^-fall within a row of H, in random order: inside the bound,
+    and no further off than the multiply-adds of the same call (a handle with device checks)."""
+    rng = np.random.default_rng(int(K + fall))
+    rows = -(-(1 << 24) // (16 * K * 16))
+    pat = _uniform(rows, K)
+    vals = rng.standard_normal(pat.nnz)
+    H = _handle(pat, vals)
+    monkeypatch.setenv("VBCSR_DEBUG_CHECKS", "1")
+    plain = _handle(pat, vals)
+    X = rng.standard_normal((K, 16)) * np.exp(-fall * rng.random((K, 16)))
+    dense = vals.reshape(rows, K // 16, 16, 16).transpose(0, 2, 1, 3).reshape(rows * 16, K)[:2048].astype(np.longdouble)
+    exact = dense @ X.astype(np.longdouble)
+    mag = (np.abs(dense) @ np.abs(X).astype(np.longdouble)).astype(np.float64)
+    Xd = torch.from_numpy(X).cuda()
+    e, ec = (np.abs((P.spmm(Xd)[:2048].cpu().numpy() - exact).astype(np.float64)) / mag / U for P in (H, plain))
+    assert e.max() <= K + 2
+    assert np.sqrt(np.mean(e ** 2)) <= np.sqrt(np.mean(ec ** 2))
+    assert any("slice_product" in n for n in _kernels(lambda: H.spmm(Xd)))
+    assert not any("slice" in n for n in _kernels(lambda: plain.spmm(Xd)))
+
+
+def _spiked(b, cols, k, complex_values, seed):
+    """A dense operator of b-row items with one huge entry in every seventh row, met by a panel
+    whose row there is zero in the odd columns: one unresolved output a column pair."""
+    rng = np.random.default_rng(seed)
+    wb = -(-cols // b)
+    rows = max(-(-(1 << 24) // (b * wb * b * (16 if k > 8 else 8))), 4)
+    pat = BlockPattern(np.full(rows, b), np.full(wb, b), np.arange(rows + 1) * wb, np.tile(np.arange(wb), rows))
+    K = wb * b
+    D = rng.standard_normal((rows * b, K))
+    X = rng.standard_normal((K, k))
+    if complex_values:
+        D = D + 1j * rng.standard_normal(D.shape)
+        X = X + 1j * rng.standard_normal(X.shape)
+    D[::7, K - 2] *= 1e9
+    X[K - 2, 1::4] = 0.0
+    vals = D.reshape(rows, b, wb, b).transpose(0, 2, 1, 3).reshape(-1)
+    return pat, np.ascontiguousarray(vals), D, X
+
+
+@pytest.mark.parametrize("b", [3, 8, 9, 13, 16])
+@pytest.mark.parametrize("k", [5, 8, 16, 21])
+@pytest.mark.parametrize("kind", [np.float64, np.complex128])
+def test_single_unresolved_outputs(b, k, kind):
+    """Forward and adjoint, with the fused epilogue, alpha a power of two and not."""
+    from paper_2609_04397_gb300 import VBCSR
+    cplx = kind is np.complex128
+    pat, vals, D, X = _spiked(b, 160, k, cplx, b + k)
+    H = VBCSR.from_pattern(pat, vals, torch.complex128 if cplx else torch.float64, "cuda:0")
+    rng = np.random.default_rng(1)
+    K = D.shape[1]
+    some = np.unique(np.concatenate([np.arange(0, min(200, len(D))), np.arange(0, len(D), max(len(D) // 200, 1))]))
+    wide = np.clongdouble if cplx else np.longdouble
+    for alpha in (2.0, -0.3):
+        Y0, Z, R = (rng.standard_normal((len(D), k)).astype(kind) for _ in range(3))
+        Y, dot = torch.from_numpy(Y0.copy()).cuda(), torch.zeros(1, dtype=torch.float64, device="cuda:0")
+        H.spmm_ex(torch.from_numpy(X).cuda(), alpha, -1.0, Y, gamma=0.5, Z=torch.from_numpy(Z).cuda(),
+                  R=torch.from_numpy(R).cuda(), dot_out=dot)
+        got = Y.cpu().numpy()
+        ref = alpha * (D[some].astype(wide) @ X.astype(wide)) - Y0[some] + 0.5 * Z[some]
+        mag = abs(alpha) * (np.abs(D[some]) @ np.abs(X)) + np.abs(Y0[some]) + np.abs(Z[some])
+        # a complex term is two real ones of each component
+        bound = ((4 if cplx else 1) * K + 8) * U * mag
+        assert (np.abs((got[some] - ref).astype(kind)) <= bound).all()
+        terms = np.sum(np.abs(R * got))
+        assert abs(dot.item() - np.sum((np.conj(R) * got).real)) <= 1e-12 * terms
+    G = rng.standard_normal((len(D), k)).astype(kind)
+    G[:, 1] = 0.0
+    G[0, 1] = 1.0
+    got = H.spmm_adjoint(torch.from_numpy(G).cuda()).cpu().numpy()
+    ref = np.conj(D.T).astype(kind) @ G
+    mag = np.abs(D.T) @ np.abs(G)
+    # both sides are chains of len(D) terms at most (blocked on the host)
+    assert (np.abs(got - ref) <= 2 * (4 if cplx else 1) * len(D) * U * mag).all()
+    assert any("slice_product" in n for n in _kernels(lambda: H.spmm(torch.from_numpy(X).cuda())))
+
+
+@pytest.mark.parametrize("k", [5, 16, 40])
+@pytest.mark.parametrize("b", [9, 13])
+def test_heavy_tailed_panels(b, k):
+    """Panels whose largest entries are far above the rest (Student's t with 2 degrees of
+    freedom): second attempts at most passes, single outputs, items left to multiply-adds."""
+    rng = np.random.default_rng(b * k)
+    wb = 340 // b
+    rows = -(-(1 << 24) // (b * wb * b * (16 if k > 8 else 8)))
+    pat = BlockPattern(np.full(rows, b), np.full(40 * wb, b), np.arange(rows + 1) * wb,
+                       np.sort(np.argsort(rng.random((rows, 40 * wb)), axis=1)[:, :wb], axis=1).reshape(-1))
+    vals = rng.standard_normal(pat.nnz)
+    X = rng.standard_t(2, (pat.n_cols, k))
+    Y0 = rng.standard_normal((pat.n_rows, k))
+    H = _handle(pat, vals)
+    Y = torch.from_numpy(Y0.copy()).cuda()
+    H.spmm(torch.from_numpy(X).cuda(), -2.0, 0.5, Y)
+    got = Y.cpu().numpy()
+    K = wb * b
+    cols = pat.block_col_idx.reshape(rows, wb)
+    for r in range(0, rows, max(rows // 40, 1)):
+        D = vals.reshape(rows, wb, b, b)[r].transpose(1, 0, 2).reshape(b, K).astype(np.longdouble)
+        x = X.reshape(-1, b, k)[cols[r]].reshape(K, k).astype(np.longdouble)
+        ref = -2.0 * (D @ x) + 0.5 * Y0[r * b:(r + 1) * b]
+        mag = 2.0 * (np.abs(D) @ np.abs(x)) + 0.5 * np.abs(Y0[r * b:(r + 1) * b])
+        assert (np.abs(got[r * b:(r + 1) * b] - ref) <= (K + 4) * U * mag).all()
+    assert any("slice_product" in n for n in _kernels(lambda: H.spmm(torch.from_numpy(X).cuda())))
