@@ -294,10 +294,10 @@ int vbcsr_spmm_ex(vbcsr_t *A, int transpose, int64_t k, double alpha, const void
  *  Aop  device [n_rows, k], lda >= k;  Bop  device [n_cols, k], ldb >= k
  *  D    device, nnz elements of the matrix dtype; beta == 0: D is not read
  * FP64 operators of at least 2^22 stored entries x columns, 6 <= k <= 768, and work items
- * of a few hundred entries form it on
- * the tensor cores like the native products, with fixed-point copies of Aop and Bop in a
- * buffer of the handle (8 bytes an element, columns rounded up to 16), allocated and
- * grown on first use as theirs are, and by FMA where those would be.
+ * of a few hundred entries form it on the tensor cores like the native products (an
+ * error within k 2^-53 of sum |a b| and the rounding of the result), with fixed-point
+ * copies of Aop and Bop in a buffer of the handle (8 bytes an element, columns rounded up
+ * to 16), allocated and grown on first use as theirs are, and by FMA where those would be.
  * (This operation has no counterpart in the paper.)
  */
 int vbcsr_sddmm(vbcsr_t *A, int64_t k, double alpha, const void *Aop, int64_t lda,

@@ -17,7 +17,15 @@ namespace vbcsr {
 namespace {
 
 constexpr int kSdDigits = 8;
-constexpr float kSddmmGuard = 16.f;
+// Least sum of |leading digit| products of an output. In units of the last place (2^-63
+// of a scale) a column's term is off by up to 2^62 (the rounding of an operand) and
+// 2^64.8 (7 pairs of level 8 left out), and a one-step sum (k <= 16) by another 2^68 cut
+// off in slice_value: 2^65.2 k + 2^68 together. An estimate G means sum |a b| of at least
+// 0.248 G 2^112 (a leading digit d of a magnitude of (d - 0.502) 2^56 or more), and the
+// error is within k 2^-53 of it, the bound of a k-term chain, from G = 296 + 2060 / k on:
+// 640 at kSddmmMinCols. (At 16, sums of 18 columns were off by up to 160 2^-53. Rows of
+// six normal entries reach 704 but for one output in 10^5.)
+constexpr float kSddmmGuard = 704.f;
 
 // Fixed-point rows of A (blockIdx.y = 0) and B (1): G lanes a row, kp columns
 // (a multiple of 16; columns past k are zero). exps: scale exponent of a row,

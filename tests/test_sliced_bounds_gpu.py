@@ -80,6 +80,25 @@ def test_products_just_above_the_check(K, k):
     assert any("slice_product" in n for n in _kernels(lambda: H.spmm(X)))
 
 
+@pytest.mark.parametrize("k", [6, 16, 18, 40])
+def test_sampled_products_just_above_the_check(k):
+    """Every common column of the two rows has a small leading digit and six of -128."""
+    n = -(-(1 << 22) // (k * 1024)) + 1
+    pat = _uniform(max(n // 4, 1), 1024)
+    for d in (1, 2, 3, 4, 6, 8, 11):
+        e = float((d << 56) - 128 * sum(1 << (8 * i) for i in range(1, 7))) * 2.0 ** -62
+        A = np.full((pat.n_rows, k), e)
+        B = np.full((pat.n_cols, k), e)
+        A[:, 0], A[:, 1], B[:, 0], B[:, 1] = 1.97, 0.0, 0.0, 1.97
+        exact, mag = _sums(A[0], B[0])
+        H = _handle(pat, np.zeros(pat.nnz))
+        got = H.sddmm(torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda()).cpu().numpy()
+        err = max(abs(Fraction(v) - exact) for v in np.unique(got).tolist())
+        assert err <= (k + 2) * Fraction(U) * mag, (d, float(err / mag) / U)
+    assert any("slice_sddmm" in s for s in _kernels(lambda: H.sddmm(torch.from_numpy(A).cuda(),
+                                                                    torch.from_numpy(B).cuda())))
+
+
 @pytest.mark.parametrize("K", [128, 320, 752])
 @pytest.mark.parametrize("fall", [3.0, 7.0, 14.0])
 def test_falling_panels(K, fall, monkeypatch):
