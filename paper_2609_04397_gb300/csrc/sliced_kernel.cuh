@@ -11,7 +11,9 @@ namespace {
 
 constexpr int kSliceList = (kSliceKMax + 16) * sizeof(int32_t);   // X rows of an item and of one step more
 constexpr int kSliceState = 16;   // bytes that a warp keeps from item to item
-constexpr int kSliceSingles = 32; // unresolved outputs of a pass computed one by one
+// unresolved outputs of a pass computed one by one: at most a quarter of the pass (they take
+// about twice the FP64 pipe's time of an item's common multiply-adds, and far more latency)
+constexpr int kSliceSingles = 32;
 constexpr int kSliceStages = 4;   // value tiles in flight per warp (16 columns, up to 1792 bytes each)
 
 // What a warp keeps from item to item, behind its list: [0] the structure of the last item,
@@ -133,7 +135,7 @@ __device__ __noinline__ void slice_digit_sums(const unsigned char *tiles, int B,
 // made a second time with CAREFUL (code that would cost the first one registers): outputs
 // below kSliceGuard are looked at with the sums that their error really depends on
 // (slice_guard), and those that the fixed point does not resolve are computed by
-// slice_one_output, up to kSliceSingles of them (rows of few entries have one now and
+// slice_one_output, a few of them (kSliceSingles; rows of few entries have one now and
 // then: corners of a cluster, 40 to 120 columns; without this the k = 32 product on 50k
 // zinc-blende atoms took 1.52 ms, all 16 columns of such items by multiply-adds). It
 // returns false when there are more or a row has no scale.
@@ -326,7 +328,9 @@ __device__ __forceinline__ bool slice_pass(const ProdArgs &a, const SliceArgs &q
 #pragma unroll
             for (int h = 0; h < NX; ++h)
                 if (e9 != 0 && ec[2 * h] != 0 && nlow[2 * h] < slice_guard(sum[8] + sum[16 + g + 8 * h], K)) bad |= 256u << h;
-        if (!__all_sync(0xffffffffu, scaled) || __reduce_add_sync(0xffffffffu, __popc(bad)) > kSliceSingles) return false;
+        if (!__all_sync(0xffffffffu, scaled) ||
+            __reduce_add_sync(0xffffffffu, __popc(bad)) > min(kSliceSingles, w.B * (WIDE ? 4 : 2)))
+            return false;
         __syncwarp();   // before the next pass's tiles go where the sums were
     }
     auto store = [&](int64_t row, int64_t c, double o) {
@@ -437,7 +441,7 @@ __global__ void __launch_bounds__(128, WIDE ? 3 : 4) slice_product_kernel(const 
         const uint32_t *cmax = q.cmax + (int64_t)si.strct * q.ldp;
         if ((uint32_t)si.strct != state[0]) {
             // a small structure, or one with a column outside the sliced range or mostly tiny, is not sliced
-            const uint32_t most = (uint32_t)q.struct_rows[si.strct] >> 2;
+            const uint32_t most = (uint32_t)q.struct_rows[si.strct] / 8 * 3;
             uint32_t plain = q.struct_nnz[si.strct] < q.min_nnz ? ~0u : 0u;
             for (int c0 = 0; c0 < (int)a.k; c0 += 32) {
                 const int c = c0 + lane;

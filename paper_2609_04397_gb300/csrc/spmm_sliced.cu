@@ -67,8 +67,8 @@ __global__ void __launch_bounds__(256) slice_colmax_kernel(const SliceChunk *chu
 }
 
 // X as biased fixed point [rows, ldp] (8 bytes an element, 7 of them digits);
-// columns k .. ldp - 1 are zero. ccnt counts the elements below 2^-10 of their
-// column's maximum. CPLX: two rows for a row of X, x = (re, im) and i x = (-im, re).
+// columns k .. ldp - 1 are zero. ccnt counts the elements below 2^-kSliceTiny
+// of their column's maximum. CPLX: two rows for a row of X, x = (re, im) and i x = (-im, re).
 template <bool CPLX>
 __global__ void __launch_bounds__(256) slice_panel_kernel(const SliceChunk *chunks, int64_t n_chunks, int per,
                                                           const double *__restrict__ X, int64_t ldx, int k, int ldp,
@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(256) slice_panel_kernel(const SliceChunk *chun
 #pragma unroll 4
                 for (int r = w.ty; r < c.nrows; r += w.TY) {
                     const double v = live ? x[(int64_t)r * ldx] : 0.0;
-                    tiny += live && (slice_mag(v) >> 20) + 10 < (M >> 20);
+                    tiny += live && (slice_mag(v) >> 20) + kSliceTiny < (M >> 20);
                     if (CPLX) {
                         // i x: -im in the real column, re in the imaginary one (the neighbour's value)
                         o[2 * (int64_t)r * ldp] = slice_bytes(v, E);

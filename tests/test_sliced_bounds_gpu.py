@@ -205,3 +205,36 @@ def test_heavy_tailed_panels(b, k):
         mag = 2.0 * (np.abs(D) @ np.abs(x)) + 0.5 * np.abs(Y0[r * b:(r + 1) * b])
         assert (np.abs(got[r * b:(r + 1) * b] - ref) <= (K + 4) * U * mag).all()
     assert any("slice_product" in n for n in _kernels(lambda: H.spmm(torch.from_numpy(X).cuda())))
+
+
+def _time(fn, n=10):
+    fn()
+    best = 1e9
+    for _ in range(5):
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        a.record()
+        for _ in range(n):
+            fn()
+        b.record()
+        torch.cuda.synchronize()
+        best = min(best, a.elapsed_time(b) / n)
+    return best
+
+
+@pytest.mark.parametrize("k", [8, 16])
+def test_panels_of_mostly_tiny_entries_are_not_tried(k):
+    """Columns of 1 and -1 and one entry 2^9 or 2^13 times as large: neither is resolved, both
+    run multiply-adds without a digit product before them."""
+    rng = np.random.default_rng(k)
+    n, wb, b = 6000, 24, 13
+    cols = np.sort((np.arange(n)[:, None] + 7 * np.arange(wb)) % n, axis=1)
+    pat = BlockPattern(np.full(n, b), np.full(n, b), np.arange(n + 1) * wb, cols.reshape(-1))
+    H = _handle(pat, rng.standard_normal(pat.nnz))
+    X = torch.randn(pat.n_cols, k, dtype=torch.float64, device="cuda:0").sign()
+    Y = torch.empty(pat.n_rows, k, dtype=torch.float64, device="cuda:0")
+    times = []
+    for peak in (2.0 ** 9, 2.0 ** 13):
+        X[77] = peak
+        times.append(_time(lambda: H.spmm(X, 1.0, 0.0, Y)))
+        assert any("slice_product" in s for s in _kernels(lambda: H.spmm(X, 1.0, 0.0, Y)))
+    assert times[0] <= 1.05 * times[1], times
