@@ -91,7 +91,7 @@ struct SlicePlan {
     int64_t *struct_nnz = nullptr;  // stored entries of every structure, 0 where its items are too small: [2][structures]
     int64_t max_nnz[2] = {0, 0};    // of the largest structure (kSliceItemNnz[0], [1])
     uint8_t *vdig = nullptr;        // value tiles, built on first use
-    int32_t *rexp = nullptr;        // scale exponent of every output row
+    int32_t *rexp = nullptr;        // scale exponent of every output row, then its parts (SliceArgs::rparts)
     bool no_room = false;           // an allocation failed: keep to the multiply-add kernels
     bool stale = false;             // the values changed since the tiles were built
     bool captured = false;          // a captured product reads the tiles: every change of the values rebuilds them
@@ -943,7 +943,7 @@ static int refresh_slices(vbcsr_t *A, bool trans, cudaStream_t s) {
     const AdjList tl = {A->tl_pbase, A->tl_kp, A->tl_bi, A->tl_xrow, A->tl_vcol};
     CUDA_TRY(launch_slice_values(A->dtype == VBCSR_C128, trans, trans ? A->adj_lpt : A->fwd_lpt, p.items,
                                  trans ? A->n_adj_items : A->n_fwd_items, tl, (const double *)A->panel, p.vdig, p.rexp,
-                                 s),
+                                 p.rexp + (trans ? A->n_cols : A->n_rows), s),
              "slice values");
     return VBCSR_OK;
 }
@@ -988,7 +988,7 @@ static size_t slice_x_elems(const vbcsr_t *A, bool trans, int64_t k) {
     return (size_t)((trans ? A->n_rows : A->n_cols) * slice_ldp(k)) * (A->dtype == VBCSR_C128 ? 2 : 1);
 }
 
-static size_t slice_tab_elems(const vbcsr_t *A, int64_t ldp) { return 4 + 2 * (size_t)A->n_structs * (size_t)ldp; }
+static size_t slice_tab_elems(const vbcsr_t *A, int64_t ldp) { return 4 + 3 * (size_t)A->n_structs * (size_t)ldp; }
 
 static bool slice_buffers_ready(const vbcsr_t *A, bool trans, int64_t k) {
     return A->slice[trans].vdig && A->xdig_elems >= slice_x_elems(A, trans, k) &&
@@ -1235,7 +1235,7 @@ static int slice_prepare(vbcsr_t *A, bool trans, int64_t k, bool may_alloc, cuda
     if (!p.vdig) {
         cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
         CUDA_TRY(cudaThreadExchangeStreamCaptureMode(&mode), "capture mode");
-        cudaError_t e = p.rexp ? cudaSuccess : A->alloc(&p.rexp, (size_t)(trans ? A->n_cols : A->n_rows));
+        cudaError_t e = p.rexp ? cudaSuccess : A->alloc(&p.rexp, 2 * (size_t)(trans ? A->n_cols : A->n_rows));
         if (e == cudaSuccess) e = A->alloc(&p.vdig, (size_t)p.digit_bytes);
         cudaThreadExchangeStreamCaptureMode(&mode);
         if (e != cudaSuccess) rc = cuda_fail(e, "alloc value digits");
@@ -1485,6 +1485,7 @@ static int run_product(vbcsr_t *A, bool trans, int64_t k, double alpha, const vo
         const SlicePlan &p = A->slice[trans];
         const int xld = slice_ldp(kr);
         uint32_t *cmax = A->stab + 4, *ccnt = cmax + (size_t)A->n_structs * xld;
+        uint32_t *cown = ccnt + (size_t)A->n_structs * xld;
         CUDA_TRY(cudaMemsetAsync(A->stab, 0, slice_tab_elems(A, xld) * sizeof(uint32_t), s), "reset column maxima");
         if (cplx) {
             a.k = kr;
@@ -1493,15 +1494,17 @@ static int run_product(vbcsr_t *A, bool trans, int64_t k, double alpha, const vo
             a.ldz *= 2;
             a.ldr *= 2;
         }
-        CUDA_TRY(launch_slice_panel(cplx, p.chunks, p.n_chunks, (const double *)X, a.ldx, (int)kr, xld, cmax, ccnt,
+        CUDA_TRY(launch_slice_panel(cplx, p.chunks, p.n_chunks, (const double *)X, a.ldx, (int)kr, xld, cmax, ccnt, cown,
                                     A->xdig, s),
                  "slice X");
         sa.sitems = p.items;
         sa.vdig = p.vdig;
         sa.rexp = p.rexp;
+        sa.rparts = p.rexp + (trans ? A->n_cols : A->n_rows);
         sa.xdig = A->xdig;
         sa.cmax = cmax;
         sa.ccnt = ccnt;
+        sa.cown = cown;
         sa.struct_rows = p.struct_rows;
         sa.struct_nnz = p.struct_nnz + (slice_small_items(kr, repeated) ? A->n_structs : 0);
         sa.min_nnz = slice_min_nnz(kr, repeated);

@@ -199,8 +199,10 @@ struct SliceArgs {
     const SliceItem *sitems;      // parallel to ProdArgs::items
     const uint8_t *vdig;          // value tiles
     const int32_t *rexp;          // scale exponent of every output row (0: zero row, -1: not sliced)
+    const int32_t *rparts;        // complex: whether a row has real parts (bit 0), imaginary ones (bit 1)
     const uint64_t *xdig;         // fixed-point X, ldp columns
     const uint32_t *cmax, *ccnt;  // [structures, ldp]: high word of the column maxima, tiny elements
+    const uint32_t *cown;         // complex, [structures, ldp]: whether the real column has an entry that is not zero
     const int32_t *struct_rows;   // X rows of every structure
     const int64_t *struct_nnz;    // stored entries of every structure
     int64_t min_nnz;              // slice_min_nnz of this product
@@ -211,9 +213,10 @@ cudaError_t launch_slice_product(bool trans, const ProdArgs &a, const SliceArgs 
 // complex operators: k, ldx and the other leading dimensions count real columns (two a complex one)
 cudaError_t launch_slice_product_c128(bool trans, const ProdArgs &a, const SliceArgs &q, cudaStream_t s);
 cudaError_t launch_slice_panel(bool cplx, const SliceChunk *chunks, int64_t n_chunks, const double *X, int64_t ldx, int k,
-                               int ldp, uint32_t *cmax, uint32_t *ccnt, uint64_t *out, cudaStream_t s);
+                               int ldp, uint32_t *cmax, uint32_t *ccnt, uint32_t *cown, uint64_t *out, cudaStream_t s);
 cudaError_t launch_slice_values(bool cplx, bool trans, const WorkItem *items, const SliceItem *sitems, int64_t n_items,
-                                const AdjList &tl, const double *panel, uint8_t *dig, int32_t *rexp, cudaStream_t s);
+                                const AdjList &tl, const double *panel, uint8_t *dig, int32_t *rexp, int32_t *rparts,
+                                cudaStream_t s);
 const void *slice_kernel_ptr(bool trans, int64_t k);
 const void *slice_c128_kernel_ptr(bool trans, int64_t k);
 size_t slice_smem_bytes();

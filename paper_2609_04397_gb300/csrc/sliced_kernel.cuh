@@ -316,18 +316,28 @@ __device__ __forceinline__ bool slice_pass(const ProdArgs &a, const SliceArgs &q
         int *sum = reinterpret_cast<int *>(ring);
         slice_digit_sums(vsrc, w.B, K, q.xdig, q.ldp, n0, s_x, sum, lane);
         bool scaled = e9 >= 0;
+        // a complex output whose every term has a part that is zero throughout is an exact zero
+        auto zero = [&](int r, int c) {
+            if (sizeof(T) == sizeof(double)) return false;
+            const uint32_t *own = q.cown + (cmax - q.cmax);
+            const int parts = q.rparts[w.yrow + r];
+            return !((parts & 1) && own[n0 + c]) && !((parts & 2) && own[(n0 + c) ^ 1]);
+        };
 #pragma unroll
         for (int n = 0; n < NA; ++n)
 #pragma unroll
             for (int j = 0; j < (PAIR ? 2 : 4); ++j) {
                 scaled &= er[n][j] >= 0;
-                const float guard = slice_guard(sum[row_of(n, j >> 1, j & 1)] + sum[16 + col_of(j >> 1, j & 1)], K);
-                if (er[n][j] != 0 && ec[j] != 0 && low[n][j] < guard) bad |= 1u << (4 * n + j);
+                const int r = row_of(n, j >> 1, j & 1), c = col_of(j >> 1, j & 1);
+                if (er[n][j] != 0 && ec[j] != 0 && low[n][j] < slice_guard(sum[r] + sum[16 + c], K) && !zero(r, c))
+                    bad |= 1u << (4 * n + j);
             }
         if (NINTH && t4 == 0)
 #pragma unroll
             for (int h = 0; h < NX; ++h)
-                if (e9 != 0 && ec[2 * h] != 0 && nlow[2 * h] < slice_guard(sum[8] + sum[16 + g + 8 * h], K)) bad |= 256u << h;
+                if (e9 != 0 && ec[2 * h] != 0 && nlow[2 * h] < slice_guard(sum[8] + sum[16 + g + 8 * h], K) &&
+                    !zero(8, g + 8 * h))
+                    bad |= 256u << h;
         if (!__all_sync(0xffffffffu, scaled) ||
             __reduce_add_sync(0xffffffffu, __popc(bad)) > min(kSliceSingles, w.B * (WIDE ? 4 : 2)))
             return false;

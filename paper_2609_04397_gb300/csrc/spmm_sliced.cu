@@ -37,7 +37,7 @@ __device__ __forceinline__ void over_chunks(const SliceChunk *chunks, int64_t n_
 template <bool CPLX>
 __global__ void __launch_bounds__(256) slice_colmax_kernel(const SliceChunk *chunks, int64_t n_chunks, int per,
                                                            const double *__restrict__ X, int64_t ldx, int k, int ldp,
-                                                           uint32_t *cmax) {
+                                                           uint32_t *cmax, uint32_t *cown) {
     __shared__ uint32_t red[256];
     const ColWalk w(k);
     for (int c0 = 0; c0 < k; c0 += w.TX) {
@@ -59,7 +59,10 @@ __global__ void __launch_bounds__(256) slice_colmax_kernel(const SliceChunk *chu
             }
             if (w.ty == 0 && col < k && red[w.tx]) {
                 atomicMax(cmax + (int64_t)c.strct * ldp + col, red[w.tx]);
-                if (CPLX) atomicMax(cmax + (int64_t)c.strct * ldp + (col ^ 1), red[w.tx]);
+                if (CPLX) {
+                    atomicMax(cmax + (int64_t)c.strct * ldp + (col ^ 1), red[w.tx]);
+                    cown[(int64_t)c.strct * ldp + col] = 1;   // a part that is not all zero
+                }
             }
             m = 0;
         });
@@ -68,7 +71,9 @@ __global__ void __launch_bounds__(256) slice_colmax_kernel(const SliceChunk *chu
 
 // X as biased fixed point [rows, ldp] (8 bytes an element, 7 of them digits);
 // columns k .. ldp - 1 are zero. ccnt counts the elements below 2^-kSliceTiny
-// of their column's maximum. CPLX: two rows for a row of X, x = (re, im) and i x = (-im, re).
+// of their column's maximum (CPLX: of which both parts are: a real panel's zero imaginary
+// parts are not resolved worse for it). CPLX: two rows for a row of X, x = (re, im) and
+// i x = (-im, re).
 template <bool CPLX>
 __global__ void __launch_bounds__(256) slice_panel_kernel(const SliceChunk *chunks, int64_t n_chunks, int per,
                                                           const double *__restrict__ X, int64_t ldx, int k, int ldp,
@@ -89,15 +94,17 @@ __global__ void __launch_bounds__(256) slice_panel_kernel(const SliceChunk *chun
 #pragma unroll 4
                 for (int r = w.ty; r < c.nrows; r += w.TY) {
                     const double v = live ? x[(int64_t)r * ldx] : 0.0;
-                    tiny += live && (slice_mag(v) >> 20) + kSliceTiny < (M >> 20);
+                    uint32_t mag = slice_mag(v);
                     if (CPLX) {
                         // i x: -im in the real column, re in the imaginary one (the neighbour's value)
                         o[2 * (int64_t)r * ldp] = slice_bytes(v, E);
                         const double u = live ? x[(int64_t)r * ldx + (col & 1 ? -1 : 1)] : 0.0;
+                        mag = max(mag, slice_mag(u));
                         o[(2 * (int64_t)r + 1) * ldp] = slice_bytes(col & 1 ? u : -u, E);
                     } else {
                         o[(int64_t)r * ldp] = slice_bytes(v, E);
                     }
+                    tiny += live && (mag >> 20) + kSliceTiny < (M >> 20);
                 }
             }
             if (!last) return;
@@ -149,7 +156,7 @@ __device__ __forceinline__ void adj_columns(const double *panel, const int64_t *
 
 template <int BP, bool CPLX>
 __device__ __forceinline__ void adj_item_digits(const double *panel, const int64_t *s_a, const WorkItem &w, uint8_t *dst,
-                                                uint8_t *stage, int32_t *rexp, int lane) {
+                                                uint8_t *stage, int32_t *rexp, int32_t *rparts, int lane) {
     const int K = CPLX ? 2 * w.K : w.K;
     uint32_t m = 0;
     for (int t0 = 0; t0 < K; t0 += 32) {
@@ -159,7 +166,11 @@ __device__ __forceinline__ void adj_item_digits(const double *panel, const int64
         for (int u = 0; u < BP; ++u) m = max(m, slice_mag(v[u]));
     }
 #pragma unroll
-    for (int h = BP; h < 32; h <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, h));
+    for (int h = 2 * BP; h < 32; h <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, h));
+    // lanes BP apart hold neighbouring virtual columns (CPLX: the two parts of a value)
+    const uint32_t other = __shfl_xor_sync(0xffffffffu, m, BP);
+    if (CPLX && lane < w.B) rparts[w.yrow + lane] = (m != 0) | (other != 0) << 1;
+    m = max(m, other);
     const int E = m == 0 ? 0 : (slice_exp_ok(m) ? slice_exp(m) : -1), q = lane % BP;
     if (lane < w.B) rexp[w.yrow + lane] = E;
     const int nt = (K + 15) >> 4;
@@ -182,7 +193,7 @@ __device__ __forceinline__ void adj_item_digits(const double *panel, const int64
 template <bool TRANS, bool CPLX>
 __global__ void __launch_bounds__(128) slice_values_kernel(const WorkItem *items, const SliceItem *sitems,
                                                            int64_t n_items, AdjList tl, const double *panel,
-                                                           uint8_t *dig, int32_t *rexp) {
+                                                           uint8_t *dig, int32_t *rexp, int32_t *rparts) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int warps = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint8_t *stage = smem_raw + (size_t)warp * 32 * kSliceTile;
@@ -202,10 +213,10 @@ __global__ void __launch_bounds__(128) slice_values_kernel(const WorkItem *items
             }
             __syncwarp();
             uint8_t *dst = dig + si.doff;
-            if (w.B > 8) adj_item_digits<16, CPLX>(panel, s_a, w, dst, stage, rexp, lane);
-            else if (w.B > 4) adj_item_digits<8, CPLX>(panel, s_a, w, dst, stage, rexp, lane);
-            else if (w.B > 2) adj_item_digits<4, CPLX>(panel, s_a, w, dst, stage, rexp, lane);
-            else adj_item_digits<2, CPLX>(panel, s_a, w, dst, stage, rexp, lane);
+            if (w.B > 8) adj_item_digits<16, CPLX>(panel, s_a, w, dst, stage, rexp, rparts, lane);
+            else if (w.B > 4) adj_item_digits<8, CPLX>(panel, s_a, w, dst, stage, rexp, rparts, lane);
+            else if (w.B > 2) adj_item_digits<4, CPLX>(panel, s_a, w, dst, stage, rexp, rparts, lane);
+            else adj_item_digits<2, CPLX>(panel, s_a, w, dst, stage, rexp, rparts, lane);
         } else {
             constexpr int cw = CPLX ? 2 : 1;
             const int K = cw * w.K;
@@ -228,6 +239,11 @@ __global__ void __launch_bounds__(128) slice_values_kernel(const WorkItem *items
 #pragma unroll
             for (int p = 0; p < 16; ++p) {
                 const uint32_t r = __reduce_max_sync(0xffffffffu, m[p]);
+                if (CPLX) {   // even lanes hold the real parts
+                    const unsigned any = __ballot_sync(0xffffffffu, m[p] != 0);
+                    if (lane == p && p < w.B)
+                        rparts[w.yrow + p] = ((any & 0x55555555u) != 0) | ((any & 0xaaaaaaaau) != 0) << 1;
+                }
                 const int e = r == 0 ? 0 : (slice_exp_ok(r) ? slice_exp(r) : -1);
                 if (lane == p) {
                     s_e[warp][p] = e;
@@ -267,16 +283,16 @@ cudaError_t launch_slice_product(bool trans, const ProdArgs &a, const SliceArgs 
 }
 
 cudaError_t launch_slice_panel(bool cplx, const SliceChunk *chunks, int64_t n_chunks, const double *X, int64_t ldx, int k,
-                               int ldp, uint32_t *cmax, uint32_t *ccnt, uint64_t *out, cudaStream_t s) {
+                               int ldp, uint32_t *cmax, uint32_t *ccnt, uint32_t *cown, uint64_t *out, cudaStream_t s) {
     if (n_chunks == 0) return cudaSuccess;
     // about 2048 elements a CTA: several chunks of narrow panels
     const int per = k >= 8 ? 1 : 8 / k;
     const unsigned grid = (unsigned)((n_chunks + per - 1) / per);
     if (cplx) {
-        slice_colmax_kernel<true><<<grid, 256, 0, s>>>(chunks, n_chunks, per, X, ldx, k, ldp, cmax);
+        slice_colmax_kernel<true><<<grid, 256, 0, s>>>(chunks, n_chunks, per, X, ldx, k, ldp, cmax, cown);
         slice_panel_kernel<true><<<grid, 256, 0, s>>>(chunks, n_chunks, per, X, ldx, k, ldp, cmax, ccnt, out);
     } else {
-        slice_colmax_kernel<false><<<grid, 256, 0, s>>>(chunks, n_chunks, per, X, ldx, k, ldp, cmax);
+        slice_colmax_kernel<false><<<grid, 256, 0, s>>>(chunks, n_chunks, per, X, ldx, k, ldp, cmax, cown);
         slice_panel_kernel<false><<<grid, 256, 0, s>>>(chunks, n_chunks, per, X, ldx, k, ldp, cmax, ccnt, out);
     }
     return cudaGetLastError();
@@ -284,7 +300,7 @@ cudaError_t launch_slice_panel(bool cplx, const SliceChunk *chunks, int64_t n_ch
 
 template <bool TRANS, bool CPLX>
 static cudaError_t values_launch(const WorkItem *items, const SliceItem *sitems, int64_t n_items, const AdjList &tl,
-                                 const double *panel, uint8_t *dig, int32_t *rexp, cudaStream_t s) {
+                                 const double *panel, uint8_t *dig, int32_t *rexp, int32_t *rparts, cudaStream_t s) {
     const int warps = 4;
     const size_t smem = (size_t)warps * (32 * kSliceTile + (TRANS ? kSliceKMax * sizeof(int64_t) : 0));
     cudaError_t e = cudaFuncSetAttribute((const void *)slice_values_kernel<TRANS, CPLX>,
@@ -292,18 +308,19 @@ static cudaError_t values_launch(const WorkItem *items, const SliceItem *sitems,
     if (e != cudaSuccess) return e;
     const int64_t need = (n_items + warps - 1) / warps;
     slice_values_kernel<TRANS, CPLX><<<(unsigned)(need < 65535 ? need : 65535), warps * 32, smem, s>>>(
-        items, sitems, n_items, tl, panel, dig, rexp);
+        items, sitems, n_items, tl, panel, dig, rexp, rparts);
     return cudaGetLastError();
 }
 
 cudaError_t launch_slice_values(bool cplx, bool trans, const WorkItem *items, const SliceItem *sitems, int64_t n_items,
-                                const AdjList &tl, const double *panel, uint8_t *dig, int32_t *rexp, cudaStream_t s) {
+                                const AdjList &tl, const double *panel, uint8_t *dig, int32_t *rexp, int32_t *rparts,
+                                cudaStream_t s) {
     if (n_items == 0) return cudaSuccess;
     if (cplx)
-        return trans ? values_launch<true, true>(items, sitems, n_items, tl, panel, dig, rexp, s)
-                     : values_launch<false, true>(items, sitems, n_items, tl, panel, dig, rexp, s);
-    return trans ? values_launch<true, false>(items, sitems, n_items, tl, panel, dig, rexp, s)
-                 : values_launch<false, false>(items, sitems, n_items, tl, panel, dig, rexp, s);
+        return trans ? values_launch<true, true>(items, sitems, n_items, tl, panel, dig, rexp, rparts, s)
+                     : values_launch<false, true>(items, sitems, n_items, tl, panel, dig, rexp, rparts, s);
+    return trans ? values_launch<true, false>(items, sitems, n_items, tl, panel, dig, rexp, rparts, s)
+                 : values_launch<false, false>(items, sitems, n_items, tl, panel, dig, rexp, rparts, s);
 }
 
 }  // namespace vbcsr

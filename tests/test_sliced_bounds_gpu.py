@@ -238,3 +238,37 @@ def test_panels_of_mostly_tiny_entries_are_not_tried(k):
         times.append(_time(lambda: H.spmm(X, 1.0, 0.0, Y)))
         assert any("slice_product" in s for s in _kernels(lambda: H.spmm(X, 1.0, 0.0, Y)))
     assert times[0] <= 1.05 * times[1], times
+
+
+@pytest.mark.parametrize("k", [5, 8, 13])
+@pytest.mark.parametrize("kpoint", [[0.13, -0.27, 0.41], [0.0, 0.0, 0.0]])
+def test_real_panels_of_complex_operators_are_sliced(k, kpoint):
+    """Zero imaginary parts are no reason for multiply-adds (a panel of unit columns takes
+    them and gives their time), nor are the outputs that they make exact zeros where the
+    operator is real as well."""
+    import oracle
+    import synthetic as syn
+    from paper_2609_04397_gb300 import VBCSR
+    w = syn.zincblende_crystal(8)
+    H = VBCSR.from_images(w.bsize, w.edge_i, w.edge_j, w.edge_R, w.edge_values, device="cuda:0")
+    H.set_kpoint(kpoint)
+    rb, cb, rp, ci = H.pattern
+    pat = BlockPattern(rb, cb, rp, ci)
+    rng = np.random.default_rng(k)
+    full = rng.standard_normal((pat.n_rows, k)) + 1j * rng.standard_normal((pat.n_rows, k))
+    vals = H.get_values().cpu().numpy()
+    assert any(kpoint) or (vals.imag == 0).all()
+    times = {}
+    unit = np.eye(pat.n_rows, k, dtype=complex)
+    for name, P in (("real", full.real.astype(complex)), ("nearly real", full.real + 1e-9j * full.imag), ("unit", unit)):
+        Xd = torch.from_numpy(P).cuda()
+        Y = torch.empty_like(Xd)
+        for fn, ref in ((H.spmm, oracle.spmm_complex), (H.spmm_adjoint, oracle.spmm_adjoint_complex)):
+            got = fn(Xd, 1.0, 0.0, Y).cpu().numpy()
+            mag = (oracle.spmm if fn == H.spmm else oracle.spmm_adjoint)(pat, np.abs(vals), np.abs(P))
+            # two chains of at most 2 x 380 terms
+            assert (np.abs(got - ref(pat, vals, P)) <= 4 * 760 * U * mag).all(), name
+            if not any(kpoint) and name == "real":
+                assert (got.imag == 0).all()
+        times[name] = _time(lambda: H.spmm(Xd, 1.0, 0.0, Y))
+    assert times["real"] <= 0.85 * times["unit"], times
