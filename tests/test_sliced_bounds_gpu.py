@@ -272,3 +272,43 @@ def test_real_panels_of_complex_operators_are_sliced(k, kpoint):
                 assert (got.imag == 0).all()
         times[name] = _time(lambda: H.spmm(Xd, 1.0, 0.0, Y))
     assert times["real"] <= 0.85 * times["unit"], times
+
+
+@pytest.mark.parametrize("k", [17, 33, 40, 560])
+def test_one_bad_column_leaves_the_other_passes_sliced(k):
+    """A column with a NaN, an Inf or one entry only sends its own 16 columns to multiply-adds:
+    the bits of the others are those of a panel without it (from column 496 on a panel's
+    columns are taken together)."""
+    rng = np.random.default_rng(k)
+    n, wb, b = 400, 24, 13
+    cols = np.sort((np.arange(n)[:, None] + 7 * np.arange(wb)) % n, axis=1)
+    pat = BlockPattern(np.full(n, b), np.full(n, b), np.arange(n + 1) * wb, cols.reshape(-1))
+    vals = rng.standard_normal(pat.nnz)
+    H = _handle(pat, vals)
+    X = rng.standard_normal((pat.n_cols, k))
+    clean = H.spmm(torch.from_numpy(X).cuda()).cpu().numpy()
+    import oracle
+    for bad in sorted({0, 16, k - 1, min(k - 1, 500)}):
+        for kind in ("nan", "inf", "unit"):
+            Z = X.copy()
+            if kind == "unit":
+                Z[:, bad] = 0.0
+                Z[7, bad] = 1.0
+            else:
+                Z[7, bad] = float(kind)
+            got = H.spmm(torch.from_numpy(Z).cuda()).cpu().numpy()
+            lo = 16 * (bad // 16)
+            hi = lo + 16
+            if bad >= 496:
+                lo, hi = 496, k
+            same = np.r_[0:lo, min(hi, k):k]
+            assert np.array_equal(got[:, same], clean[:, same]), (bad, kind)
+            own = slice(lo, min(hi, k, lo + 16))
+            with np.errstate(invalid="ignore"):
+                ref = oracle.spmm(pat, vals, np.ascontiguousarray(Z[:, own]))
+            mag = oracle.spmm(pat, np.abs(vals), np.abs(np.ascontiguousarray(Z[:, own])))
+            assert np.array_equal(np.isnan(got[:, own]), np.isnan(ref))
+            fin = np.isfinite(ref)
+            # two chains of 312 terms
+            assert (np.abs(got[:, own][fin] - ref[fin]) <= 640 * U * mag[fin]).all(), (bad, kind)
+    assert any("slice_product" in s for s in _kernels(lambda: H.spmm(torch.from_numpy(X).cuda())))
