@@ -80,6 +80,19 @@ struct DevBuf {
     size_t bytes = 0;
 };
 
+// Allocations of one buffer of the sliced products, without which they run multiply-adds:
+// the least size that failed is not asked for again for a while (a shortage can pass: a
+// caching allocator that gives memory back), smaller ones are.
+struct Room {
+    size_t failed = SIZE_MAX;
+    int calls = 0;
+    bool may_try(size_t bytes) { return bytes < failed || ++calls % 64 == 0; }
+    void result(size_t bytes, bool ok) {
+        if (!ok) failed = std::min(failed, bytes);
+        else if (bytes >= failed) failed = SIZE_MAX;
+    }
+};
+
 // One direction (forward, adjoint) of the sliced FP64 products
 struct SlicePlan {
     bool applies = false;           // the planner's rule: nearly all of the work is in rows narrow enough
@@ -92,7 +105,7 @@ struct SlicePlan {
     int64_t max_nnz[2] = {0, 0};    // of the largest structure (kSliceItemNnz[0], [1])
     uint8_t *vdig = nullptr;        // value tiles, built on first use
     int32_t *rexp = nullptr;        // scale exponent of every output row, then its parts (SliceArgs::rparts)
-    bool no_room = false;           // an allocation failed: keep to the multiply-add kernels
+    Room room;                      // of vdig
     bool stale = false;             // the values changed since the tiles were built
     bool captured = false;          // a captured product reads the tiles: every change of the values rebuilds them
     bool untracked = false;         // a capture changes the values with no tiles to rebuild: multiply-adds only
@@ -157,7 +170,7 @@ struct vbcsr_matrix {
     uint64_t *sdpan = nullptr;   // fixed-point rows of A and B of the sliced pattern-sampled product
     size_t sdpan_elems = 0;
     bool xdig_captured = false, stab_captured = false, sdpan_captured = false;   // a graph holds the buffer
-    bool sd_no_room = false;
+    Room xdig_room, stab_room, sdpan_room;
     uint32_t *stab = nullptr;
     size_t stab_elems = 0;
     WorkItem *fwd_items = nullptr, *adj_items = nullptr;   // bucketed by row count
@@ -908,33 +921,57 @@ static int grow(vbcsr_t *A, T **buf, size_t *have, size_t need, cudaStream_t s, 
     return VBCSR_OK;
 }
 
-// The same for a buffer of the native products, which need none without slicing: graphs
-// that hold the old one (*captured) stay valid, so it is kept until the handle goes, and
-// the new one is at least twice its size (what is kept stays below what is in use).
-// A capture on another thread is not disturbed by the allocation.
+// An optional allocation: *p stays NULL when the device has no room. A capture on another
+// thread is not disturbed by it.
 template <typename T>
-static int grow_native(vbcsr_t *A, T **buf, size_t *have, size_t need, bool *captured, cudaStream_t s,
-                       const char *what) {
-    if (need <= *have) return VBCSR_OK;
+static int alloc_optional(vbcsr_t *A, T **p, size_t count, Room *room, const char *what) {
+    *p = nullptr;
+    if (!room->may_try(count * sizeof(T))) return VBCSR_OK;
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     CUDA_TRY(cudaThreadExchangeStreamCaptureMode(&mode), "capture mode");
-    int rc = VBCSR_OK;
-    if (*captured) {
-        T *more = nullptr;
-        const size_t n = std::max(need, 2 * *have);
-        const cudaError_t e = A->alloc(&more, n);
-        if (e == cudaSuccess) {
-            *buf = more;
-            *have = n;
-            *captured = false;
-        } else {
-            rc = cuda_fail(e, what);
-        }
-    } else {
-        rc = grow(A, buf, have, need, s, what);
-    }
+    const cudaError_t e = A->alloc(p, count);
+    if (e == cudaErrorMemoryAllocation) cudaGetLastError();
     cudaThreadExchangeStreamCaptureMode(&mode);
-    return rc;
+    if (e != cudaSuccess && e != cudaErrorMemoryAllocation) return cuda_fail(e, what);
+    room->result(count * sizeof(T), e == cudaSuccess);
+    return VBCSR_OK;
+}
+
+static void release(vbcsr_t *A, void *p) {
+    for (auto &b : A->bufs)
+        if (p && b.p == p) {
+            cudaFree(b.p);
+            A->device_bytes -= (int64_t)b.bytes;
+            b.p = nullptr;
+        }
+}
+
+// The same as grow for a buffer of the native products, which need none without slicing
+// (*have stays as it is when there is no room): graphs that hold the old one (*captured) stay
+// valid, so it is kept until the handle goes, and the new one is twice its size where that
+// fits (what is kept stays below what is in use). A wider call that does not fit leaves the
+// narrower ones their buffer.
+template <typename T>
+static int grow_native(vbcsr_t *A, T **buf, size_t *have, size_t need, bool *captured, Room *room, cudaStream_t s,
+                       const char *what) {
+    if (need <= *have) return VBCSR_OK;
+    T *more = nullptr;
+    size_t n = *captured ? std::max(need, 2 * *have) : need;
+    int rc = alloc_optional(A, &more, n, room, what);
+    if (!rc && !more && n > need) rc = alloc_optional(A, &more, n = need, room, what);
+    if (rc || !more) return rc;
+    if (!*captured && *buf) {
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        CUDA_TRY(cudaThreadExchangeStreamCaptureMode(&mode), "capture mode");
+        const cudaError_t e = cudaStreamSynchronize(s);
+        if (e == cudaSuccess) release(A, *buf);
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        CUDA_TRY(e, "synchronize");
+    }
+    *buf = more;
+    *have = n;
+    *captured = false;
+    return VBCSR_OK;
 }
 
 // The digit tiles of one direction, from the values now in the pages
@@ -998,7 +1035,7 @@ static bool slice_buffers_ready(const vbcsr_t *A, bool trans, int64_t k) {
 // Builds what a sliced product needs and is missing (*ready = true when it can
 // run). Nothing is allocated while the stream is being captured or when the
 // caller must not allocate; when the device has no room, the product runs
-// multiply-adds from then on.
+// multiply-adds.
 static int slice_prepare(vbcsr_t *A, bool trans, int64_t k, bool may_alloc, cudaStream_t s, bool *ready);
 
 extern "C" int vbcsr_set_values(vbcsr_t *A, const void *values, int on_device, void *stream) {
@@ -1230,34 +1267,26 @@ static int slice_prepare(vbcsr_t *A, bool trans, int64_t k, bool may_alloc, cuda
         }
         return VBCSR_OK;
     }
-    if (!may_alloc || p.no_room || cap) return VBCSR_OK;
+    if (!may_alloc || cap) return VBCSR_OK;
     int rc = VBCSR_OK;
-    if (!p.vdig) {
-        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-        CUDA_TRY(cudaThreadExchangeStreamCaptureMode(&mode), "capture mode");
-        cudaError_t e = p.rexp ? cudaSuccess : A->alloc(&p.rexp, 2 * (size_t)(trans ? A->n_cols : A->n_rows));
-        if (e == cudaSuccess) e = A->alloc(&p.vdig, (size_t)p.digit_bytes);
-        cudaThreadExchangeStreamCaptureMode(&mode);
-        if (e != cudaSuccess) rc = cuda_fail(e, "alloc value digits");
+    if (!p.rexp) rc = alloc_optional(A, &p.rexp, 2 * (size_t)(trans ? A->n_cols : A->n_rows), &p.room, "alloc scales");
+    if (!rc && p.rexp && !p.vdig) {
+        rc = alloc_optional(A, &p.vdig, (size_t)p.digit_bytes, &p.room, "alloc value digits");
         p.stale = p.vdig != nullptr;
     }
-    if (!rc && p.stale) {
+    if (!rc && p.vdig)
+        rc = grow_native(A, &A->xdig, &A->xdig_elems, slice_x_elems(A, trans, k), &A->xdig_captured, &A->xdig_room, s,
+                         "alloc fixed-point X");
+    if (!rc && p.vdig)
+        rc = grow_native(A, &A->stab, &A->stab_elems, slice_tab_elems(A, slice_ldp(k)), &A->stab_captured,
+                         &A->stab_room, s, "alloc column maxima");
+    if (rc) return rc;
+    *ready = slice_buffers_ready(A, trans, k);
+    if (*ready && p.stale) {
         rc = refresh_slices(A, trans, s);
         p.stale = rc != VBCSR_OK;
     }
-    if (!rc)
-        rc = grow_native(A, &A->xdig, &A->xdig_elems, slice_x_elems(A, trans, k), &A->xdig_captured, s,
-                         "alloc fixed-point X");
-    if (!rc)
-        rc = grow_native(A, &A->stab, &A->stab_elems, slice_tab_elems(A, slice_ldp(k)), &A->stab_captured, s,
-                         "alloc column maxima");
-    if (rc == VBCSR_ERR_NO_MEMORY) {
-        p.no_room = true;
-        return VBCSR_OK;
-    }
-    if (rc) return rc;
-    *ready = true;
-    return VBCSR_OK;
+    return rc;
 }
 
 static int run_product(vbcsr_t *A, bool trans, int64_t k, double alpha, const void *X, int64_t ldx, double beta,
@@ -1652,20 +1681,12 @@ static int run_sddmm_f64(vbcsr_t *A, const SddmmArgs &a, cudaStream_t s) {
     if (sliced) {
         const int64_t kp = (a.k + 15) / 16 * 16, rows = A->n_rows + A->n_cols;
         const size_t need = (size_t)(rows * kp + (rows + 1) / 2);
-        if (need > A->sdpan_elems) {
-            if (A->sd_no_room || capturing(s)) {
-                sliced = false;
-            } else {
-                const int rc = grow_native(A, &A->sdpan, &A->sdpan_elems, need, &A->sdpan_captured, s,
-                                           "alloc fixed-point panels");
-                if (rc == VBCSR_ERR_NO_MEMORY) {
-                    A->sd_no_room = true;
-                    sliced = false;
-                } else if (rc) {
-                    return rc;
-                }
-            }
+        if (need > A->sdpan_elems && !capturing(s)) {
+            const int rc = grow_native(A, &A->sdpan, &A->sdpan_elems, need, &A->sdpan_captured, &A->sdpan_room, s,
+                                       "alloc fixed-point panels");
+            if (rc) return rc;
         }
+        sliced = need <= A->sdpan_elems;
         if (sliced) {
             A->sdpan_captured |= capturing(s);
             uint64_t *fa = A->sdpan, *fb = fa + A->n_rows * kp;

@@ -312,3 +312,47 @@ def test_one_bad_column_leaves_the_other_passes_sliced(k):
             # two chains of 312 terms
             assert (np.abs(got[:, own][fin] - ref[fin]) <= 640 * U * mag[fin]).all(), (bad, kind)
     assert any("slice_product" in s for s in _kernels(lambda: H.spmm(torch.from_numpy(X).cuda())))
+
+
+def test_panel_that_does_not_fit_leaves_narrower_ones_sliced():
+    """With the device almost full a wide product and a wide sampled one run multiply-adds;
+    narrower ones keep their buffers, and the wide ones are sliced again when there is room."""
+    import synthetic as syn
+    w = syn.amorphous(700, side=60.0 * (700 / 20000) ** (1 / 3))
+    H = _handle(w.pattern, w.values)
+    k, wide = 16, 8192
+    X, A = (torch.randn(w.pattern.n_rows, wide, dtype=torch.float64, device="cuda:0") for _ in range(2))
+    Xk, Ak, Xs, As = X[:, :k].contiguous(), A[:, :k].contiguous(), X[:, :700].contiguous(), A[:, :700].contiguous()
+    Y, D = torch.empty_like(X), torch.empty(w.pattern.nnz, dtype=torch.float64, device="cuda:0")
+    first = H.spmm(Xk)
+    H.sddmm(Ak, Xk)
+    Yp = torch.cat([H.spmm(X[:, c:c + 4].contiguous()) for c in range(0, 64, 4)], 1)   # multiply-adds
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    leave = 24 << 20
+    full = []
+    for part in (1 << 32, 1 << 28, 1 << 24):
+        while torch.cuda.mem_get_info()[0] > leave + part:
+            full.append(torch.empty(part, dtype=torch.uint8, device="cuda:0"))
+    H.spmm(X, 1.0, 0.0, Y)
+    H.sddmm(As, Xs, 1.0, 0.0, D)
+    again = torch.empty_like(first)
+    H.spmm(Xk, 1.0, 0.0, again)
+    torch.cuda.synchronize()
+    full.clear()
+    torch.cuda.empty_cache()
+    bound = 1600 * U * H_abs_product(w, X[:, :64])   # two chains of at most 768 terms
+    assert ((Y[:, :64] - Yp).abs() <= bound).all()
+    assert torch.equal(again, first)
+    names = _kernels(lambda: (H.spmm(Xk), H.sddmm(Ak, Xk)))
+    assert any("slice_product" in s for s in names) and any("slice_sddmm" in s for s in names)
+    for _ in range(70):
+        H.spmm(X, 1.0, 0.0, Y)
+        H.sddmm(As, Xs, 1.0, 0.0, D)
+    names = _kernels(lambda: (H.spmm(X, 1.0, 0.0, Y), H.sddmm(As, Xs, 1.0, 0.0, D)))
+    assert any("slice_product" in s for s in names) and any("slice_sddmm" in s for s in names)
+
+
+def H_abs_product(w, X):
+    """sum |h x| of every output"""
+    return _handle(w.pattern, np.abs(w.values)).spmm(X.abs().contiguous())
