@@ -542,8 +542,8 @@ int vbcsr_get_tuning(const vbcsr_t *A, int32_t *kc_by_b, int32_t *warps_by_b, in
  * whichever schedule is faster (unless flags has VBCSR_TUNE_NO_PERSISTENT).
  * X and Y are device panels of the product's shapes; Y is overwritten. The
  * call synchronises `stream` repeatedly (a set-up step: do not capture it in
- * a CUDA graph). A native FP64 product that runs on the tensor cores takes the
- * same time in every trial. For the tensor-core precisions it only chooses, for the
+ * a CUDA graph). The trials of a native FP64 product run by FMA at every size: the
+ * tiles serve the products that do. For the tensor-core precisions it only chooses, for the
  * forward product, between the plain and the shared-memory-staged kernel.
  * (The per-shape-group tuning of tiles has no counterpart in the paper.)
  */

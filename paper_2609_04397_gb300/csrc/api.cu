@@ -169,6 +169,7 @@ struct vbcsr_matrix {
     size_t xdig_elems = 0;
     uint64_t *sdpan = nullptr;   // fixed-point rows of A and B of the sliced pattern-sampled product
     size_t sdpan_elems = 0;
+    bool tuning = false;         // vbcsr_autotune times the multiply-add kernels
     bool xdig_captured = false, stab_captured = false, sdpan_captured = false;   // a graph holds the buffer
     Room xdig_room, stab_room, sdpan_room;
     uint32_t *stab = nullptr;
@@ -1016,7 +1017,7 @@ static int slices_changed(vbcsr_t *A, cudaStream_t s) {
 // True when a native FP64 product of k columns runs sliced.
 static bool slice_applies(const vbcsr_t *A, bool trans, int64_t k, bool repeated) {
     const SlicePlan &p = A->slice[trans];
-    return p.applies && !p.untracked && k <= (1 << 20) &&
+    return p.applies && !p.untracked && !A->tuning && k <= (1 << 20) &&
            p.max_nnz[slice_small_items(k, repeated)] >= slice_min_nnz(k, repeated) && !A->debug_checks;
 }
 
@@ -2386,6 +2387,13 @@ extern "C" int vbcsr_autotune(vbcsr_t *A, int transpose, int64_t k, const void *
     }
     cudaStream_t s = (cudaStream_t)stream;
     const bool trans = transpose == 1;
+    // the tiles and the schedule are those of the multiply-adds, which narrower products and
+    // what is not sliced still run: timing sliced products would pick them by chance
+    struct Tuning {
+        vbcsr_matrix *A;
+        explicit Tuning(vbcsr_matrix *m) : A(m) { A->tuning = true; }
+        ~Tuning() { A->tuning = false; }
+    } tuning(A);
     const int reps = 3;
     const int kcs[] = {1, 2, 4, 8, 16, 32};
     const int wss[] = {2, 4, 8};

@@ -356,3 +356,19 @@ def test_panel_that_does_not_fit_leaves_narrower_ones_sliced():
 def H_abs_product(w, X):
     """sum |h x| of every output"""
     return _handle(w.pattern, np.abs(w.values)).spmm(X.abs().contiguous())
+
+
+def _amorphous():
+    import synthetic as syn
+    w = syn.amorphous(700, side=60.0 * (700 / 20000) ** (1 / 3))
+    return w, _handle(w.pattern, w.values)
+
+
+def test_autotune_times_the_multiply_adds():
+    """At a width that runs sliced the tuner still chooses the multiply-adds' tiles by their
+    own times: narrower products use them."""
+    w, H = _amorphous()
+    X = torch.randn(w.pattern.n_cols, 16, dtype=torch.float64, device="cuda:0")
+    names = _kernels(lambda: H.autotune(16))
+    assert any("fma" in s for s in names) and not any("slice" in s for s in names)
+    assert any("slice_product" in s for s in _kernels(lambda: H.spmm(X)))
