@@ -108,7 +108,8 @@ struct SlicePlan {
     Room room;                      // of vdig
     bool stale = false;             // the values changed since the tiles were built
     bool captured = false;          // a captured product reads the tiles: every change of the values rebuilds them
-    bool untracked = false;         // a capture changes the values with no tiles to rebuild: multiply-adds only
+    bool untracked = false;         // a capture changes the values with no tiles to rebuild: every call rebuilds them
+    unsigned long long capture = 0; // the capture that holds a rebuild of stale tiles
 };
 
 }  // namespace
@@ -986,16 +987,21 @@ static int refresh_slices(vbcsr_t *A, bool trans, cudaStream_t s) {
     return VBCSR_OK;
 }
 
-static bool capturing(cudaStream_t s) {
+// (*id: of the capture)
+static bool capturing(cudaStream_t s, unsigned long long *id = nullptr) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    return cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+    unsigned long long at = 0;
+    const bool known = cudaStreamGetCaptureInfo(s, &cap, &at) == cudaSuccess;
+    if (id) *id = at;
+    return !known || cap != cudaStreamCaptureStatusNone;
 }
 
 // The pages have (or, under capture, will have) new values. The tiles are
 // rebuilt by the next product that reads them: a training step that sets the
 // values twice and uses one direction each time builds each once. Tiles that a
 // captured product reads, and changes that are themselves captured, are rebuilt
-// here, since the host does not see the replays.
+// here, since the host does not see the replays. A captured change with no tiles to
+// rebuild makes every later call rebuild them first (untracked): a recurrence once.
 static int slices_changed(vbcsr_t *A, cudaStream_t s) {
     for (int t = 0; t < 2; ++t) {
         SlicePlan &p = A->slice[t];
@@ -1017,8 +1023,13 @@ static int slices_changed(vbcsr_t *A, cudaStream_t s) {
 // True when a native FP64 product of k columns runs sliced.
 static bool slice_applies(const vbcsr_t *A, bool trans, int64_t k, bool repeated) {
     const SlicePlan &p = A->slice[trans];
-    return p.applies && !p.untracked && !A->tuning && k <= (1 << 20) &&
+    return p.applies && !A->tuning && k <= (1 << 20) &&
            p.max_nnz[slice_small_items(k, repeated)] >= slice_min_nnz(k, repeated) && !A->debug_checks;
+}
+
+// At the start of a call: tiles whose values a replay may have changed
+static void slices_untracked(vbcsr_t *A) {
+    for (SlicePlan &p : A->slice) p.stale |= p.untracked && p.vdig;
 }
 
 // k counts real columns here and below (two a column of a complex operator)
@@ -1255,16 +1266,18 @@ static bool fused_x_applies(const vbcsr_t *A, const ModePlan &p) {
 static int slice_prepare(vbcsr_t *A, bool trans, int64_t k, bool may_alloc, cudaStream_t s, bool *ready) {
     *ready = slice_buffers_ready(A, trans, k);
     SlicePlan &p = A->slice[trans];
-    const bool cap = capturing(s);
+    unsigned long long id = 0;
+    const bool cap = capturing(s, &id);
     if (*ready) {
         p.captured |= cap;
         A->xdig_captured |= cap;
         A->stab_captured |= cap;
-        if (p.stale) {
-            // under capture the rebuild belongs to the graph: the tiles stay stale for eager calls
+        if (p.stale && !(cap && p.capture == id)) {
+            // under capture the rebuild belongs to the graph, once: the tiles stay stale for eager calls
             int rc = refresh_slices(A, trans, s);
             if (rc) return rc;
-            if (!cap) p.stale = false;
+            if (cap) p.capture = id;
+            else p.stale = false;
         }
         return VBCSR_OK;
     }
@@ -1341,6 +1354,7 @@ static int run_product(vbcsr_t *A, bool trans, int64_t k, double alpha, const vo
         if (rc) return rc;
     }
     const int64_t kr = cplx ? 2 * k : k;   // real columns
+    if (!repeated) slices_untracked(A);    // a recurrence's call does at its start
     bool sliced = (f64 || cplx) && mode == VBCSR_PREC_NATIVE && alpha != 0.0 &&
                   slice_applies(A, trans, kr, repeated);
     if (sliced) {
@@ -1795,6 +1809,7 @@ static int run_chebyshev(vbcsr_t *A, int64_t k, const double *R, int64_t ldr, in
     epi.ldr = ldr;
     // t_1 = H~ R  -> buf[1];  t_0 (a copy of R) -> buf[0]
     epi.dot_out = moments + 1;
+    slices_untracked(A);
     // with the fused form, t_n is also kept converted in xs[n & 1]
     const FusedX fx0 = {nullptr, xs[1]};
     int rc = run_product(A, false, k, 1.0, R, ldr, 0.0, buf[1], k, &epi, precision, s, scale, xs[1] ? &fx0 : nullptr,
@@ -1856,6 +1871,7 @@ extern "C" int vbcsr_chebyshev_backward(vbcsr_t *A, int64_t k, const double *R, 
     const int64_t nseg = (M - 1 + E - 1) / E;
     bool first = true;
     int rc;
+    slices_untracked(A);
     vbcsr_epilogue_t epi;
     for (int64_t sg = nseg - 1; sg >= 0; --sg) {
         const int64_t n_lo = sg * E, n_hi = std::min((sg + 1) * E - 1, M - 2);
@@ -1928,6 +1944,7 @@ extern "C" int vbcsr_kpm_moments(vbcsr_t *A, int64_t k, const double *R, int64_t
         int rc = cheb_fused_buffers(A, k, precision, xs, s);
         if (rc) return rc;
     }
+    slices_untracked(A);
     int rc = self_dot(R, ldr, moments);                                     // mu_0
     if (rc || M == 1) return rc;
     vbcsr_epilogue_t epi;

@@ -372,3 +372,45 @@ def test_autotune_times_the_multiply_adds():
     names = _kernels(lambda: H.autotune(16))
     assert any("fma" in s for s in names) and not any("slice" in s for s in names)
     assert any("slice_product" in s for s in _kernels(lambda: H.spmm(X)))
+
+
+def test_captured_values_before_any_product():
+    """A captured change of the values on a handle without digit tiles does not keep its products
+    off the tensor cores: every call rebuilds the tiles, a recurrence and a graph once."""
+    import oracle
+    import synthetic as syn
+    w, H = _amorphous()
+    pat, k = w.pattern, 16
+    X = np.random.default_rng(1).standard_normal((pat.n_cols, k))
+    Xd = torch.from_numpy(X).cuda()
+    v = [syn.random_values(pat, s) / 40 for s in range(4)]
+    buf = torch.from_numpy(v[0]).cuda()
+    H.set_values(buf)
+    setv = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(setv):
+        H.set_values(buf)
+
+    def same(i, y):
+        ref, mag = oracle.spmm(pat, v[i], X), oracle.spmm(pat, np.abs(v[i]), np.abs(X))
+        assert (np.abs(y.cpu().numpy() - ref) <= 1600 * U * mag).all()   # two chains of at most 768 terms
+
+    assert any("slice_product" in s for s in _kernels(lambda: H.spmm(Xd)))
+    same(0, H.spmm(Xd))
+    buf.copy_(torch.from_numpy(v[1]))
+    setv.replay()
+    same(1, H.spmm(Xd))
+    Y = torch.empty(2, pat.n_rows, k, dtype=torch.float64, device="cuda:0")
+    prod = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(prod):
+        H.spmm(Xd, 1.0, 0.0, Y[0])
+        H.spmm(Xd, 1.0, 0.0, Y[1])
+    for i in (2, 3):
+        buf.copy_(torch.from_numpy(v[i]))
+        setv.replay()
+        prod.replay()
+        same(i, Y[0])
+        same(i, Y[1])
+    assert sum("slice_values" in s for s in _kernels(prod.replay)) == 1
+    R = torch.randn(pat.n_rows, k, dtype=torch.float64, device="cuda:0")
+    names = _kernels(lambda: H.chebyshev(R, 6))
+    assert sum("slice_product" in s for s in names) == 5 and sum("slice_values" in s for s in names) == 1
