@@ -90,7 +90,9 @@ typedef enum {
  *          an entry, one copy a direction) and of X are buffers that the handle
  *          owns, allocated on first use and grown like those of the mixed
  *          modes; while `stream` is being captured, or when the device has no
- *          room, nothing is allocated and such a call runs by FMA. Make one
+ *          room (less than a quarter of its memory would be left), nothing
+ *          is allocated and such a call runs by FMA; vbcsr_set_sliced keeps a
+ *          handle on FMA and gives its buffers back. Make one
  *          ordinary call before a capture so that the graph gets the
  *          tensor-core form; a graph stays valid when later calls need larger
  *          buffers.
@@ -534,6 +536,14 @@ int vbcsr_set_bucket_tuning(vbcsr_t *A, int32_t B, int32_t kc, int32_t warps_per
 int vbcsr_set_schedule(vbcsr_t *A, int32_t schedule, int32_t persist_warps);
 int vbcsr_get_tuning(const vbcsr_t *A, int32_t *kc_by_b, int32_t *warps_by_b, int32_t *schedule,
                      int32_t *persist_warps);
+
+/*
+ * vbcsr_set_sliced: enabled = 0 keeps the handle's native FP64 products on FMA and frees the
+ * digit buffers (up to 14 bytes a stored entry) that no captured graph uses, after
+ * synchronising `stream` (do not call it during a capture); 1 (the default) lets later calls
+ * use the tensor cores again and build them anew.
+ */
+int vbcsr_set_sliced(vbcsr_t *A, int enabled, void *stream);
 
 /*
  * Autotuner: times the product (transpose = 0 forward, 1 adjoint) at width k

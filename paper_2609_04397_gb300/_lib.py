@@ -59,6 +59,7 @@ SIGNATURES = {
     "vbcsr_set_tuning": ([_p, _i32, _i32], _int),
     "vbcsr_set_bucket_tuning": ([_p, _i32, _i32, _i32], _int),
     "vbcsr_set_schedule": ([_p, _i32, _i32], _int),
+    "vbcsr_set_sliced": ([_p, _int, _p], _int),
     "vbcsr_get_tuning": ([_p, _p, _p, _p, _p], _int),
     "vbcsr_autotune": ([_p, _int, _i64, _p, _i64, _p, _i64, _int, _i32, _p], _int),
     "vbcsr_check": ([_p, _p], _int),

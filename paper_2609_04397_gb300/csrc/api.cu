@@ -107,6 +107,7 @@ struct SlicePlan {
     int32_t *rexp = nullptr;        // scale exponent of every output row, then its parts (SliceArgs::rparts)
     Room room;                      // of vdig
     bool stale = false;             // the values changed since the tiles were built
+    bool held = false;              // a graph reads or writes the tiles: they stay until the handle goes
     bool captured = false;          // a captured product reads the tiles: every change of the values rebuilds them
     bool untracked = false;         // a capture changes the values with no tiles to rebuild: every call rebuilds them
     unsigned long long capture = 0; // the capture that holds a rebuild of stale tiles
@@ -171,6 +172,7 @@ struct vbcsr_matrix {
     uint64_t *sdpan = nullptr;   // fixed-point rows of A and B of the sliced pattern-sampled product
     size_t sdpan_elems = 0;
     bool tuning = false;         // vbcsr_autotune times the multiply-add kernels
+    bool no_slices = false;      // vbcsr_set_sliced: native products keep to the multiply-adds
     bool xdig_captured = false, stab_captured = false, sdpan_captured = false;   // a graph holds the buffer
     Room xdig_room, stab_room, sdpan_room;
     uint32_t *stab = nullptr;
@@ -923,15 +925,19 @@ static int grow(vbcsr_t *A, T **buf, size_t *have, size_t need, cudaStream_t s, 
     return VBCSR_OK;
 }
 
-// An optional allocation: *p stays NULL when the device has no room. A capture on another
-// thread is not disturbed by it.
+// An optional allocation: *p stays NULL when the device has no room, which is when less
+// than a quarter of its memory would be left: a caller whose operator and panels nearly fill
+// it needs the rest itself. A capture on another thread is not disturbed by it.
 template <typename T>
 static int alloc_optional(vbcsr_t *A, T **p, size_t count, Room *room, const char *what) {
     *p = nullptr;
     if (!room->may_try(count * sizeof(T))) return VBCSR_OK;
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     CUDA_TRY(cudaThreadExchangeStreamCaptureMode(&mode), "capture mode");
-    const cudaError_t e = A->alloc(p, count);
+    size_t left = 0, total = 0;
+    cudaError_t e = cudaMemGetInfo(&left, &total);
+    if (e == cudaSuccess)
+        e = left < count * sizeof(T) + total / 4 ? cudaErrorMemoryAllocation : A->alloc(p, count);
     if (e == cudaErrorMemoryAllocation) cudaGetLastError();
     cudaThreadExchangeStreamCaptureMode(&mode);
     if (e != cudaSuccess && e != cudaErrorMemoryAllocation) return cuda_fail(e, what);
@@ -1010,6 +1016,7 @@ static int slices_changed(vbcsr_t *A, cudaStream_t s) {
         if (!p.vdig) {
             p.untracked |= cap;
         } else if (cap || p.captured) {
+            p.held |= cap;
             int rc = refresh_slices(A, t == 1, s);
             if (rc) return rc;
             if (!cap) p.stale = false;
@@ -1023,7 +1030,7 @@ static int slices_changed(vbcsr_t *A, cudaStream_t s) {
 // True when a native FP64 product of k columns runs sliced.
 static bool slice_applies(const vbcsr_t *A, bool trans, int64_t k, bool repeated) {
     const SlicePlan &p = A->slice[trans];
-    return p.applies && !A->tuning && k <= (1 << 20) &&
+    return p.applies && !A->tuning && !A->no_slices && k <= (1 << 20) &&
            p.max_nnz[slice_small_items(k, repeated)] >= slice_min_nnz(k, repeated) && !A->debug_checks;
 }
 
@@ -1049,6 +1056,33 @@ static bool slice_buffers_ready(const vbcsr_t *A, bool trans, int64_t k) {
 // caller must not allocate; when the device has no room, the product runs
 // multiply-adds.
 static int slice_prepare(vbcsr_t *A, bool trans, int64_t k, bool may_alloc, cudaStream_t s, bool *ready);
+
+extern "C" int vbcsr_set_sliced(vbcsr_t *A, int enabled, void *stream) {
+    if (!A) return fail(VBCSR_ERR_INVALID_ARG, "handle is NULL");
+    if (enabled != 0 && enabled != 1) return fail(VBCSR_ERR_INVALID_ARG, "enabled must be 0 or 1");
+    if (!enabled && capturing((cudaStream_t)stream))
+        return fail(VBCSR_ERR_UNSUPPORTED, "the stream is being captured");
+    A->no_slices = enabled == 0;
+    if (enabled) return VBCSR_OK;
+    CUDA_TRY(cudaStreamSynchronize((cudaStream_t)stream), "synchronize");
+    for (SlicePlan &p : A->slice) {
+        if (p.held) continue;
+        release(A, p.vdig);
+        release(A, p.rexp);
+        p.vdig = nullptr;
+        p.rexp = nullptr;
+    }
+    auto give_back = [&](auto **buf, size_t *have, bool captured) {
+        if (captured) return;
+        release(A, *buf);
+        *buf = nullptr;
+        *have = 0;
+    };
+    give_back(&A->xdig, &A->xdig_elems, A->xdig_captured);
+    give_back(&A->stab, &A->stab_elems, A->stab_captured);
+    give_back(&A->sdpan, &A->sdpan_elems, A->sdpan_captured);
+    return VBCSR_OK;
+}
 
 extern "C" int vbcsr_set_values(vbcsr_t *A, const void *values, int on_device, void *stream) {
     if (!A) return fail(VBCSR_ERR_INVALID_ARG, "handle is NULL");
@@ -1270,6 +1304,7 @@ static int slice_prepare(vbcsr_t *A, bool trans, int64_t k, bool may_alloc, cuda
     const bool cap = capturing(s, &id);
     if (*ready) {
         p.captured |= cap;
+        p.held |= cap;
         A->xdig_captured |= cap;
         A->stab_captured |= cap;
         if (p.stale && !(cap && p.capture == id)) {
@@ -1691,7 +1726,7 @@ static SddmmArgs sddmm_args(vbcsr_t *A) {
 // widths whose level sums stay exact; else by multiply-adds, as on a stream that is
 // being captured before the buffers exist.
 static int run_sddmm_f64(vbcsr_t *A, const SddmmArgs &a, cudaStream_t s) {
-    bool sliced = a.k >= kSddmmMinCols && a.k <= kSliceKMax && a.alpha != 0.0 && A->nnz * a.k >= kSddmmMinWork &&
+    bool sliced = a.k >= kSddmmMinCols && a.k <= kSliceKMax && a.alpha != 0.0 && A->nnz * a.k >= kSddmmMinWork && !A->no_slices &&
                   A->nnz >= (a.k < 16 ? kSddmmItemNnz : kSliceItemNnz[1]) * A->n_fwd_items && !A->debug_checks;
     if (sliced) {
         const int64_t kp = (a.k + 15) / 16 * 16, rows = A->n_rows + A->n_cols;

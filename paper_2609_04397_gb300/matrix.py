@@ -205,6 +205,12 @@ class VBCSR:
                 | (0 if scalar_kernel else 4) | (0 if value_ring else 8) | (0 if pipelined_f32 else 16))
         check(lib().vbcsr_set_schedule(self._h, code, persist_warps), "vbcsr_set_schedule")
 
+    def set_sliced(self, enabled: bool = True):
+        """False keeps native FP64 products on multiply-adds and frees the digit buffers of
+        the tensor-core ones (7 bytes an entry and direction, and panels) that no captured
+        graph uses; True lets later calls build them anew."""
+        check(lib().vbcsr_set_sliced(self._h, int(enabled), _stream(self.device)), "vbcsr_set_sliced")
+
     def get_tuning(self) -> dict:
         kc = np.zeros(17, np.int32)
         w = np.zeros(17, np.int32)

@@ -414,3 +414,51 @@ def test_captured_values_before_any_product():
     R = torch.randn(pat.n_rows, k, dtype=torch.float64, device="cuda:0")
     names = _kernels(lambda: H.chebyshev(R, 6))
     assert sum("slice_product" in s for s in names) == 5 and sum("slice_values" in s for s in names) == 1
+
+
+def _device_bytes(H):
+    import ctypes
+    from paper_2609_04397_gb300 import _lib
+    info = _lib.Info()
+    assert _lib.lib().vbcsr_get_info(H.handle, ctypes.byref(info)) == 0
+    return info.device_bytes
+
+
+def test_digit_buffers_leave_memory_and_are_given_back():
+    """No digit buffers while they would leave less than a quarter of the device's memory;
+    set_sliced(False) frees those that no graph holds, and products run multiply-adds."""
+    w, H = _amorphous()
+    k = 16
+    X = torch.randn(w.pattern.n_cols, k, dtype=torch.float64, device="cuda:0")
+    Y = torch.empty(w.pattern.n_rows, k, dtype=torch.float64, device="cuda:0")
+    bare = _device_bytes(H)
+    torch.cuda.empty_cache()
+    free, total = torch.cuda.mem_get_info()
+    full = [torch.empty(1 << 32, dtype=torch.uint8, device="cuda:0") for _ in range((free - total // 5) >> 32)]
+    assert not any("slice" in s for s in _kernels(lambda: H.spmm(X, 1.0, 0.0, Y)))
+    assert _device_bytes(H) == bare
+    full.clear()
+    torch.cuda.empty_cache()
+    for _ in range(70):
+        H.spmm(X, 1.0, 0.0, Y)
+    assert any("slice_product" in s for s in _kernels(lambda: H.spmm(X, 1.0, 0.0, Y)))
+    first = Y.clone()
+    D = H.sddmm(X[:, :6].contiguous(), X[:, :6].contiguous())
+    assert _device_bytes(H) > bare + 7 * w.pattern.nnz
+    H.set_sliced(False)
+    assert _device_bytes(H) == bare
+    names = _kernels(lambda: (H.spmm(X, 1.0, 0.0, Y), H.sddmm(X[:, :6].contiguous(), X[:, :6].contiguous())))
+    assert names and not any("slice" in s for s in names)
+    assert ((Y - first).abs() <= 1600 * U * H_abs_product(w, X)).all()   # two chains of at most 768 terms
+    H.set_sliced(True)
+    assert torch.equal(H.spmm(X), first) and torch.equal(H.sddmm(X[:, :6].contiguous(), X[:, :6].contiguous()), D)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        H.spmm(X, 1.0, 0.0, Y)
+    H.set_sliced(False)
+    Y.zero_()
+    graph.replay()
+    assert torch.equal(Y, first)
+    H.set_values(torch.from_numpy(2.0 * w.values).cuda())
+    graph.replay()
+    assert torch.equal(Y, 2.0 * first)
