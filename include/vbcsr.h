@@ -77,7 +77,8 @@ typedef enum {
  *          of whose work nine tenths lie in rows of at most 768 entries (384
  *          complex) run these rows on the tensor cores, from 2^24 stored
  *          entries x columns per structure and 5 columns on, inside a
- *          recurrence from 2^22 and 3 (a complex column counts as two, a
+ *          recurrence from 2^22 and 3, of a batch when the structures above this
+ *          hold two fifths of its entries, an eighth in a recurrence (a complex column counts as two, a
  *          complex entry too; 5 to 7 columns count as 8) and work items of a
  *          few hundred entries: rows of H and columns of X as 56-bit fixed-point
  *          integers in exact base-256 digits, their products summed exactly

@@ -462,3 +462,36 @@ def test_digit_buffers_leave_memory_and_are_given_back():
     H.set_values(torch.from_numpy(2.0 * w.values).cuda())
     graph.replay()
     assert torch.equal(Y, 2.0 * first)
+
+
+@pytest.mark.parametrize("small,sliced", [(1, True), (8, False)])
+def test_batches_are_sliced_for_their_share_of_large_structures(small, sliced):
+    """One structure above the size line beside small ones: sliced when it holds two fifths of the
+    batch's entries, else multiply-adds throughout, as one launch without passes over X."""
+    import oracle
+    import synthetic as syn
+    from paper_2609_04397_gb300 import VBCSR
+    pats = [syn.random_pattern(n, n, (4, 9, 13), 0.15, n, empty_rows=0, unsorted=True)
+            for n in [330] + [220 + s for s in range(small)]]
+    pats = [BlockPattern(p.row_bsize, p.row_bsize, p.block_row_ptr, p.block_col_idx) for p in pats]
+    nnz = np.array([p.nnz for p in pats])
+    assert nnz[0] * 16 >= 1 << 24 > nnz[1] * 16 and (nnz[0] / nnz.sum() >= 0.5 if sliced else nnz[0] / nnz.sum() <= 0.35)
+    offs = np.cumsum([0] + [len(p.row_bsize) for p in pats])
+    ptr = np.concatenate([[0]] + [p.block_row_ptr[1:] + s for p, s in zip(pats, np.cumsum([0] + [p.nblk for p in pats]))])
+    col = np.concatenate([p.block_col_idx for p in pats])
+    rb = np.concatenate([p.row_bsize for p in pats])
+    vals = [syn.random_values(p, i) for i, p in enumerate(pats)]
+    H = VBCSR.from_batched(offs, offs, rb, rb, ptr, col, np.concatenate(vals), torch.float64, "cuda:0")
+    X = np.random.default_rng(0).standard_normal((int(rb.sum()), 16))
+    Xd = torch.from_numpy(X).cuda()
+    names = _kernels(lambda: H.spmm(Xd))
+    assert any("slice" in s for s in names) == sliced
+    got, r, c = H.spmm(Xd).cpu().numpy(), 0, 0
+    for p, v in zip(pats, vals):
+        x = np.ascontiguousarray(X[c:c + p.n_cols])
+        mag = oracle.spmm(p, np.abs(v), np.abs(x))
+        # two chains of a row's terms
+        assert (np.abs(got[r:r + p.n_rows] - oracle.spmm(p, v, x)) <= 2 * p.n_cols * U * mag).all()
+        r, c = r + p.n_rows, c + p.n_cols
+    # in a recurrence the lines are lower
+    assert any("slice_product" in s for s in _kernels(lambda: H.chebyshev(Xd, 4)))
