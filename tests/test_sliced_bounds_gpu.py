@@ -495,3 +495,37 @@ def test_batches_are_sliced_for_their_share_of_large_structures(small, sliced):
         r, c = r + p.n_rows, c + p.n_cols
     # in a recurrence the lines are lower
     assert any("slice_product" in s for s in _kernels(lambda: H.chebyshev(Xd, 4)))
+
+
+def test_what_is_not_sliced_runs_multiply_adds():
+    """The column floors, the size line and small work items, each seen in a trace that shows the
+    multiply-add kernel that ran instead."""
+    import synthetic as syn
+
+    def sliced(fn, plain):
+        names = _kernels(fn)
+        yes = any("slice" in s for s in names)
+        assert yes or any(plain in s for s in names), names
+        return yes
+
+    w, H = _amorphous()
+    lo, hi = H.gershgorin()
+    H.shift_scale((lo + hi) / 2, 0.51 * (hi - lo))
+    X = torch.randn(w.pattern.n_cols, 16, dtype=torch.float64, device="cuda:0")
+    for k in (1, 2, 3, 4, 5, 8, 16):
+        Xk = X[:, :k].contiguous()
+        kc = max(8, 1 << (k - 1).bit_length())
+        single = k >= 5 and w.pattern.nnz * kc >= 1 << 24
+        repeated = k >= 3 and w.pattern.nnz * k >= 1 << 22
+        assert sliced(lambda: H.spmm(Xk), "fma") == single
+        assert sliced(lambda: H.spmm_adjoint(Xk), "fma") == single
+        assert sliced(lambda: H.chebyshev(Xk, 4), "fma") == repeated
+        assert sliced(lambda: H.sddmm(Xk, Xk), "sddmm") == (k >= 6 and w.pattern.nnz * k >= 1 << 22)
+    n = 14_000   # 2 x 2 blocks, 40 a row: 160 entries a work item
+    cols = np.sort((np.arange(n)[:, None] + 3 * np.arange(40)) % n, axis=1)
+    pat = BlockPattern(np.full(n, 2), np.full(n, 2), np.arange(n + 1) * 40, cols.reshape(-1))
+    H = _handle(pat, syn.random_values(pat, 1))
+    X = torch.randn(pat.n_cols, 8, dtype=torch.float64, device="cuda:0")
+    assert not sliced(lambda: H.spmm(X), "fma")
+    assert not sliced(lambda: H.spmm_adjoint(X), "fma")
+    assert not sliced(lambda: H.sddmm(X, X), "sddmm")
