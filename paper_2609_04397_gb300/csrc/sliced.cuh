@@ -14,11 +14,13 @@
 //    -128 .. 127: one byte each, which f16 holds exactly;
 //  * products of digits i and j (digit 0 the most significant) are integers up
 //    to 2^14 and belong to level i + j, of weight 256^-(i + j). Sums over
-//    kSliceFlush columns stay below 2^24 in the levels that matter, so the FP32
-//    accumulators hold them exactly, in any order; longer rows carry each
-//    level's upper part into the next one up every kSliceFlush columns;
-//  * the levels 0 .. 7 (34 digit pairs) are added as integers and rounded to
-//    FP64 once. What is dropped is about 2^-58 of (row scale) x (column scale).
+//    kSliceFlush steps stay below 2^24 in the levels 0 to 4 whatever the digits,
+//    so the FP32 accumulators hold them exactly, in any order (kSliceFlush on the
+//    levels below); longer rows carry each level's upper part into the next one up
+//    every kSliceFlush steps;
+//  * the levels 0 .. 7 (34 of the 49 digit pairs) are added as integers and rounded
+//    to FP64 once. The pairs left out are below 2^-61 of (row scale) x (column scale)
+//    a term, the rounding of an element to 56 bits below 2^-56.
 //
 // An FP64 multiply-add chain instead rounds at every step; on panels of entries of
 // like size the sliced product is the nearer one to the exact result. The scales
@@ -55,8 +57,8 @@ constexpr float kSliceGuard = 4352.f;
 // The same with the sum of the leading digits' magnitudes of the row and of the column over
 // the K terms at hand: sum |h| + sum |x| <= (digits + 1.004 K) 2^48, the levels left out
 // are below 2^48.4 K, sum |h x| is at least 0.248 of the estimate times 2^96. Panels whose
-// column maxima lie far above most entries stay resolved by it (Student's t with 3 degrees
-// of freedom, 20k disordered atoms, k = 8: 886 us by kSliceGuard alone, 546 by multiply-adds).
+// column maxima lie far above most entries stay resolved by it (Student's t with 3 degrees of
+// freedom, 20k disordered atoms, k = 8: 325 us, 886 by kSliceGuard alone, 546 by multiply-adds).
 __device__ __forceinline__ float slice_guard(int digits, int K) {
     return fminf(kSliceGuard, 66.f * ((float)digits / (float)K + 3.7f));
 }
@@ -68,7 +70,12 @@ __device__ __forceinline__ float slice_guard(int digits, int K) {
 // tried and runs 1.6 to 2.3 times as fast as multiply-adds on 20k atoms.
 constexpr int kSliceTiny = 8;
 constexpr int kSliceLevels = 8;
-constexpr int kSliceFlush = 12;        // 16-column steps between carries: 5 products x 192 columns x 2^14 < 2^24
+// 16-column steps between carries: 5 products x 192 columns x 2^14 < 2^24 in level 4. The
+// levels 5, 6 and 7 have 6, 7 and 6 products: sums of nearly extreme digits throughout pass
+// 2^24 there and lose a unit or two of 2^-54, 2^-62, 2^-70 of the scales' product a step; in
+// level 5 (and 6) that takes leading digits near 128 of both (of one) operands, whose sum
+// |h x| (sum |h| + sum |x|, see kSliceGuard) is then far above the loss.
+constexpr int kSliceFlush = 12;
 constexpr int kSliceTile = kSliceDigits * 16;   // bytes of one row of a 16-column value tile
 // biased FP64 exponents a row or column maximum may have (the products of two
 // stay clear of overflow and of subnormal results)

@@ -10,6 +10,7 @@ namespace vbcsr {
 namespace {
 
 constexpr int kSliceList = (kSliceKMax + 16) * sizeof(int32_t);   // X rows of an item and of one step more
+constexpr uint32_t kSliceWary = 2;  // such passes after which the first attempt of a wide kernel is CAREFUL
 constexpr int kSliceState = 16;   // bytes that a warp keeps from item to item
 // unresolved outputs of a pass computed one by one: at most a quarter of the pass (they take
 // about twice the FP64 pipe's time of an item's common multiply-adds, and far more latency)
@@ -18,7 +19,7 @@ constexpr int kSliceStages = 4;   // value tiles in flight per warp (16 columns,
 
 // What a warp keeps from item to item, behind its list: [0] the structure of the last item,
 // [1] its passes that run multiply-adds: bit p for the 16 columns of pass p, bit 31 for pass
-// 31 and all after it; [2] whether the last pass had outputs below kSliceGuard
+// 31 and all after it; [2] passes with outputs below kSliceGuard since a CAREFUL one had none
 __device__ __forceinline__ volatile uint32_t *slice_state(unsigned char *ring) {
     return reinterpret_cast<volatile uint32_t *>(ring + kSliceStages * 16 * kSliceTile + kSliceList);
 }
@@ -112,6 +113,63 @@ __device__ __noinline__ void slice_digit_sums(const unsigned char *tiles, int B,
     __syncwarp();
 }
 
+// Whether slice_guard resolves every output of a pass of 16 columns (or the last ones) that has
+// some below kSliceGuard, from the leading digits alone: lane % 16 a column, the two halves
+// 8 rows each. Complex T: an output whose every term has a part that is zero throughout is an
+// exact zero. A small loop: the code of the CAREFUL pass, fetched for one item near the end
+// of a launch, took 119,000 clocks (20k zinc-blende atoms, k = 16: 350 us with it for every such
+// pass, 334 with this first, 316 with none).
+template <typename T>
+__device__ __noinline__ bool slice_recheck(const SliceArgs &q, const unsigned char *tiles, int B, int K, int64_t yrow,
+                                           int64_t k, int64_t n0, const uint32_t *cmax, const int32_t *s_x, int lane) {
+    const int64_t c = n0 + (lane & 15);
+    const int r0 = lane >> 4 << 3;
+    const uint32_t zero = 0x80808080u;
+    unsigned low[8], rows[8], cols = 0;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) low[r] = rows[r] = 0;
+    for (int t = 0; t < K; t += 16, tiles += B * kSliceTile) {
+        uint32_t x[4] = {zero, zero, zero, zero};   // leading digits of four X rows a word
+        if (c < q.ldp)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                x[i] = 0;
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    x[i] |= (uint32_t)(__ldg(q.xdig + (int64_t)s_x[t + 4 * i + j] * q.ldp + c) >> 48 & 0xff) << (8 * j);
+            }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) x[i] = __vabsdiffu4(x[i], zero), cols += __dp4a(x[i], 0x01010101u, 0u);
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            if (r0 + r >= B) break;
+            const uint4 v = __ldg(reinterpret_cast<const uint4 *>(tiles + 16 * (r0 + r)));
+            const uint32_t h[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint32_t d = __vabsdiffu4(h[i], zero);
+                rows[r] = __dp4a(d, 0x01010101u, rows[r]);
+                low[r] = __dp4a(d, x[i], low[r]);
+            }
+        }
+    }
+    bool ok = true;
+    const bool live = c < k && cmax[c] != 0;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+        if (r0 + r >= B) break;
+        const int e = q.rexp[yrow + r0 + r];
+        bool out = live && e != 0;
+        if (sizeof(T) > sizeof(double) && out) {
+            const uint32_t *own = q.cown + (cmax - q.cmax);
+            const int parts = q.rparts[yrow + r0 + r];
+            out = ((parts & 1) && own[c]) || ((parts & 2) && own[c ^ 1]);
+        }
+        ok &= e >= 0 && (!out || (float)low[r] >= slice_guard((int)(rows[r] + cols), K));
+    }
+    return __all_sync(0xffffffffu, ok);
+}
+
 // One pass of an item: up to 16 columns (WIDE) or up to 8, steps of 16 virtual
 // columns. A step's value tile (7 digits x B rows x 16 bytes, contiguous) comes
 // through a ring of shared-memory stages by asynchronous copies; the 16 gathered
@@ -131,10 +189,10 @@ __device__ __noinline__ void slice_digit_sums(const unsigned char *tiles, int B,
 // alone with its digits as the N side, one more MMA per digit of X (PAIR: per two)
 // instead of another group of 8 rows: 44 MMAs a wide step instead of 72, 25 a
 // narrow one instead of 36 (50k zinc-blende atoms, k = 32: 1.43 ms against 1.56).
-// Returns false, with nothing written, when an output is below kSliceGuard. Such a pass is
-// made a second time with CAREFUL (code that would cost the first one registers): outputs
-// below kSliceGuard are looked at with the sums that their error really depends on
-// (slice_guard), and those that the fixed point does not resolve are computed by
+// Returns false, with nothing written, when an output is below kSliceGuard and not `force`.
+// Such a pass is made a second time: with force (wide kernels) when the sums that its error
+// really depends on resolve it (slice_recheck), else with CAREFUL (code that would cost the
+// first one registers): outputs that slice_guard does not resolve are computed by
 // slice_one_output, a few of them (kSliceSingles; rows of few entries have one now and
 // then: corners of a cluster, 40 to 120 columns; without this the k = 32 product on 50k
 // zinc-blende atoms took 1.52 ms, all 16 columns of such items by multiply-adds). It
@@ -142,7 +200,7 @@ __device__ __noinline__ void slice_digit_sums(const unsigned char *tiles, int B,
 template <bool TRANS, bool WIDE, int NR, bool NINTH, bool CAREFUL, typename T>
 __device__ __forceinline__ bool slice_pass(const ProdArgs &a, const SliceArgs &q, const WorkItem &w,
                                            const unsigned char *vsrc, int K, int64_t n0, const uint32_t *cmax,
-                                           unsigned char *ring, const int32_t *s_x, int lane, double &dot) {
+                                           unsigned char *ring, const int32_t *s_x, int lane, bool force, double &dot) {
     constexpr int S = kSliceStages, kStage = 16 * kSliceTile;
     const int nsteps = (K + 15) >> 4;
     constexpr int NX = WIDE ? 2 : 1, NA = WIDE ? NR : 1;
@@ -308,11 +366,11 @@ __device__ __forceinline__ bool slice_pass(const ProdArgs &a, const SliceArgs &q
         for (int h = 0; h < NX; ++h)   // lanes t4 = 0 hold digit 0
             ok &= e9 == 0 || ec[2 * h] == 0 || t4 != 0 || nlow[2 * h] >= kSliceGuard;
     }
-    if (!CAREFUL && !__all_sync(0xffffffffu, ok)) return false;
+    if (!CAREFUL && !__all_sync(0xffffffffu, ok || force)) return false;
     uint32_t bad = 0;   // those for slice_one_output: bit 4 n + j, 8 + h for the ninth row's column g + 8 h
     if (CAREFUL) {
         const bool again = !__all_sync(0xffffffffu, ok);
-        if (lane == 0) slice_state(ring)[2] = again;
+        if (lane == 0) slice_state(ring)[2] = again ? max(slice_state(ring)[2], 1u) : 0u;
         int *sum = reinterpret_cast<int *>(ring);
         slice_digit_sums(vsrc, w.B, K, q.xdig, q.ldp, n0, s_x, sum, lane);
         bool scaled = e9 >= 0;
@@ -339,7 +397,7 @@ __device__ __forceinline__ bool slice_pass(const ProdArgs &a, const SliceArgs &q
                     !zero(8, g + 8 * h))
                     bad |= 256u << h;
         if (!__all_sync(0xffffffffu, scaled) ||
-            __reduce_add_sync(0xffffffffu, __popc(bad)) > min(kSliceSingles, w.B * (WIDE ? 4 : 2)))
+            __reduce_add_sync(0xffffffffu, __popc(bad)) > min(min(kSliceSingles, K >> 4), w.B * (WIDE ? 4 : 2)))
             return false;
         __syncwarp();   // before the next pass's tiles go where the sums were
     }
@@ -398,19 +456,20 @@ __device__ __forceinline__ bool slice_pass(const ProdArgs &a, const SliceArgs &q
 template <bool TRANS, bool WIDE, bool CAREFUL, typename T>
 __device__ __forceinline__ bool slice_pass_rows(const ProdArgs &a, const SliceArgs &q, const WorkItem &w,
                                                 const unsigned char *vsrc, int K, int64_t n0, const uint32_t *cmax,
-                                                unsigned char *ring, const int32_t *s_x, int lane, double &dot) {
-    return w.B <= 8 ? slice_pass<TRANS, WIDE, 1, false, CAREFUL, T>(a, q, w, vsrc, K, n0, cmax, ring, s_x, lane, dot)
-           : w.B == 9 ? slice_pass<TRANS, WIDE, 1, true, CAREFUL, T>(a, q, w, vsrc, K, n0, cmax, ring, s_x, lane, dot)
-                      : slice_pass<TRANS, WIDE, 2, false, CAREFUL, T>(a, q, w, vsrc, K, n0, cmax, ring, s_x, lane, dot);
+                                                unsigned char *ring, const int32_t *s_x, int lane, bool force,
+                                                double &dot) {
+    return w.B <= 8 ? slice_pass<TRANS, WIDE, 1, false, CAREFUL, T>(a, q, w, vsrc, K, n0, cmax, ring, s_x, lane, force, dot)
+           : w.B == 9 ? slice_pass<TRANS, WIDE, 1, true, CAREFUL, T>(a, q, w, vsrc, K, n0, cmax, ring, s_x, lane, force, dot)
+                      : slice_pass<TRANS, WIDE, 2, false, CAREFUL, T>(a, q, w, vsrc, K, n0, cmax, ring, s_x, lane, force, dot);
 }
 
-// The second attempt at a pass, or the only one where the warp's last pass needed two
-// (panels of a few large entries; the outputs are the same bits either way)
+// A pass with unresolved outputs, or the first attempt at one where the warp's last ones
+// had outputs below kSliceGuard (panels of a few large entries; the outputs are the same bits either way)
 template <bool TRANS, bool WIDE, typename T>
 __device__ __noinline__ bool slice_pass_again(const ProdArgs &a, const SliceArgs &q, const WorkItem &w,
                                               const unsigned char *vsrc, int K, int64_t n0, const uint32_t *cmax,
                                               unsigned char *ring, const int32_t *s_x, int lane, double &dot) {
-    return slice_pass_rows<TRANS, WIDE, true, T>(a, q, w, vsrc, K, n0, cmax, ring, s_x, lane, dot);
+    return slice_pass_rows<TRANS, WIDE, true, T>(a, q, w, vsrc, K, n0, cmax, ring, s_x, lane, false, dot);
 }
 
 // One warp per work item (up to 16 output rows). WIDE: k > 8, passes of 16
@@ -419,8 +478,8 @@ __device__ __noinline__ bool slice_pass_again(const ProdArgs &a, const SliceArgs
 // Complex operators (T = double2, TA its arithmetic): the kernel sees two real
 // columns a complex one and two virtual columns a complex value, re meeting the
 // X row x and im the row i x (slice_panel_kernel).
-// (The arguments are grid constants: the calls take their addresses, and a copy on the
-// stack cost the loop registers, 1.45 against 1.48 ms at k = 32 on 50k zinc-blende atoms.)
+// (The arguments are grid constants: the calls take their addresses, and with a copy on the
+// stack the k = 32 product on 50k zinc-blende atoms took 1.48 ms against 1.45.)
 template <bool TRANS, bool WIDE, typename T, typename TA>
 __global__ void __launch_bounds__(128, WIDE ? 3 : 4) slice_product_kernel(const __grid_constant__ ProdArgs a,
                                                                             const __grid_constant__ SliceArgs q) {
@@ -489,7 +548,7 @@ __global__ void __launch_bounds__(128, WIDE ? 3 : 4) slice_product_kernel(const 
         }
         if constexpr (!WIDE) {   // one pass
             const bool tried = skip == 0;
-            if (!tried || state[2] || !slice_pass_rows<TRANS, false, false, T>(a, q, w, vsrc, K, 0, cmax, ring, s_x, lane, dot)) {
+            if (!tried || state[2] || !slice_pass_rows<TRANS, false, false, T>(a, q, w, vsrc, K, 0, cmax, ring, s_x, lane, false, dot)) {
                 const WorkItem wc = w;   // copies: the calls take addresses, which would keep w and dot in memory
                 double dc = dot;
                 if (!tried || !slice_pass_again<TRANS, false, T>(a, q, wc, vsrc, K, 0, cmax, ring, s_x, lane, dc))
@@ -503,14 +562,24 @@ __global__ void __launch_bounds__(128, WIDE ? 3 : 4) slice_product_kernel(const 
                 // sliced up to the next pass that is not tried
                 const uint32_t left = skip >> min((int)(n0 >> 4), 31);
                 const int64_t stop = left ? min(a.k, n0 + 16 * (int64_t)(__ffs(left) - 1)) : a.k;
-                bool ok = n0 >= stop || !state[2];
+                bool ok = n0 >= stop || state[2] < kSliceWary, force = false;
+            attempt:
                 for (; ok && n0 + 8 < stop; n0 += ok ? 16 : 0)
-                    ok = slice_pass_rows<TRANS, true, false, T>(a, q, w, vsrc, K, n0, cmax, ring, s_x, lane, dot);
+                    ok = slice_pass_rows<TRANS, true, false, T>(a, q, w, vsrc, K, n0, cmax, ring, s_x, lane, force, dot), force = false;
                 if (ok && n0 < stop) {
-                    ok = slice_pass_rows<TRANS, false, false, T>(a, q, w, vsrc, K, n0, cmax, ring, s_x, lane, dot);
+                    ok = slice_pass_rows<TRANS, false, false, T>(a, q, w, vsrc, K, n0, cmax, ring, s_x, lane, force, dot);
                     n0 += ok ? 8 : 0;
                 }
                 if (n0 >= a.k) break;
+                if (!ok && state[2] < kSliceWary) {
+                    __syncwarp();
+                    if (lane == 0) state[2] = state[2] + 1;
+                    __syncwarp();
+                }
+                if (!ok && state[2] < kSliceWary && slice_recheck<T>(q, vsrc, w.B, K, w.yrow, a.k, n0, cmax, s_x, lane)) {
+                    ok = force = true;
+                    goto attempt;
+                }
                 const WorkItem wc = w;   // copies: the calls take addresses, which would keep w and dot in memory
                 double dc = dot;
                 const bool wide = n0 + 8 < a.k;

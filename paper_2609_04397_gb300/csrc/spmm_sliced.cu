@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(256) slice_panel_kernel(const SliceChunk *chun
 // [tile][digit][row][16 columns], two tiles at a time staged in shared memory
 // and stored 16 bytes a lane. Forward items are read with the lanes along a row
 // of the page; adjoint ones (TRANS), whose rows are the columns of the pages'
-// blocks, with BP = 1, 2, 4, 8 or 16 lanes along the item's rows (consecutive in
+// blocks, with BP = 2, 4, 8 or 16 lanes along the item's rows (consecutive in
 // the pages) and 32 / BP virtual columns a load: with a virtual column per lane
 // every load touched 32 sectors (0.47 ms for 3.8e7 entries, the forward
 // form 0.18).
