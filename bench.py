@@ -8,7 +8,7 @@ synthetic, shifted and scaled on the GPU to H~ = (H - c) / d with its spectrum
 inside [-1, 1] (Gershgorin bounds). One step is one step of the Chebyshev
 recurrence of the kernel polynomial method (Sec. V) on 16 Rademacher vectors:
 t_{n+1} = 2 H~ t_n - t_{n-1} with the moment <R, t_{n+1}> fused into the
-product's epilogue, FP64 block products (exact digit products on the FP16
+product's epilogue, FP64 block products (digit products on the FP16
 tensor cores, one FP64 rounding an output). The values (27.5 GB, 24 GB as
 digits) are far larger than the 129 MB L2, so no flush is needed.
 
@@ -85,12 +85,12 @@ MMA_F16_MAC_PER_CLK = 955
 
 # DRAM bytes (read + write) per stored entry of one FP64 Chebyshev step
 # (k = 16): ncu's dram__bytes_read.sum + dram__bytes_write.sum of the sliced
-# product with the recurrence epilogue (3.381 GB) and of the two passes over
-# t_n before it (0.141 and 0.234 GB) on the ~100k-atom nanoparticle
+# product with the recurrence epilogue (3.397 GB) and of the two passes over
+# t_n before it (0.141 and 0.233 GB) on the ~100k-atom nanoparticle
 # (336,743,405 entries), scaled by the stored entries to the headline operator
 # (values, X, Y and R all grow with the atom count). The summary is under
 # profiles/.
-TRAFFIC_F64_PER_ENTRY = 11.154
+TRAFFIC_F64_PER_ENTRY = 11.200
 
 
 def _workload(n_atoms=N_ATOMS):

@@ -81,8 +81,8 @@ typedef enum {
  *          hold two fifths of its entries, an eighth in a recurrence (a complex column counts as two, a
  *          complex entry too; 5 to 7 columns count as 8) and work items of a
  *          few hundred entries: rows of H and columns of X as 56-bit fixed-point
- *          integers in exact base-256 digits, their products summed exactly
- *          and rounded once. An output that the fixed point does not resolve
+ *          integers in base-256 digits, the leading 34 of the 49 digit products
+ *          summed as integers and rounded once. An output that the fixed point does not resolve
  *          (its terms far below its row's or column's largest), rows and
  *          columns with Inf, NaN or extreme exponents, and everything smaller
  *          is computed by FP64 FMA; either way the error of an output of K
