@@ -81,7 +81,7 @@ struct DevBuf {
     size_t bytes = 0;
 };
 
-// Allocations of one buffer of the sliced products, without which they run multiply-adds:
+// Allocations of the sliced products, without which they run multiply-adds:
 // the least size that failed is not asked for again for a while (a shortage can pass: a
 // caching allocator that gives memory back), smaller ones are.
 struct Room {
@@ -108,7 +108,7 @@ struct SlicePlan {
     int64_t nnz_all = 0;
     uint8_t *vdig = nullptr;        // value tiles, built on first use
     int32_t *rexp = nullptr;        // scale exponent of every output row, then its parts (SliceArgs::rparts)
-    Room room;                      // of vdig
+    Room room;                      // of the tiles and what comes with them
     bool stale = false;             // the values changed since the tiles were built
     bool held = false;              // a graph reads or writes the tiles: they stay until the handle goes
     bool captured = false;          // a captured product reads the tiles: every change of the values rebuilds them
@@ -177,7 +177,7 @@ struct vbcsr_matrix {
     bool tuning = false;         // vbcsr_autotune times the multiply-add kernels
     bool no_slices = false;      // vbcsr_set_sliced: native products keep to the multiply-adds
     bool xdig_captured = false, stab_captured = false, sdpan_captured = false;   // a graph holds the buffer
-    Room xdig_room, stab_room, sdpan_room;
+    Room xdig_room, sdpan_room;
     uint32_t *stab = nullptr;
     size_t stab_elems = 0;
     WorkItem *fwd_items = nullptr, *adj_items = nullptr;   // bucketed by row count
@@ -935,24 +935,24 @@ static int grow(vbcsr_t *A, T **buf, size_t *have, size_t need, cudaStream_t s, 
     return VBCSR_OK;
 }
 
-// An optional allocation: *p stays NULL when the device has no room, which is when less
-// than a quarter of its memory would be left: a caller whose operator and panels nearly fill
-// it needs the rest itself. A capture on another thread is not disturbed by it.
+// Whether a quarter of the device's memory is left beside `bytes` more: a caller whose operator
+// and panels nearly fill it needs the rest itself. Asked once for what a call is missing (the
+// query takes some 20 us).
+static bool room_left(size_t bytes) {
+    size_t left = 0, total = 0;
+    return cudaMemGetInfo(&left, &total) == cudaSuccess && left >= bytes + total / 4;
+}
+
+// An optional allocation: *p stays NULL when the device has no room. A capture on another
+// thread is not disturbed by it.
 template <typename T>
-static int alloc_optional(vbcsr_t *A, T **p, size_t count, Room *room, const char *what) {
-    *p = nullptr;
-    if (!room->may_try(count * sizeof(T))) return VBCSR_OK;
+static int alloc_optional(vbcsr_t *A, T **p, size_t count, const char *what) {
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     CUDA_TRY(cudaThreadExchangeStreamCaptureMode(&mode), "capture mode");
-    size_t left = 0, total = 0;
-    cudaError_t e = cudaMemGetInfo(&left, &total);
-    if (e == cudaSuccess)
-        e = left < count * sizeof(T) + total / 4 ? cudaErrorMemoryAllocation : A->alloc(p, count);
+    const cudaError_t e = A->alloc(p, count);
     if (e == cudaErrorMemoryAllocation) cudaGetLastError();
     cudaThreadExchangeStreamCaptureMode(&mode);
-    if (e != cudaSuccess && e != cudaErrorMemoryAllocation) return cuda_fail(e, what);
-    room->result(count * sizeof(T), e == cudaSuccess);
-    return VBCSR_OK;
+    return e == cudaSuccess || e == cudaErrorMemoryAllocation ? VBCSR_OK : cuda_fail(e, what);
 }
 
 static void release(vbcsr_t *A, void *p) {
@@ -970,13 +970,13 @@ static void release(vbcsr_t *A, void *p) {
 // fits (what is kept stays below what is in use). A wider call that does not fit leaves the
 // narrower ones their buffer.
 template <typename T>
-static int grow_native(vbcsr_t *A, T **buf, size_t *have, size_t need, bool *captured, Room *room, cudaStream_t s,
+static int grow_native(vbcsr_t *A, T **buf, size_t *have, size_t need, bool *captured, cudaStream_t s,
                        const char *what) {
     if (need <= *have) return VBCSR_OK;
     T *more = nullptr;
     size_t n = *captured ? std::max(need, 2 * *have) : need;
-    int rc = alloc_optional(A, &more, n, room, what);
-    if (!rc && !more && n > need) rc = alloc_optional(A, &more, n = need, room, what);
+    int rc = alloc_optional(A, &more, n, what);
+    if (!rc && !more && n > need) rc = alloc_optional(A, &more, n = need, what);
     if (rc || !more) return rc;
     if (!*captured && *buf) {
         cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
@@ -1336,24 +1336,34 @@ static int slice_prepare(vbcsr_t *A, bool trans, int64_t k, bool may_alloc, cuda
     }
     if (!may_alloc || cap) return VBCSR_OK;
     int rc = VBCSR_OK;
-    if (!p.rexp) rc = alloc_optional(A, &p.rexp, 2 * (size_t)(trans ? A->n_cols : A->n_rows), &p.room, "alloc scales");
+    const size_t n_out = 2 * (size_t)(trans ? A->n_cols : A->n_rows), x = slice_x_elems(A, trans, k),
+                 tab = slice_tab_elems(A, slice_ldp(k));
+    const size_t missing = (p.rexp ? 0 : n_out * sizeof(int32_t)) + (p.vdig ? 0 : (size_t)p.digit_bytes) +
+                           (x > A->xdig_elems ? x * sizeof(uint64_t) : 0) +
+                           (tab > A->stab_elems ? tab * sizeof(uint32_t) : 0);
+    Room &room = p.vdig ? A->xdig_room : p.room;
+    if (!room.may_try(missing)) return VBCSR_OK;
+    if (!room_left(missing)) {
+        room.result(missing, false);
+        return VBCSR_OK;
+    }
+    if (!p.rexp) rc = alloc_optional(A, &p.rexp, n_out, "alloc scales");
     if (!rc && p.rexp && !p.vdig) {
-        rc = alloc_optional(A, &p.vdig, (size_t)p.digit_bytes, &p.room, "alloc value digits");
+        rc = alloc_optional(A, &p.vdig, (size_t)p.digit_bytes, "alloc value digits");
         p.stale = p.vdig != nullptr;
     }
-    if (!rc && p.vdig)
-        rc = grow_native(A, &A->xdig, &A->xdig_elems, slice_x_elems(A, trans, k), &A->xdig_captured, &A->xdig_room, s,
-                         "alloc fixed-point X");
-    if (!rc && p.vdig)
-        rc = grow_native(A, &A->stab, &A->stab_elems, slice_tab_elems(A, slice_ldp(k)), &A->stab_captured,
-                         &A->stab_room, s, "alloc column maxima");
-    if (rc) return rc;
-    *ready = slice_buffers_ready(A, trans, k);
-    if (*ready && p.stale) {
+    if (!rc && p.vdig && p.stale) {   // runs while the host allocates the rest
         rc = refresh_slices(A, trans, s);
         p.stale = rc != VBCSR_OK;
     }
-    return rc;
+    if (!rc && p.vdig)
+        rc = grow_native(A, &A->xdig, &A->xdig_elems, x, &A->xdig_captured, s, "alloc fixed-point X");
+    if (!rc && p.vdig)
+        rc = grow_native(A, &A->stab, &A->stab_elems, tab, &A->stab_captured, s, "alloc column maxima");
+    if (rc) return rc;
+    *ready = slice_buffers_ready(A, trans, k);
+    room.result(missing, *ready);
+    return VBCSR_OK;
 }
 
 static int run_product(vbcsr_t *A, bool trans, int64_t k, double alpha, const void *X, int64_t ldx, double beta,
@@ -1749,10 +1759,13 @@ static int run_sddmm_f64(vbcsr_t *A, const SddmmArgs &a, cudaStream_t s) {
     if (sliced) {
         const int64_t kp = (a.k + 15) / 16 * 16, rows = A->n_rows + A->n_cols;
         const size_t need = (size_t)(rows * kp + (rows + 1) / 2);
-        if (need > A->sdpan_elems && !capturing(s)) {
-            const int rc = grow_native(A, &A->sdpan, &A->sdpan_elems, need, &A->sdpan_captured, &A->sdpan_room, s,
-                                       "alloc fixed-point panels");
+        const size_t bytes = need * sizeof(uint64_t);
+        if (need > A->sdpan_elems && !capturing(s) && A->sdpan_room.may_try(bytes)) {
+            const int rc = room_left(bytes) ? grow_native(A, &A->sdpan, &A->sdpan_elems, need, &A->sdpan_captured, s,
+                                                          "alloc fixed-point panels")
+                                            : VBCSR_OK;
             if (rc) return rc;
+            A->sdpan_room.result(bytes, need <= A->sdpan_elems);
         }
         sliced = need <= A->sdpan_elems;
         if (sliced) {
